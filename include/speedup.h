@@ -107,7 +107,12 @@ typedef struct {
                              harmonic oscillator and of the quartic potentials
                              at p <= 18, see su_fixed_shape) runs the sampler
                              specialised for that shape; 1: always the generic
-                             sampler.  Both give the same results bit for bit. */
+                             sampler.  Both give the same results bit for bit.
+                             In double precision 0 also takes the fixed-point
+                             sampler where the ranges of a, b, T and the tables
+                             allow it (even polynomial potentials, automatic
+                             segments); 1 never does.  The two agree to a
+                             double's rounding. */
 } su_options;
 
 /* per bisection level n = 0..s (N = 2^n slices) */

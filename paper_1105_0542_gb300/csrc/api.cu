@@ -396,8 +396,9 @@ static int plan_rounds(su_plan &pl, int rounds, int sms, int smem_max) {
 }
 
 // The sampler's parameters and launch shape of a plan (everything but the
-// device pointers): host work and occupancy queries only, no allocation.
-static int plan_shape(su_plan &pl, int sms, int smem_max) {
+// device pointers): host work and occupancy queries only, no allocation.  The
+// fixed-point sampler's images go behind the level tables in blob.
+static int plan_shape(su_plan &pl, int sms, int smem_max, std::vector<unsigned char> &blob) {
     using namespace su;
     SamplerParams &P = pl.P;
     const int S = pl.s;
@@ -441,6 +442,19 @@ static int plan_shape(su_plan &pl, int sms, int smem_max) {
     if (sampler_smem_bytes(P, prec) > (size_t)smem_max) {
         if (prec != SU_FP64) return fail(SU_ENOTSUP, "the level tables do not fit shared memory in single precision");
         P.tab_global = 1;
+    }
+    if (prec == SU_FP64 && !general) {
+        std::vector<int64_t> head;
+        std::vector<float> tail;
+        su::fx_plan(P, pl.T, reinterpret_cast<const double *>(blob.data()), head, tail);
+        if (P.fx.on && sampler_smem_bytes(P, prec) > (size_t)smem_max) P.fx.on = 0;
+        if (P.fx.on) {
+            P.fx.head_off = (int64_t)blob.size();
+            P.fx.tail_off = P.fx.head_off + (int64_t)(head.size() * sizeof(int64_t));
+            blob.resize((size_t)P.fx.tail_off + tail.size() * sizeof(float));
+            std::memcpy(blob.data() + P.fx.head_off, head.data(), head.size() * sizeof(int64_t));
+            std::memcpy(blob.data() + P.fx.tail_off, tail.data(), tail.size() * sizeof(float));
+        }
     }
     // launch shape: one path per thread, persistent grid over items of
     // 128 * rounds samples
@@ -488,7 +502,7 @@ static int configure(su_plan &pl) {
     int sms = 0, smem_max = 0;
     rc = device_limits(pl.device, sms, smem_max);
     if (rc) return rc;
-    rc = plan_shape(pl, sms, smem_max);
+    rc = plan_shape(pl, sms, smem_max, blob);
     if (rc) return rc;
     CU(dmalloc(&pl.d_tables, blob.size()), "device allocation (tables)");
     CU(cudaMemcpy(pl.d_tables, blob.data(), blob.size(), cudaMemcpyHostToDevice), "upload tables");
@@ -2638,7 +2652,7 @@ extern "C" int speedup_amplitude_noalloc(int model, const double *params, int n_
     int dev = 0, sms = 0, smem_max = 0;
     rc = device_limits(dev, sms, smem_max);
     if (rc) return rc;
-    rc = plan_shape(pl, sms, smem_max);
+    rc = plan_shape(pl, sms, smem_max, blob);
     if (rc) return rc;
 
     // scratch layout: tables | per-item tuples | per-block tuples | flag word;

@@ -136,8 +136,8 @@ __global__ void __launch_bounds__(kThreads, 4) nd_kernel(const __grid_constant__
     R *sw = reinterpret_cast<R *>(smem_raw);
     size_t off = per_sample ? 0 : sizeof(R) * (size_t)L * kThreads;
     off = (off + 15) & ~(size_t)15;
-    bm::Tables *bm_smem = reinterpret_cast<bm::Tables *>(smem_raw + off);
-    if constexpr (sizeof(R) == 8) bm::tables_init(bm_smem, tid, kThreads);
+    fx::Tables *bm_smem = reinterpret_cast<fx::Tables *>(smem_raw + off);
+    if constexpr (sizeof(R) == 8) fx::tables_load(bm_smem, tid, kThreads);
     __syncthreads();
 
     Stream<R> st;
@@ -279,7 +279,7 @@ size_t nd_smem_bytes(const NdParams &Q, int precision) {
     const size_t rs = precision == SU_FP32 ? sizeof(float) : sizeof(double);
     size_t off = Q.base.w_out ? 0 : rs * (size_t)Q.base.levels * kThreads;
     off = (off + 15) & ~(size_t)15;
-    return off + (precision == SU_FP32 ? 0 : sizeof(bm::Tables));
+    return off + (precision == SU_FP32 ? 0 : sizeof(fx::Tables));
 }
 
 int nd_occupancy(const NdParams &Q, int precision, size_t smem) {

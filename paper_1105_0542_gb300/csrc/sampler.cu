@@ -28,10 +28,14 @@ const void *batch_entry_f64_3();
 const void *batch_entry_f32_0();
 const void *batch_entry_f32_1();
 const void *batch_entry_f32_2();
+// the double sampler in fixed point (sampler_fx.cu)
+const void *sampler_fx_entry();
+size_t sampler_fx_smem_bytes(const SamplerParams &P);
 // the compiled-shape kernels of group g = k % kFixedGroups (sampler_inst.cu, SU_FIXED = g)
 #define SU_FIXED_GROUP(g)                        \
     const void *sampler_fixed_entry_##g(int k); \
-    const void *batch_fixed_entry_##g(int k);
+    const void *batch_fixed_entry_##g(int k);   \
+    const void *sampler_fx_fixed_entry_##g(int k);
 SU_FIXED_GROUP(0)
 SU_FIXED_GROUP(1)
 SU_FIXED_GROUP(2)
@@ -49,6 +53,9 @@ static const FixedEntry kSamplerFixed[kFixedGroups] = {
 static const FixedEntry kBatchFixed[kFixedGroups] = {
     batch_fixed_entry_0, batch_fixed_entry_1, batch_fixed_entry_2, batch_fixed_entry_3,
     batch_fixed_entry_4, batch_fixed_entry_5, batch_fixed_entry_6, batch_fixed_entry_7};
+static const FixedEntry kFxFixed[kFixedGroups] = {
+    sampler_fx_fixed_entry_0, sampler_fx_fixed_entry_1, sampler_fx_fixed_entry_2, sampler_fx_fixed_entry_3,
+    sampler_fx_fixed_entry_4, sampler_fx_fixed_entry_5, sampler_fx_fixed_entry_6, sampler_fx_fixed_entry_7};
 
 namespace {
 
@@ -102,8 +109,8 @@ __global__ void philox_words_kernel(uint64_t seed, uint32_t inst, int64_t sample
 // (j = 2t, 2t + 1) and four on the single path (j + 1 = 4t .. 4t + 3)
 __global__ void __launch_bounds__(128) normals_kernel_f64(uint64_t seed, uint32_t inst, int64_t sample0,
                                                           int64_t ns, int n, double *out) {
-    __shared__ bm::Tables tabs;
-    bm::tables_init(&tabs, threadIdx.x, blockDim.x);
+    __shared__ fx::Tables tabs;
+    fx::tables_load(&tabs, threadIdx.x, blockDim.x);
     __syncthreads();
     const int calls = (n + 1) / 2;
     const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -161,6 +168,10 @@ const void *pick_fixed(const SamplerParams &P, int precision) {
 }
 
 const void *pick(const SamplerParams &P, int precision) {
+    if (P.fx.on) {
+        const int k = fixed_shape_index(P.ncol, P.len);
+        return k < 0 ? sampler_fx_entry() : kFxFixed[k % kFixedGroups](k);
+    }
     if (const void *fn = pick_fixed(P, precision)) return fn;
     if (P.ring == RING_GENERAL) return precision == SU_FP64 ? sampler_entry_f64_3() : nullptr;
     if (P.tab_global) {
@@ -201,11 +212,12 @@ size_t batch_smem_bytes(const BatchParams &B, int precision) {
     off += (2 * sizeof(double) + rs) * (size_t)(B.L_max - 1) * kThreads;
     off = (off + 15) & ~(size_t)15;
     if (precision == SU_FP32) off += sizeof(float4) * (size_t)staged_quads(kMaxFine, true) * kThreads;
-    if (precision == SU_FP64) off += sizeof(bm::Tables);
+    if (precision == SU_FP64) off += sizeof(fx::Tables);
     return off;
 }
 
 size_t sampler_smem_bytes(const SamplerParams &P, int precision) {
+    if (P.fx.on) return sampler_fx_smem_bytes(P);
     const size_t rs = precision == SU_FP32 ? sizeof(float) : sizeof(double);
     const int C = 1 << (P.S - P.F);
     size_t off = P.w_out ? 0 : rs * (size_t)P.levels * kThreads * P.rounds;
@@ -219,7 +231,7 @@ size_t sampler_smem_bytes(const SamplerParams &P, int precision) {
     if (P.wf_on) off += sizeof(double) * (size_t)(P.S + 1) * kThreads;
     off = (off + 15) & ~(size_t)15;
     if (precision == SU_FP32) off += sizeof(float4) * (size_t)staged_quads(P.F) * kThreads;
-    if (precision == SU_FP64) off += sizeof(bm::Tables);
+    if (precision == SU_FP64) off += sizeof(fx::Tables);
     return off;
 }
 

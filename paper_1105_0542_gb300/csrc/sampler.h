@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -38,6 +39,28 @@ struct GeneralDev {
     double inv[kGenMaxSym + 1];                // 1 / n
 };
 
+// The fixed-point sampler's plan (sampler_fx.cuh; built by fx_plan).  Path
+// points are integers in units of q_unit; row d of the arrays is level n = S - d.
+constexpr int kFxCols = 4;
+struct FxLevel {
+    int ok;                   // evaluated in fixed point, else in double
+    int nc, h[kFxCols];       // columns with integer entries, and how many each (the others in single precision)
+    int ky;                   // vs is shifted left by ky before it is squared
+    int vlim;                 // |high word of vs| stays below this
+    int e;                    // weights in units of 2^-e
+    double res;               // what rounding to a unit takes from the constant entry, per slice
+};
+struct FxParams {
+    int on;
+    int qlim;                 // |high word of q| stays below this
+    int hrow;                 // room for integer entries per level
+    int sgh[SU_MAX_S + 1], sgl[SU_MAX_S + 1], shl[SU_MAX_S + 1];   // sigma_n: limbs and left shift of the product
+    int64_t qa, qb;           // endpoints
+    double q_unit;
+    FxLevel lv[SU_MAX_S];
+    int64_t head_off, tail_off;   // from the tables: [S][hrow] int64, [S][M] float
+};
+
 struct SamplerParams {
     // path: q_0 = a, q_N = b, N = 2^S, bisection widths sigma[n] (n = 1..S)
     double a, b;
@@ -71,7 +94,13 @@ struct SamplerParams {
     float *q_out;             // device: per-sample mode, single precision only: path points [sample][N+1] (or null)
     int *flags;               // device: bit 0 = non-finite weight seen
     const GeneralDev *general;  // device: RING_GENERAL only
+    FxParams fx;                // double precision: the fixed-point sampler where fx.on
 };
+
+// The fixed-point plan of a double-precision plan's tables (rows of M entries,
+// kernel_table's, for levels n = S..1): fills P.fx (on = 0 where the ranges do
+// not allow it) and the images head [S][hrow] and tail [S][M].  Host work.
+void fx_plan(SamplerParams &P, double T, const double *tables, std::vector<int64_t> &head, std::vector<float> &tail);
 
 // One instance of a batch: its path (a, b, N = 2^S, widths), its table
 // shape (one per distinct level p), its tables (L rows of M entries from

@@ -36,6 +36,7 @@
 #include <type_traits>
 
 #include "boxmuller.cuh"
+#include "fixed_point.cuh"
 #include "fixed_shapes.h"
 #include "philox.cuh"
 #include "generator.h"
@@ -52,11 +53,17 @@ struct Normal;
 template <>
 struct Normal<double> {
     // 53-bit uniforms ((w0 2^21 + w1 >> 11) + 1/2) 2^-53 from (w0,w1) and (w2,w3),
-    // through the table-driven routines of boxmuller.cuh
-    static __device__ __forceinline__ void pair(uint4 w, const bm::Tables *t, double &z0, double &z1) {
+    // through the fixed-point Box-Muller of fixed_point.cuh (units 2^-kZScale)
+    static __device__ __forceinline__ void fixed(uint4 w, const fx::Tables *t, int64_t &z0, int64_t &z1) {
         const uint64_t a = ((uint64_t)w.x << 21) | (w.y >> 11);
         const uint64_t b = ((uint64_t)w.z << 21) | (w.w >> 11);
-        bm::rotate(bm::sqrt_pos(bm::minus2log(a, t)), b, t, z0, z1);
+        fx::normals(a, b, t, z0, z1);
+    }
+    static __device__ __forceinline__ void pair(uint4 w, const fx::Tables *t, double &z0, double &z1) {
+        int64_t f0, f1;
+        fixed(w, t, f0, f1);
+        z0 = fx::to_double(f0, -fx::kZScale);
+        z1 = fx::to_double(f1, -fx::kZScale);
     }
 };
 
@@ -79,11 +86,14 @@ template <typename R>
 struct Stream {
     uint2 key;
     uint32_t inst, slo, shi;
-    const bm::Tables *bm;   // shared-memory node tables (double path)
+    const fx::Tables *bm;   // shared-memory node tables (double path)
     float4 *zq;             // single path: this thread's column (stride kThreads) of
                             // staged quads, levels 3..F of a segment (see sample_path)
     __device__ __forceinline__ uint4 words(uint32_t call) const {
         return philox4x32_10(make_uint4(call, inst, slo, shi), key);
+    }
+    __device__ __forceinline__ void fixed(uint32_t call, int64_t &z0, int64_t &z1) const {
+        Normal<double>::fixed(words(call), bm, z0, z1);
     }
     __device__ __forceinline__ void pair(uint32_t call, double &z0, double &z1) const {
         Normal<double>::pair(words(call), bm, z0, z1);
@@ -1099,7 +1109,7 @@ __global__ void __launch_bounds__(kThreads, MinCtas<R, RING, KS>::value) sampler
     off = (off + 15) & ~(size_t)15;
     float4 *zq = reinterpret_cast<float4 *>(smem_raw + off) + tid;           // single path only
     off += sizeof(R) == 4 ? sizeof(float4) * (size_t)staged_quads(P.F) * kThreads : 0;
-    bm::Tables *bm_smem = reinterpret_cast<bm::Tables *>(smem_raw + off);   // double path only
+    fx::Tables *bm_smem = reinterpret_cast<fx::Tables *>(smem_raw + off);   // double path only
 
     // stage the coefficient tables of every sampled level, the widths (and
     // the Box-Muller node tables of the double path)
@@ -1113,7 +1123,7 @@ __global__ void __launch_bounds__(kThreads, MinCtas<R, RING, KS>::value) sampler
                 tab_s[i] = g[i];
         }
         for (int i = tid; i <= SU_MAX_S; i += kThreads) sig[i] = (R)P.sigma[i];
-        if constexpr (sizeof(R) == 8) bm::tables_init(bm_smem, tid, kThreads);
+        if constexpr (sizeof(R) == 8) fx::tables_load(bm_smem, tid, kThreads);
     }
     __syncthreads();
     const PathCfg<R> pc{(R)P.a, (R)P.b, P.S, L, sig};
@@ -1250,8 +1260,8 @@ __global__ void __launch_bounds__(kThreads, BatchCtas<R, RING, KS>::value) batch
     off = (off + 15) & ~(size_t)15;
     float4 *zq = reinterpret_cast<float4 *>(smem_raw + off) + tid;           // single path only
     off += sizeof(R) == 4 ? sizeof(float4) * (size_t)staged_quads(kMaxFine, true) * kThreads : 0;
-    bm::Tables *bm_smem = reinterpret_cast<bm::Tables *>(smem_raw + off);
-    if constexpr (sizeof(R) == 8) bm::tables_init(bm_smem, tid, kThreads);
+    fx::Tables *bm_smem = reinterpret_cast<fx::Tables *>(smem_raw + off);
+    if constexpr (sizeof(R) == 8) fx::tables_load(bm_smem, tid, kThreads);
 
     Stream<R> st;
     st.key = make_uint2((uint32_t)P.seed, (uint32_t)(P.seed >> 32));

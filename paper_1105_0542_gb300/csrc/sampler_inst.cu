@@ -6,11 +6,14 @@
 // The build compiles this file once per combination so the kernels compile
 // in parallel.
 #include "sampler_impl.cuh"
+#ifdef SU_FIXED
+#include "sampler_fx.cuh"
+#endif
 
 #ifdef SU_FIXED
 // SU_FIXED = g: the single-precision even-ring samplers and batched kernels
 // with the table shapes k = g, g + kFixedGroups, .. of fixed_shapes.h
-// compiled in
+// compiled in, and the fixed-point double samplers with their tails in them
 namespace su {
 namespace {
 template <int K>
@@ -31,12 +34,22 @@ const void *fixed_batch_entry(int k) {
         return fixed_batch_entry<K + kFixedGroups>(k);
     }
 }
+template <int K>
+const void *fixed_fx_entry(int k) {
+    if constexpr (K >= kNumFixed) {
+        return nullptr;
+    } else {
+        if (k == K) return (const void *)sampler_fx_kernel<RING_EVEN, K>;
+        return fixed_fx_entry<K + kFixedGroups>(k);
+    }
+}
 }  // namespace
 
 #define SU_FIXED_NAME2(a, g) a##_##g
 #define SU_FIXED_NAME(a, g) SU_FIXED_NAME2(a, g)
 const void *SU_FIXED_NAME(sampler_fixed_entry, SU_FIXED)(int k) { return fixed_entry<SU_FIXED>(k); }
 const void *SU_FIXED_NAME(batch_fixed_entry, SU_FIXED)(int k) { return fixed_batch_entry<SU_FIXED>(k); }
+const void *SU_FIXED_NAME(sampler_fx_fixed_entry, SU_FIXED)(int k) { return fixed_fx_entry<SU_FIXED>(k); }
 }  // namespace su
 #else
 
