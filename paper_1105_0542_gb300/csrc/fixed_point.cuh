@@ -107,6 +107,99 @@ SU_FX_FN double to_double(int64_t x, int scale) {
 }
 
 // ---------------------------------------------------------------------------
+// z = tanh^2(y), 0 <= y < kTanhNodes / kTanhSteps, in units of 2^-62, from y in
+// units of 2^-53 steps of 1/64: in the step [i, i + 1) / 64 the Taylor polynomial
+// of degree 7 about its middle (the next term is at most 2^-58, at the ends of
+// the steps near y = 0), rewritten in f = 64 y - i in [0, 1).  Entries 0..4 are integers
+// in units of 2^-62, entry 5 (below 2^-30) in units of 2^-60, entries 6 and 7
+// (below 2^-36) single precision in units of 2^-60.
+constexpr int kTanhSteps = 64, kTanhNodes = 384;
+struct TanhNode {
+    int64_t c[5];
+    int32_t c5;
+    float f6, f7;
+    uint32_t pad;
+};
+struct TanhTable {
+    TanhNode n[kTanhNodes];
+};
+
+// a b / 2^120
+constexpr unsigned __int128 mul120(unsigned __int128 a, unsigned __int128 b) {
+    const unsigned __int128 m = ((unsigned __int128)1 << 60) - 1;
+    const unsigned __int128 ah = a >> 60, al = a & m, bh = b >> 60, bl = b & m;   // al bl / 2^120 is dropped
+    return ah * bh + ((ah * bl) >> 60) + ((al * bh) >> 60);
+}
+constexpr TanhTable make_tanh_table() {
+    TanhTable T{};
+    unsigned __int128 e = (unsigned __int128)1 << 120, term = e;   // exp(-1/64)
+    for (int k = 1; k < 20; ++k) {
+        term = term / (64 * k);
+        if (k & 1)
+            e -= term;
+        else
+            e += term;
+    }
+    const unsigned __int128 r = mul120(e, e);
+    const __int128 one = (__int128)1 << 62;
+    for (int i = 0; i < kTanhNodes; ++i, e = mul120(e, r)) {
+        // at y = (i + 1/2) / 64: e = exp(-2 y), a[n] the Taylor coefficients of tanh in units of 2^-62
+        const unsigned __int128 num = ((unsigned __int128)1 << 120) - e;
+        __int128 a[9] = {};
+        a[0] = (__int128)((num << 4) / (uint64_t)((((unsigned __int128)1 << 120) + e) >> 58));
+        for (int n = 0; n < 8; ++n) {
+            __int128 s = n == 0 ? one << 62 : 0;
+            for (int k = 0; k <= n; ++k) s -= a[k] * a[n - k];
+            a[n + 1] = ((s + ((__int128)1 << 61)) >> 62) / (n + 1);
+        }
+        // tanh^2 = 1 - tanh': in powers of (f - 1/2), units of 2^-104
+        __int128 b[8] = {};
+        for (int n = 0; n < 8; ++n) b[n] = ((n == 0 ? one - a[1] : -(n + 1) * a[n + 1]) * ((__int128)1 << 42)) >> (6 * n);
+        __int128 p[8] = {};
+        for (int k = 0; k < 8; ++k) {
+            __int128 binom = 1, s = 0;
+            for (int n = k; n < 8; ++n) {
+                const __int128 v = (b[n] * binom) >> (n - k);
+                s += ((n - k) & 1) ? -v : v;
+                binom = binom * (n + 1) / (n + 1 - k);
+            }
+            p[k] = s;
+        }
+        // entry k is multiplied by f (below 2^62) k times, each product a quarter: stored times 4^k
+        TanhNode &o = T.n[i];
+        for (int k = 0; k < 5; ++k)
+            o.c[k] = (int64_t)((p[k] + ((__int128)1 << (41 - 2 * k))) >> (42 - 2 * k)) - (k < 4 ? kBias : 0);
+        o.c5 = (int32_t)((p[5] + ((__int128)1 << 43)) >> 44);
+        o.f6 = (float)(double)(int64_t)(p[6] >> 30) * 0x1p-14f;
+        o.f7 = (float)(double)(int64_t)(p[7] >> 30) * 0x1p-14f;
+    }
+    return T;
+}
+
+#ifdef __CUDACC__
+static __device__ const TanhTable g_tanh = make_tanh_table();
+// the first n nodes into shared memory
+__device__ __forceinline__ void tanh_load(TanhNode *t, int n, int tid, int nthreads) {
+    const uint2 *s = reinterpret_cast<const uint2 *>(&g_tanh);
+    uint2 *d = reinterpret_cast<uint2 *>(t);
+    for (int i = tid; i < n * (int)(sizeof(TanhNode) / 8); i += nthreads) d[i] = s[i];
+}
+#endif
+
+SU_FX_FN int64_t tanh2(int64_t w, const TanhNode *__restrict__ t) {
+    const TanhNode &n = t[(int)(w >> 53)];
+    const int64_t f = (int64_t)(((uint64_t)w << 11) >> 2);         // units 2^-62
+    const Limbs fl = limbs(f);
+    const float ff = (float)hi32(f) * 0x1p-30f;
+    const int32_t g5 = n.c5 + round_int(ff * fmaf(ff, n.f7, n.f6));
+    int64_t g = n.c[4] + (int64_t)mulhi(g5, hi32(f)) * 4096;       // 2^-60 f -> 2^-62 / 4^4
+    g = mul_add(g, fl, n.c[3]);
+    g = mul_add(g, fl, n.c[2]);
+    g = mul_add(g, fl, n.c[1]);
+    return mul_add(g, fl, n.c[0]);
+}
+
+// ---------------------------------------------------------------------------
 // Box-Muller in fixed point: z0 = R cos(theta), z1 = R sin(theta),
 // R = sqrt(-2 ln u1), theta = 2 pi u2 (Sec. 4.1, both branches) for the 53-bit
 // uniforms u1 = (a + 1/2) 2^-53, u2 = (b + 1/2) 2^-53, as integers in units of

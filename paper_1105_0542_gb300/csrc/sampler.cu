@@ -29,7 +29,7 @@ const void *batch_entry_f32_0();
 const void *batch_entry_f32_1();
 const void *batch_entry_f32_2();
 // the double sampler in fixed point (sampler_fx.cu)
-const void *sampler_fx_entry();
+const void *sampler_fx_entry(int ring);
 size_t sampler_fx_smem_bytes(const SamplerParams &P);
 // the compiled-shape kernels of group g = k % kFixedGroups (sampler_inst.cu, SU_FIXED = g)
 #define SU_FIXED_GROUP(g)                        \
@@ -169,8 +169,8 @@ const void *pick_fixed(const SamplerParams &P, int precision) {
 
 const void *pick(const SamplerParams &P, int precision) {
     if (P.fx.on) {
-        const int k = fixed_shape_index(P.ncol, P.len);
-        return k < 0 ? sampler_fx_entry() : kFxFixed[k % kFixedGroups](k);
+        const int k = P.ring == RING_EVEN ? fixed_shape_index(P.ncol, P.len) : -1;
+        return k < 0 ? sampler_fx_entry(P.ring) : kFxFixed[k % kFixedGroups](k);
     }
     if (const void *fn = pick_fixed(P, precision)) return fn;
     if (P.ring == RING_GENERAL) return precision == SU_FP64 ? sampler_entry_f64_3() : nullptr;

@@ -41,7 +41,7 @@ struct GeneralDev {
 
 // The fixed-point sampler's plan (sampler_fx.cuh; built by fx_plan).  Path
 // points are integers in units of q_unit; row d of the arrays is level n = S - d.
-constexpr int kFxCols = 4;
+constexpr int kFxCols = 8;
 struct FxLevel {
     int ok;                   // evaluated in fixed point, else in double
     int nc, h[kFxCols];       // columns with integer entries, and how many each (the others in single precision)
@@ -54,6 +54,7 @@ struct FxParams {
     int on;
     int qlim;                 // |high word of q| stays below this
     int hrow;                 // room for integer entries per level
+    int ah, al, nodes;        // RING_TANH2: limbs of us -> alpha us / 2 in node steps, nodes in reach
     int sgh[SU_MAX_S + 1], sgl[SU_MAX_S + 1], shl[SU_MAX_S + 1];   // sigma_n: limbs and left shift of the product
     int64_t qa, qb;           // endpoints
     double q_unit;

@@ -52,6 +52,7 @@ constexpr int kFxSeg = 4;                        // segments of 2^4 slices (fewe
 constexpr int kRowQ = SU_MAX_S - kFxSeg + 1;
 constexpr int kFxRows = kRowQ + (1 << kFxSeg) + 1;
 struct FxView {
+    const fx::TanhNode *th;  // RING_TANH2: its nodes
     const float2 *tail;      // [S][M] single-precision entries as pairs {c, c}, zero where the entry is an integer one
     const int64_t *head;     // [S][hrow]
     int64_t *R;              // this thread's first row
@@ -62,15 +63,12 @@ struct FxView {
 // The sum of -eps W_p over B slices, integer part, in units of 2^-e: nested
 // Horner over the leading entries (last column first), B chains side by side.
 template <int B>
-__device__ __forceinline__ int64_t fx_heads(const int64_t (&us)[B], const int64_t (&vs)[B], const FxLevel &L,
+__device__ __forceinline__ int64_t fx_heads(const fx::Limbs (&Z)[B], const int64_t (&vs)[B], const FxLevel &L,
                                             const int64_t *__restrict__ h) {
-    fx::Limbs Z[B], Y[B];
+    fx::Limbs Y[B];
     int64_t acc[B];
 #pragma unroll
-    for (int b = 0; b < B; ++b) {
-        Z[b] = fx::limbs(fx::square(fx::limbs(us[b])) << 1);
-        Y[b] = fx::limbs(fx::square(fx::limbs(vs[b] << L.ky)));
-    }
+    for (int b = 0; b < B; ++b) Y[b] = fx::limbs(fx::square(fx::limbs(vs[b] << L.ky)) << 1);
     for (int j = L.nc - 1; j >= 0; --j) {
         int64_t g[B];
         const int64_t top = *h++;
@@ -95,16 +93,29 @@ __device__ __forceinline__ int64_t fx_heads(const int64_t (&us)[B], const int64_
     return s;
 }
 
-// z = (us / 2Q)^2 and y = (vs / V)^2 in single precision, from the high words
+// z in units of 2^-63 from us
+template <int RING>
+__device__ __forceinline__ fx::Limbs fx_ring(int64_t us, const FxParams &X, const fx::TanhNode *th) {
+    if constexpr (RING == RING_EVEN)
+        return fx::limbs(fx::square(fx::limbs(us)) << 1);
+    else
+        return fx::limbs(fx::tanh2(fx::mul(us < 0 ? -us : us, fx::Limbs{X.ah, X.al}), th) << 1);
+}
+
+// a high word in units of 1
 __device__ __forceinline__ float fx_unit(int32_t h) { return (float)h * 0x1p-31f; }
 
 // BT slices between the points q[k stp], k = 0..BT: the single-precision
 // entries (packed pairs of slices), then in batches of four the integer ones.
-template <int BT, typename SP>
-__device__ __forceinline__ void fx_batch(const int64_t *__restrict__ q, int stp, const FxLevel &L,
-                                         const float2 *__restrict__ tail, const int64_t *__restrict__ head, const SP &P,
-                                         float2 &ts, Acc96 &acc, int &vm) {
+// (z = us^2 is cheaper made again for them than kept, tanh^2 is kept.)
+template <int RING, int BT, typename SP>
+__device__ __forceinline__ void fx_batch(const int64_t *__restrict__ q, int stp, const FxLevel &L, const FxParams &X,
+                                         const fx::TanhNode *th, const float2 *__restrict__ tail,
+                                         const int64_t *__restrict__ head, const SP &P, float2 &ts, Acc96 &acc,
+                                         int &vm) {
     constexpr int BP = BT < 2 ? 1 : BT / 2;
+    constexpr bool kKeep = RING != RING_EVEN;
+    fx::Limbs Zk[kKeep ? BT : 1];
     float2 Zf[BP], Yf[BP], af[BP];
     {
         int64_t l = q[0];
@@ -121,11 +132,17 @@ __device__ __forceinline__ void fx_batch(const int64_t *__restrict__ q, int stp,
                 const int64_t r = q[(2 * m + s + 1) * stp];
                 const int64_t us = l + r, vs = r - l;
                 vm = max(vm, abs(fx::hi32(vs)));
-                u[s] = fx_unit(fx::hi32(us));
+                if constexpr (kKeep) {
+                    Zk[2 * m + s] = fx_ring<RING>(us, X, th);
+                    u[s] = fx_unit(Zk[2 * m + s].h);
+                } else {
+                    u[s] = fx_unit(fx::hi32(us));
+                }
                 v[s] = fx_unit((int32_t)__funnelshift_l(fx::lo32(vs), (uint32_t)fx::hi32(vs), L.ky));
                 l = r;
             }
-            Zf[m] = __fmul2_rn(make_float2(u[0], u[1]), make_float2(u[0], u[1]));
+            Zf[m] = kKeep ? make_float2(u[0], u[1])
+                          : __fmul2_rn(make_float2(u[0], u[1]), make_float2(u[0], u[1]));
             Yf[m] = __fmul2_rn(make_float2(v[0], v[1]), make_float2(v[0], v[1]));
         }
     }
@@ -133,35 +150,45 @@ __device__ __forceinline__ void fx_batch(const int64_t *__restrict__ q, int stp,
 #pragma unroll
     for (int m = 0; m < BP; ++m) ts = __fadd2_rn(ts, BT < 2 ? make_float2(af[m].x, 0.f) : af[m]);
     constexpr int B = BT < 4 ? BT : 4;
-#pragma unroll 1
-    for (int k1 = 0; k1 < BT; k1 += B) {
-        int64_t us[B], vs[B], l = q[k1 * stp];
+    auto heads = [&](int k1) {
+        fx::Limbs Z[B];
+        int64_t vs[B], l = q[k1 * stp];
 #pragma unroll
         for (int b = 0; b < B; ++b) {
             const int64_t r = q[(k1 + b + 1) * stp];
-            us[b] = l + r;
+            if constexpr (kKeep)
+                Z[b] = Zk[k1 + b];
+            else
+                Z[b] = fx_ring<RING>(l + r, X, th);
             vs[b] = r - l;
             l = r;
         }
-        acc.add(fx_heads<B>(us, vs, L, head));
+        acc.add(fx_heads<B>(Z, vs, L, head));
+    };
+    if constexpr (kKeep) {   // unrolled: Zk stays in registers
+#pragma unroll
+        for (int k1 = 0; k1 < BT; k1 += B) heads(k1);
+    } else {
+#pragma unroll 1
+        for (int k1 = 0; k1 < BT; k1 += B) heads(k1);
     }
 }
 
 // One level of a segment: ns slices between points stp apart (2^F = ns stp / kThreads).
-template <typename SP>
+template <int RING, typename SP>
 __device__ __forceinline__ void fx_level(const int64_t *__restrict__ q, int ns, int stp, const FxLevel &L,
-                                         const float2 *__restrict__ tail, const int64_t *__restrict__ head, const SP &P,
+                                         const FxParams &X, const fx::TanhNode *th, const float2 *__restrict__ tail, const int64_t *__restrict__ head, const SP &P,
                                          Acc96 &acc, bool &bad) {
     float2 ts = make_float2(0.f, 0.f);
     int vm = 0;
     if (ns >= 8) {
 #pragma unroll 1
-        for (int k = 0; k < ns; k += 8) fx_batch<8>(q + k * stp, stp, L, tail, head, P, ts, acc, vm);
+        for (int k = 0; k < ns; k += 8) fx_batch<RING, 8>(q + k * stp, stp, L, X, th, tail, head, P, ts, acc, vm);
     } else if (ns == 4) {
-        fx_batch<4>(q, stp, L, tail, head, P, ts, acc, vm);
+        fx_batch<RING, 4>(q, stp, L, X, th, tail, head, P, ts, acc, vm);
     } else {
 #pragma unroll 1
-        for (int k = 0; k < ns; ++k) fx_batch<1>(q + k * stp, stp, L, tail, head, P, ts, acc, vm);
+        for (int k = 0; k < ns; ++k) fx_batch<RING, 1>(q + k * stp, stp, L, X, th, tail, head, P, ts, acc, vm);
     }
     acc.add(__float2ll_rn(ts.x + ts.y));
     bad |= vm >= L.vlim;
@@ -234,7 +261,7 @@ __device__ __forceinline__ void fx_path(const SamplerParams &P, const SP &V, con
         const FxLevel &L = X.lv[d];
         if (L.ok) {
             Acc96 a = acc[d];
-            fx_level(q, ns, stp, L, sm.tail + d * P.M, sm.head + d * X.hrow, V, a, bad);
+            fx_level<RING>(q, ns, stp, L, X, sm.th, sm.tail + d * P.M, sm.head + d * X.hrow, V, a, bad);
             acc[d] = a;
         } else {
             for (int k = 0; k < ns; ++k)
@@ -315,7 +342,7 @@ __device__ __forceinline__ void fx_path(const SamplerParams &P, const SP &V, con
 }
 
 // ------------------------------------------------------------------ the kernel
-// Shared memory: node tables | tail[S][M] pairs | head[S][hrow] | rows[kFxRows][kThreads];
+// Shared memory: node tables | tail[S][M] pairs | head[S][hrow] | tanh nodes | rows[kFxRows][kThreads];
 // the weights sw[levels][chunk] in the rows where one round needs no more,
 // else after them.
 __host__ __device__ inline bool fx_share_sw(const SamplerParams &P) {
@@ -334,9 +361,12 @@ __global__ void __launch_bounds__(kThreads, 4) sampler_fx_kernel(const __grid_co
     off += sizeof(float2) * (size_t)P.S * P.M;
     int64_t *head = reinterpret_cast<int64_t *>(smem_raw + off);
     off += sizeof(int64_t) * (size_t)P.S * P.fx.hrow;
+    fx::TanhNode *th = reinterpret_cast<fx::TanhNode *>(smem_raw + off);
+    if constexpr (RING == RING_TANH2) off += sizeof(fx::TanhNode) * (size_t)P.fx.nodes;
     int64_t *rows = reinterpret_cast<int64_t *>(smem_raw + off);
     double *sw = reinterpret_cast<double *>(rows + (fx_share_sw(P) ? 0 : kFxRows * kThreads));
     FxView sm;
+    sm.th = th;
     sm.tail = tail;
     sm.head = head;
     sm.R = rows + tid;
@@ -345,6 +375,7 @@ __global__ void __launch_bounds__(kThreads, 4) sampler_fx_kernel(const __grid_co
         const float *gt = reinterpret_cast<const float *>(g + P.fx.tail_off);
         const int64_t *gh = reinterpret_cast<const int64_t *>(g + P.fx.head_off);
         fx::tables_load(bm, tid, kThreads);
+        if constexpr (RING == RING_TANH2) fx::tanh_load(th, P.fx.nodes, tid, kThreads);
         for (int i = tid; i < P.S * P.M; i += kThreads) tail[i] = make_float2(gt[i], gt[i]);
         for (int i = tid; i < P.S * P.fx.hrow; i += kThreads) head[i] = gh[i];
     }

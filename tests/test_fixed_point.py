@@ -24,6 +24,8 @@ extern "C" void normals(const uint32_t *w, long n, double *z) {
         z[2 * i + 1] = fx::to_double(b, -fx::kZScale);
     }
 }
+static const fx::TanhTable H = fx::make_tanh_table();
+extern "C" int64_t tanh2(int64_t w) { return fx::tanh2(w, H.n); }
 extern "C" int64_t mul(int64_t x, int64_t f) { return fx::mul(x, fx::limbs(f)); }
 extern "C" int64_t square(int64_t x) { return fx::square(fx::limbs(x)); }
 extern "C" double to_double(int64_t x, int s) { return fx::to_double(x, s); }
@@ -41,6 +43,7 @@ def lib(tmp_path_factory):
     i64 = ctypes.c_int64
     L.mul.argtypes, L.mul.restype = [i64, i64], i64
     L.square.argtypes, L.square.restype = [i64], i64
+    L.tanh2.argtypes, L.tanh2.restype = [i64], i64
     L.to_double.argtypes, L.to_double.restype = [i64, ctypes.c_int], ctypes.c_double
     return L
 
@@ -73,3 +76,13 @@ def test_products_and_conversions(lib):
         if abs(x) < 2 ** 63 - 2 ** 32:
             assert 0 <= (x * x >> 64) - lib.square(x) <= 2
         assert lib.to_double(x, -57) == pytest.approx(x * 2.0 ** -57, rel=2.0 ** -53)
+
+
+def test_tanh2(lib):
+    """z = tanh^2(w 2^-59) in units of 2^-62 against the same in double: the
+    argument's rounding to a double and tanh's own are below 4 2^-53 z."""
+    rng = np.random.default_rng(6)
+    ws = [int(v) for v in rng.integers(0, 384 * 2 ** 53, 2000)] + [(i << 53) + e for i in (0, 1, 63, 383) for e in (0, 1, 2 ** 53 - 1)]
+    for w in ws:
+        z = np.tanh(w * 2.0 ** -59) ** 2
+        assert abs(lib.tanh2(w) * 2.0 ** -62 - z) <= 2.0 ** -57 + 2.0 ** -51 * z

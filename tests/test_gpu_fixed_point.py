@@ -28,6 +28,7 @@ CASES = [("ho", [1.0], 0.0, 1.0, 1.0, 4, s, 129, s0) for s, s0 in ((1, 0), (2, 0
 CASES += [("aho", [1.0, 1.0], -0.3, 0.4, 0.5, p, s, 257, s0)
           for p, s, s0 in ((1, 5, 0), (4, 1, FAR[1] - 100), (7, 6, 0), (10, 4, FAR[2] - 128), (18, 10, FAR[0] - 3),
                            (21, 7, FAR[1] - 255))]
+CASES += [("mpt", [1.5, 1.2], -0.4, 0.6, 0.5, p, s, 130, s0) for p, s, s0 in ((1, 3, 0), (4, 6, FAR[0] - 64), (10, 9, 0), (12, 5, FAR[2]))]
 CASES += [("dw", [1.0], -1.0, 1.0, 1.0, 12, 8, 100, 0), ("poly", [0.1, 0.0, 0.5, 0.0, 0.1, 0.0, 0.02], 0.2, 0.0, 0.3, 5, 7, 64, 0)]
 
 
