@@ -588,34 +588,75 @@ static int configure_nd(su_plan &pl) {
             tabd[(size_t)d * M + i] = t[(size_t)i];
         }
     }
+    // the program over all entries, the level tables in its order (the kernel's
+    // variables are 2 x and 2 xb), and in double precision each level's split
     const size_t rs = prec == SU_FP32 ? sizeof(float) : sizeof(double);
-    std::vector<unsigned char> blob(tabd.size() * rs);
-    if (prec == SU_FP32)
-        for (size_t i = 0; i < tabd.size(); ++i) reinterpret_cast<float *>(blob.data())[i] = (float)tabd[i];
-    else
-        std::memcpy(blob.data(), tabd.data(), blob.size());
-    int ndev = 0;
-    cudaError_t e = cudaGetDeviceCount(&ndev);
-    if (e != cudaSuccess || ndev == 0) {
-        cudaGetLastError();
-        return fail(SU_ECUDA, "no CUDA device available (%s)", cudaGetErrorString(e));
+    const int nv = 2 * pl.nd;
+    NdParams &Q = pl.Q;
+    std::memset(&Q, 0, sizeof Q);
+    NdProgram G;
+    std::vector<int> every((size_t)M), heads;
+    for (int i = 0; i < M; ++i) every[(size_t)i] = i;
+    nd_order(pl.N.mono, nv, Q.order);
+    nd_program(pl.N.mono, every, nv, Q.order, G);
+    const int Mp = (int)G.slot.size();
+    auto scaled = [&](int d, int e) {
+        int deg = 0;
+        for (unsigned char x : pl.N.mono[(size_t)e]) deg += x;
+        return std::ldexp(tabd[(size_t)d * M + e], -deg);
+    };
+    std::vector<double> full((size_t)std::max(S, 1) * Mp, 0.0);
+    std::vector<float> pairs((size_t)std::max(S, 1) * Mp * 2, 0.0f);
+    std::vector<uint32_t> hwords;
+    std::vector<double> hcoef;
+    for (int d = 0; d < S; ++d) {
+        std::vector<char> in_double((size_t)M, 0);
+        if (prec == SU_FP64 && d < pl.levels && pl.opt.kernel == 0) {
+            nd_split(pl.N.mono, pl.nd, pl.nd_a.data(), pl.nd_b.data(), pl.T, S - d,
+                     std::vector<double>(tabd.begin() + (long)d * M, tabd.begin() + (long)(d + 1) * M), heads);
+            // worth it where the double part is short; the others have to be floats
+            std::vector<char> head((size_t)M, 0);
+            for (int e : heads) head[(size_t)e] = 1;
+            bool fits = !heads.empty() && 2 * heads.size() <= (size_t)M;
+            for (int e = 0; e < M; ++e) fits = fits && (head[(size_t)e] || std::fabs(scaled(d, e)) < 1e30);
+            if (fits) {
+                NdProgram H;
+                nd_program(pl.N.mono, heads, nv, Q.order, H);
+                Q.heads[d] = (int)heads.size();
+                Q.hsq[d] = H.sq;
+                Q.hw[d] = (int)hwords.size();
+                Q.hc[d] = (int)hcoef.size();
+                hwords.insert(hwords.end(), H.words.begin(), H.words.end());
+                for (int e : H.slot) hcoef.push_back(e < 0 ? 0.0 : scaled(d, e));
+                for (int e : heads) in_double[(size_t)e] = 1;
+            }
+        }
+        for (int i = 0; i < Mp; ++i) {
+            const int e = G.slot[(size_t)i];
+            if (e < 0) continue;
+            full[(size_t)d * Mp + i] = scaled(d, e);
+            pairs[2 * ((size_t)d * Mp + i)] = pairs[2 * ((size_t)d * Mp + i) + 1] = in_double[(size_t)e] ? 0.0f : (float)scaled(d, e);
+        }
     }
-    CU(cudaGetDevice(&pl.device), "cudaGetDevice");
-    int sms = 0;
-    CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, pl.device), "SM count");
+    int sms = 0, smem_max = 0;
+    int rc = device_limits(pl.device, sms, smem_max);
+    if (rc) return rc;
+    // one device block: full tables (double) | pairs | double parts | words
+    std::vector<unsigned char> blob;
+    auto put = [&](const void *src, size_t bytes) {
+        const size_t at = blob.size();
+        blob.resize((at + bytes + 255) / 256 * 256, 0);
+        if (bytes) std::memcpy(blob.data() + at, src, bytes);
+        return at;
+    };
+    const size_t o_full = prec == SU_FP64 ? put(full.data(), full.size() * sizeof(double)) : 0;
+    const size_t o_pairs = put(pairs.data(), pairs.size() * sizeof(float));
+    const size_t o_hc = put(hcoef.data(), hcoef.size() * sizeof(double));
+    const size_t o_hw = put(hwords.data(), hwords.size() * sizeof(uint32_t));
+    const size_t o_w = put(G.words.data(), G.words.size() * sizeof(uint32_t));
     CU(dmalloc(&pl.d_tables, blob.size()), "device allocation (tables)");
     CU(cudaMemcpy(pl.d_tables, blob.data(), blob.size(), cudaMemcpyHostToDevice), "upload tables");
-    std::vector<GeneralNode> nodes(pl.N.depth.size());
-    for (size_t t = 0; t < nodes.size(); ++t) {
-        if (pl.N.count[t] > 65535) return fail(SU_ENOTSUP, "a monomial group has more than 65535 entries");
-        nodes[t].depth = (unsigned char)pl.N.depth[t];
-        nodes[t].sym = (unsigned char)pl.N.sym[t];
-        nodes[t].count = (unsigned short)pl.N.count[t];
-        nodes[t].first = pl.N.first[t];
-    }
-    CU(dmalloc(&pl.d_general, nodes.size() * sizeof(GeneralNode)), "device allocation (program)");
-    CU(cudaMemcpy(pl.d_general, nodes.data(), nodes.size() * sizeof(GeneralNode), cudaMemcpyHostToDevice),
-       "upload program");
+    unsigned char *dev = static_cast<unsigned char *>(pl.d_tables);
 
     SamplerParams &P = pl.P;
     std::memset(&P, 0, sizeof P);
@@ -624,8 +665,8 @@ static int configure_nd(su_plan &pl) {
     P.F = 0;
     P.rounds = 1;
     P.levels = pl.levels;
-    P.M = M;
-    P.tables = pl.d_tables;
+    P.M = Mp;
+    P.tables = prec == SU_FP64 ? dev + o_full : dev + o_pairs;
     P.seed = pl.seed;
     P.instance = pl.opt.instance;
     P.n_mc = pl.n_mc;
@@ -634,19 +675,28 @@ static int configure_nd(su_plan &pl) {
     const int64_t bsz = (pl.n_mc + pl.n_blocks - 1) / pl.n_blocks;
     P.items_per_block = (bsz + kThreads - 1) / kThreads;
     P.n_items = P.items_per_block * pl.n_blocks;
-    NdParams &Q = pl.Q;
-    std::memset(&Q, 0, sizeof Q);
     Q.base = P;
     Q.D = pl.nd;
-    Q.H = pl.N.H;
-    Q.G = pl.N.G;
-    Q.n_nodes = (int)nodes.size();
-    Q.nodes = static_cast<const GeneralNode *>(pl.d_general);
+    Q.sq = G.sq;
+    Q.n_words = (int)G.words.size();
+    Q.words = reinterpret_cast<const uint32_t *>(dev + o_w);
+    Q.tail = reinterpret_cast<const float2 *>(dev + o_pairs);
+    Q.hwords = reinterpret_cast<const uint32_t *>(dev + o_hw);
+    Q.hcoef = reinterpret_cast<const double *>(dev + o_hc);
+    Q.n_hwords = (int)hwords.size();
+    Q.n_hcoef = (int)hcoef.size();
     for (int c = 0; c < pl.nd; ++c) {
         Q.a[c] = pl.nd_a[(size_t)c];
         Q.b[c] = pl.nd_b[(size_t)c];
+        Q.reach[c] = std::max(std::fabs(Q.a[c]), std::fabs(Q.b[c])) + 2.4 * std::sqrt(pl.T);
     }
+    // program and tables in shared memory where that leaves the register-bound residency
+    Q.staged = 1;
     pl.smem = nd_smem_bytes(Q, prec);
+    if (pl.smem > (size_t)std::min(smem_max, 56 * 1024)) {
+        Q.staged = 0;
+        pl.smem = nd_smem_bytes(Q, prec);
+    }
     const int occ = nd_occupancy(Q, prec, pl.smem);
     if (occ < 1) return fail(SU_ECUDA, "sampler cannot be resident (%s)", cudaGetErrorString(cudaGetLastError()));
     pl.grid = (int)std::min<int64_t>(P.n_items, (int64_t)sms * occ);

@@ -9,125 +9,130 @@
 namespace su {
 namespace {
 
-// z[sym] with z in registers: a chain of selects on the integer pipes
-// instead of a dynamically indexed local-memory load
-template <typename R, int D>
-__device__ __forceinline__ R pick(const R (&z)[2 * D], int sym) {
-    R v = z[0];
-#pragma unroll
-    for (int i = 1; i < 2 * D; ++i) v = sym == i ? z[i] : v;
-    return v;
-}
+// Lanes of the evaluation: two slices in a packed pair of floats, or one double.
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ void vzero(float2 &a) { a = make_float2(0.f, 0.f); }
+__device__ __forceinline__ void vzero(double &a) { a = 0.0; }
 
-// out[i] = in[i] * z[i][sym] for the B slices.  sym is the same for every
-// thread (a node of the program): from three coordinates on a chain of
-// uniform branches picks the register (2d - 1 selects per slice cost more:
-// the 3D anharmonic oscillator in single precision 147 -> 135 ms); with one
-// or two coordinates the selects are as fast.
-template <typename R, int D, int B, int K = 0>
-__device__ __forceinline__ void mul_sym(R (&out)[B], const R (&in)[B], const R (&z)[B][2 * D], int sym) {
-    if constexpr (D < 3) {
+// The variables of B lanes in program order: z_k, and the Horner variable of
+// depth k (z_k or its square).
+template <typename VT, int NV, int B>
+struct Vars {
+    VT z[NV][B], m[NV][B];
+    __device__ __forceinline__ void close(unsigned sq) {
 #pragma unroll
-        for (int i = 0; i < B; ++i) out[i] = in[i] * pick<R, D>(z[i], sym);
-    } else if constexpr (K < 2 * D - 1) {
-        if (sym == K) {
+        for (int k = 0; k < NV; ++k)
 #pragma unroll
-            for (int i = 0; i < B; ++i) out[i] = in[i] * z[i][K];
-        } else {
-            mul_sym<R, D, B, K + 1>(out, in, z, sym);
+            for (int i = 0; i < B; ++i) m[k][i] = (sq >> k) & 1 ? vmul(z[k][i], z[k][i]) : z[k][i];
+    }
+};
+
+// t = the polynomial in z_K.. at w (words) and c (coefficients), both moved past it
+template <int K, typename VT, int NV, int B>
+__device__ __forceinline__ void nd_poly(const uint32_t *__restrict__ &w, const VT *__restrict__ &c,
+                                        const Vars<VT, NV, B> &v, VT (&t)[B]) {
+    const uint32_t hd = *w++;
+    const int n = (int)(hd & 0xffffu);
+    if constexpr (K == NV - 1) {
+#pragma unroll
+        for (int i = 0; i < B; ++i) vzero(t[i]);
+        if (n) {
+            const VT top = *c;
+#pragma unroll
+            for (int i = 0; i < B; ++i) t[i] = top;
+#pragma unroll 1
+            for (int e = 1; e < n; ++e) {
+                const VT ce = c[e];
+#pragma unroll
+                for (int i = 0; i < B; ++i) t[i] = vfma(t[i], v.m[K][i], ce);
+            }
+            c += n;
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < B; ++i) out[i] = in[i] * z[i][K];
+        for (int i = 0; i < B; ++i) vzero(t[i]);
+#pragma unroll 1
+        for (int e = 0; e < n; ++e) {
+            VT u[B];
+            nd_poly<K + 1>(w, c, v, u);
+#pragma unroll
+            for (int i = 0; i < B; ++i) t[i] = vfma(t[i], v.m[K][i], u[i]);
+        }
+    }
+    if (hd & kNdOdd) {
+#pragma unroll
+        for (int i = 0; i < B; ++i) t[i] = vmul(t[i], v.z[K][i]);
     }
 }
 
-// One stack entry of B slices as one aligned vector (8 to 32 bytes: one or
-// two 16-byte local accesses per node for all B slices).
-template <typename R, int B>
-struct alignas(sizeof(R) * B) Lanes {
-    R v[B];
-};
+// x (rounded to nearest) for |x| < 2^127 as a float, on the integer pipes
+__device__ __forceinline__ float narrow(double x) {
+    const uint64_t u = (uint64_t)__double_as_longlong(x);
+    const uint64_t mag = (u & 0x7FFFFFFFFFFFFFFFULL) + (1ULL << 28);
+    const uint32_t f = mag >= (897ULL << 52) ? (uint32_t)(mag >> 29) - (896u << 23) : 0u;
+    return __uint_as_float(f | ((uint32_t)(u >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ float narrow(float x) { return x; }
 
-// -eps W for B slices at once, each with variables z = (x_1..x_D, xb_1..xb_D):
-// the monomial program walked depth first (each prefix node its parent times
-// one variable, the parent the top of the stack), each node's entries
-// combined by Horner in z_H^G and added times its monomial; the B slices
-// share every node and coefficient load.
-template <typename R, int D, int B>
-__device__ __forceinline__ void nd_multi(const R (&z)[B][2 * D], const R *__restrict__ coef, const NdParams &Q,
-                                         R (&w)[B]) {
-    Lanes<R, B> stk[kNdMaxDepth + 1];
-    R Y[B], acc[B];
+// the sum of 2 BP slices' -eps W in single precision (points pt(k0 stp).. of R)
+template <typename R, int D, int BP, typename PT>
+__device__ __forceinline__ float nd_single(const NdParams &Q, const uint32_t *w, const float2 *c, PT &&pt, int k0, int stp) {
+    Vars<float2, 2 * D, BP> v;
 #pragma unroll
-    for (int i = 0; i < B; ++i) {
-        stk[0].v[i] = 1;
-        acc[i] = 0;
-        Y[i] = 1;
-    }
-    for (int g = 0; g < Q.G; ++g) mul_sym<R, D, B>(Y, Y, z, Q.H);
-    const GeneralNode *__restrict__ nodes = Q.nodes;
-    for (int t = 0; t < Q.n_nodes; ++t) {
-        const GeneralNode nd = nodes[t];
-        Lanes<R, B> m;
-        if (t) {
-            const Lanes<R, B> par = stk[nd.depth - 1];
-            mul_sym<R, D, B>(m.v, par.v, z, nd.sym);
-            stk[nd.depth] = m;
-        } else {
+    for (int k = 0; k < 2 * D; ++k) {
+        // l + r = 2x of a coordinate, or r - l = 2xb (the entries carry the powers of two)
+        const int var = Q.order[k], cc = var >= D ? var - D : var;
+        const R sg = var >= D ? (R)-1 : (R)1;
+        R l = pt(k0 * stp, cc);
 #pragma unroll
-            for (int i = 0; i < B; ++i) m.v[i] = 1;
-        }
-        const int cnt = nd.count;
-        if (cnt) {
-            const R *c = coef + nd.first;
-            R h[B];
-            const R top = c[cnt - 1];
-#pragma unroll
-            for (int i = 0; i < B; ++i) h[i] = top;
-#pragma unroll 4
-            for (int e = cnt - 2; e >= 0; --e) {
-                const R ce = c[e];
-#pragma unroll
-                for (int i = 0; i < B; ++i) h[i] = fma(h[i], Y[i], ce);
-            }
-#pragma unroll
-            for (int i = 0; i < B; ++i) acc[i] = fma(h[i], m.v[i], acc[i]);
+        for (int i = 0; i < BP; ++i) {
+            const R a = pt((k0 + 2 * i + 1) * stp, cc), b = pt((k0 + 2 * i + 2) * stp, cc);
+            v.z[k][i] = make_float2(narrow(fma(sg, l, a)), narrow(fma(sg, a, b)));
+            l = b;
         }
     }
+    v.close(Q.sq);
+    float2 t[BP];
+    nd_poly<0>(w, c, v, t);
+    float s = 0;
 #pragma unroll
-    for (int i = 0; i < B; ++i) w[i] = acc[i];
+    for (int i = 0; i < BP; ++i) s += t[i].x + t[i].y;
+    return s;
 }
 
-// Slices k..k+B-1 of a level (points pt(k*stp) .. pt((k+B)*stp)), added to w
-// two at a time in ascending order.
-template <typename R, int D, int B, typename PT>
-__device__ __forceinline__ void nd_block(const R *__restrict__ tab, const NdParams &Q, PT &&pt, int k, int stp,
-                                         R &w) {
-    R z[B][2 * D];
+// two slices' -eps W in double
+template <int D, typename PT>
+__device__ __forceinline__ double nd_double(const NdParams &Q, unsigned sq, const uint32_t *w, const double *c, PT &&pt,
+                                            int k0, int stp) {
+    Vars<double, 2 * D, 2> v;
 #pragma unroll
-    for (int c = 0; c < D; ++c) {
-        R pl = pt(k * stp, c);
-#pragma unroll
-        for (int i = 0; i < B; ++i) {
-            const R pr = pt((k + i + 1) * stp, c);
-            z[i][c] = (R)0.5 * (pl + pr);
-            z[i][D + c] = (R)0.5 * (pr - pl);
-            pl = pr;
-        }
+    for (int k = 0; k < 2 * D; ++k) {
+        const int var = Q.order[k], cc = var >= D ? var - D : var;
+        const double sg = var >= D ? -1.0 : 1.0;
+        const double a = pt(k0 * stp, cc), b = pt((k0 + 1) * stp, cc), e = pt((k0 + 2) * stp, cc);
+        v.z[k][0] = fma(sg, a, b);
+        v.z[k][1] = fma(sg, b, e);
     }
-    R wv[B];
-    nd_multi<R, D, B>(z, tab, Q, wv);
-#pragma unroll
-    for (int i = 0; i < B; i += 2) w += wv[i] + wv[i + 1];
+    v.close(sq);
+    double t[2];
+    nd_poly<0>(w, c, v, t);
+    return t[0] + t[1];
 }
 
-// R = double or float (the path, W and the per-level sums; the item's
-// log-sum-exp tuples in double either way).
-// Shared memory: sw[levels][kThreads] (R, reduced runs) | Box-Muller node tables (double).
+// R = double or float (the path and the per-level sums; the item's log-sum-exp
+// tuples in double either way).
+// Shared memory: sw[levels][kThreads] (R, reduced runs) | Box-Muller node tables
+// (double) | where Q.staged: words | pairs [S][M] | double part's entries, words.
 // Global scratch per slot: the 2^(S-F) + 1 segment endpoints (F = min(S, kNdSeg)).
+//
+// What bounds it.  Single precision: instruction issue, most of it the packed
+// multiply-adds of the nest and the loops around them.  Double: the FP64 pipe
+// (2 lanes a cycle) in the double part, a tenth of the entries on fine levels.
 template <typename R, int D>
-__global__ void __launch_bounds__(kThreads, 4) nd_kernel(const __grid_constant__ NdParams Q) {
+__global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __grid_constant__ NdParams Q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const SamplerParams &P = Q.base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -137,7 +142,28 @@ __global__ void __launch_bounds__(kThreads, 4) nd_kernel(const __grid_constant__
     size_t off = per_sample ? 0 : sizeof(R) * (size_t)L * kThreads;
     off = (off + 15) & ~(size_t)15;
     fx::Tables *bm_smem = reinterpret_cast<fx::Tables *>(smem_raw + off);
-    if constexpr (sizeof(R) == 8) fx::tables_load(bm_smem, tid, kThreads);
+    if constexpr (sizeof(R) == 8) {
+        fx::tables_load(bm_smem, tid, kThreads);
+        off += sizeof(fx::Tables);
+    }
+    const uint32_t *words = Q.words, *hwords = Q.hwords;
+    const float2 *pairs = sizeof(R) == 8 ? Q.tail : reinterpret_cast<const float2 *>(P.tables);
+    const double *hcoef = Q.hcoef;
+    if (Q.staged) {
+        auto stage = [&](auto *&src, int n) {
+            using T = typename std::remove_const<typename std::remove_pointer<typename std::remove_reference<decltype(src)>::type>::type>::type;
+            T *dst = reinterpret_cast<T *>(smem_raw + off);
+            for (int i = tid; i < n; i += kThreads) dst[i] = src[i];
+            src = dst;
+            off = (off + sizeof(T) * (size_t)n + 15) & ~(size_t)15;
+        };
+        stage(words, Q.n_words);
+        stage(pairs, S * P.M);
+        if constexpr (sizeof(R) == 8) {
+            stage(hcoef, Q.n_hcoef);
+            stage(hwords, Q.n_hwords);
+        }
+    }
     __syncthreads();
 
     Stream<R> st;
@@ -152,7 +178,7 @@ __global__ void __launch_bounds__(kThreads, 4) nd_kernel(const __grid_constant__
     R *q = reinterpret_cast<R *>(Q.paths) + (int64_t)blockIdx.x * kThreads + tid;
     auto co = [&](int i, int c) -> R & { return q[((int64_t)i * D + c) * ps]; };
     R seg[((1 << kNdSeg) + 1) * D];
-    constexpr int kB = sizeof(R) == 8 ? 2 : 8;   // slices per pass of the program
+    constexpr int kBP = D == 4 ? 2 : 4;          // pairs of slices per pass of the single-precision program
 
     for (int64_t item = P.item0 + blockIdx.x; item < P.n_items; item += gridDim.x) {
         const int64_t b = item / P.items_per_block;
@@ -188,59 +214,93 @@ __global__ void __launch_bounds__(kThreads, 4) nd_kernel(const __grid_constant__
                     return pick4(zc, g + 1);
                 }
             };
-            // coarse levels n = 1..S-F: midpoint i at segment endpoint (2i+1) 2^(S-F-n)
-            for (int c = 0; c < D; ++c) {
-                co(0, c) = Q.a[c];
-                co(C, c) = Q.b[c];
-            }
-            for (int n = 1; n <= Cn; ++n) {
-                const R sg = (R)P.sigma[n];
-                const int h = 1 << (Cn - n), j0 = (1 << (n - 1)) - 1;
-                for (int i = 0; i < (1 << (n - 1)); ++i) {
-                    const int idx = (2 * i + 1) * h;
-                    for (int c = 0; c < D; ++c)
-                        co(idx, c) = fma(sg, normal((uint32_t)((j0 + i) * D + c)), (R)0.5 * (co(idx - h, c) + co(idx + h, c)));
-                }
-            }
-            // w_n = -eps_n sum_k W on the level-n subpath (level n = S - dl),
-            // slices in ascending order, kB at a time (fewer on a level of two or four)
             R wloc[SU_MAX_S];
-            for (int dl = 0; dl < L; ++dl) wloc[dl] = 0;
-            auto slices = [&](const R *tab, auto &&pt, int stp, int ns, R &w) {
-                if (ns < kB) {
-                    if constexpr (kB > 4) {
-                        if (ns == 4) {
-                            nd_block<R, D, 4>(tab, Q, pt, 0, stp, w);
-                            return;
+            // pass 0 with the split levels; again with every level in double
+            // for a path that leaves the split's reach
+            for (int pass = 0; pass < 2; ++pass) {
+                bool far = false;
+                auto seen = [&](R v, int c) {
+                    if constexpr (sizeof(R) == 8) {
+                        const int hi = __double2hiint(v) & 0x7fffffff;
+                        far |= hi > __double2hiint(Q.reach[c]);
+                    }
+                    return v;
+                };
+                // coarse levels n = 1..S-F: midpoint i at segment endpoint (2i+1) 2^(S-F-n)
+                have = 0xffffffffu;
+                for (int c = 0; c < D; ++c) {
+                    co(0, c) = Q.a[c];
+                    co(C, c) = Q.b[c];
+                }
+                for (int n = 1; n <= Cn; ++n) {
+                    const R sg = (R)P.sigma[n];
+                    const int h = 1 << (Cn - n), j0 = (1 << (n - 1)) - 1;
+                    for (int i = 0; i < (1 << (n - 1)); ++i) {
+                        const int idx = (2 * i + 1) * h;
+                        for (int c = 0; c < D; ++c)
+                            co(idx, c) = seen(fma(sg, normal((uint32_t)((j0 + i) * D + c)), (R)0.5 * (co(idx - h, c) + co(idx + h, c))), c);
+                    }
+                }
+                // w_n = -eps_n sum_k W on the level-n subpath (level n = S - dl),
+                // slices in ascending order, several at a time
+                for (int dl = 0; dl < L; ++dl) wloc[dl] = 0;
+                auto slices = [&](int dl, auto &&pt, int stp, int ns) {
+                    R w = 0;
+                    if constexpr (sizeof(R) == 4) {
+                        const float2 *c = pairs + (size_t)dl * P.M;
+                        if (ns >= 2 * kBP) {
+#pragma unroll 1
+                            for (int k = 0; k < ns; k += 2 * kBP) w += nd_single<R, D, kBP>(Q, words, c, pt, k, stp);
+                        } else {
+#pragma unroll 1
+                            for (int k = 0; k < ns; k += 2) w += nd_single<R, D, 1>(Q, words, c, pt, k, stp);
+                        }
+                    } else if (pass == 0 && Q.heads[dl] > 0) {
+                        const float2 *c = pairs + (size_t)dl * P.M;
+                        float tail = 0;
+                        if (ns >= 2 * kBP) {
+#pragma unroll 1
+                            for (int k = 0; k < ns; k += 2 * kBP) tail += nd_single<R, D, kBP>(Q, words, c, pt, k, stp);
+                        } else {
+#pragma unroll 1
+                            for (int k = 0; k < ns; k += 2) tail += nd_single<R, D, 1>(Q, words, c, pt, k, stp);
+                        }
+#pragma unroll 1
+                        for (int k = 0; k < ns; k += 2)
+                            w += nd_double<D>(Q, Q.hsq[dl], hwords + Q.hw[dl], hcoef + Q.hc[dl], pt, k, stp);
+                        w += (double)tail;
+                    } else {
+#pragma unroll 1
+                        for (int k = 0; k < ns; k += 2)
+                            w += nd_double<D>(Q, Q.sq, words, reinterpret_cast<const double *>(P.tables) + (size_t)dl * P.M, pt, k, stp);
+                    }
+                    wloc[dl] += w;
+                };
+#pragma unroll 1
+                for (int dl = F; dl < L; ++dl)   // coarse levels: between segment endpoints
+                    slices(dl, co, 1 << (dl - F), 1 << (S - dl));
+                // fine levels n = S-F+1..S, one segment at a time
+                auto fp = [&](int i, int c) -> R & { return seg[i * D + c]; };
+#pragma unroll 1
+                for (int sgi = 0; sgi < C; ++sgi) {
+                    for (int c = 0; c < D; ++c) {
+                        fp(0, c) = co(sgi, c);
+                        fp(NF, c) = co(sgi + 1, c);
+                    }
+                    for (int n = Cn + 1; n <= S; ++n) {
+                        const R sg = (R)P.sigma[n];
+                        const int h = 1 << (S - n), m = 1 << (n - Cn - 1);
+                        const int j0 = (1 << (n - 1)) - 1 + sgi * m;
+                        for (int il = 0; il < m; ++il) {
+                            const int idx = (2 * il + 1) * h;
+                            for (int c = 0; c < D; ++c)
+                                fp(idx, c) = seen(fma(sg, normal((uint32_t)((j0 + il) * D + c)), (R)0.5 * (fp(idx - h, c) + fp(idx + h, c))), c);
                         }
                     }
-                    nd_block<R, D, 2>(tab, Q, pt, 0, stp, w);
-                    return;
+#pragma unroll 1
+                    for (int dl = 0; dl < min(F, L); ++dl) slices(dl, fp, 1 << dl, NF >> dl);
                 }
-                for (int k = 0; k < ns; k += kB) nd_block<R, D, kB>(tab, Q, pt, k, stp, w);
-            };
-            const R *tabs = reinterpret_cast<const R *>(P.tables);
-            for (int dl = F; dl < L; ++dl)   // coarse levels: between segment endpoints
-                slices(tabs + (size_t)dl * P.M, co, 1 << (dl - F), 1 << (S - dl), wloc[dl]);
-            // fine levels n = S-F+1..S, one segment at a time
-            auto fp = [&](int i, int c) -> R & { return seg[i * D + c]; };
-            for (int sgi = 0; sgi < C; ++sgi) {
-                for (int c = 0; c < D; ++c) {
-                    fp(0, c) = co(sgi, c);
-                    fp(NF, c) = co(sgi + 1, c);
-                }
-                for (int n = Cn + 1; n <= S; ++n) {
-                    const R sg = (R)P.sigma[n];
-                    const int h = 1 << (S - n), m = 1 << (n - Cn - 1);
-                    const int j0 = (1 << (n - 1)) - 1 + sgi * m;
-                    for (int il = 0; il < m; ++il) {
-                        const int idx = (2 * il + 1) * h;
-                        for (int c = 0; c < D; ++c)
-                            fp(idx, c) = fma(sg, normal((uint32_t)((j0 + il) * D + c)), (R)0.5 * (fp(idx - h, c) + fp(idx + h, c)));
-                    }
-                }
-                for (int dl = 0; dl < min(F, L); ++dl)
-                    slices(tabs + (size_t)dl * P.M, fp, 1 << dl, NF >> dl, wloc[dl]);
+                if (!far) break;
             }
             bool bad = false;
             for (int dl = 0; dl < L; ++dl) bad |= isnan(wloc[dl]) || (isinf(wloc[dl]) && wloc[dl] > 0);
@@ -277,9 +337,18 @@ const void *nd_fn(int D, int precision) {
 
 size_t nd_smem_bytes(const NdParams &Q, int precision) {
     const size_t rs = precision == SU_FP32 ? sizeof(float) : sizeof(double);
-    size_t off = Q.base.w_out ? 0 : rs * (size_t)Q.base.levels * kThreads;
-    off = (off + 15) & ~(size_t)15;
-    return off + (precision == SU_FP32 ? 0 : sizeof(fx::Tables));
+    auto up = [](size_t x) { return (x + 15) & ~(size_t)15; };
+    size_t off = up(Q.base.w_out ? 0 : rs * (size_t)Q.base.levels * kThreads);
+    if (precision != SU_FP32) off += sizeof(fx::Tables);
+    if (Q.staged) {
+        off = up(off + sizeof(uint32_t) * (size_t)Q.n_words);
+        off = up(off + sizeof(float2) * (size_t)Q.base.S * Q.base.M);
+        if (precision != SU_FP32) {
+            off = up(off + sizeof(double) * (size_t)Q.n_hcoef);
+            off = up(off + sizeof(uint32_t) * (size_t)Q.n_hwords);
+        }
+    }
+    return off;
 }
 
 int nd_occupancy(const NdParams &Q, int precision, size_t smem) {

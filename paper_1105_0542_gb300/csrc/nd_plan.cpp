@@ -1,0 +1,163 @@
+// The evaluation program of a several-coordinates plan and, for double
+// precision, its split into a double and a single-precision part (host).
+//
+// Program.  W is evaluated by nested Horner: the 2d variables in a fixed order
+// z_0..z_{2d-1}, a polynomial in z_k whose coefficients are polynomials in
+// z_{k+1}, and so on.  One word per polynomial, depth first, highest power
+// first: its number of coefficients (zero: the zero polynomial) and whether it
+// has a factor z_k; where the powers of a depth keep their parity inside every
+// polynomial (W of an even potential) the Horner variable of that depth is
+// z_k^2.  The innermost coefficients are the table's entries in program order.
+// Every variable sits at a known depth of a nest of loops, so its registers are
+// named in the code: no entry is looked up by symbol and no partial product is
+// stored.
+//
+// Split (double).  Entries whose root mean square over the bridge is small are
+// left to single precision: what rounding them to floats costs, 2^-25 of their
+// sum, adds up over the N slices and stays below 2^-55 of the level's weight.
+// The others form a program of their own, evaluated in double.  A path that
+// leaves max(|a|, |b|) + 2.4 sqrt(T) in a coordinate (probability 2e-5) is
+// weighed by the whole program in double.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <set>
+
+#include "sampler.h"
+
+namespace su {
+
+namespace {
+
+using Mono = std::vector<unsigned char>;
+
+struct Item {
+    const unsigned char *e;   // exponents in program order
+    int entry;
+};
+
+// items[lo, hi) sorted by exponents, highest first, equal before depth k
+void emit(const std::vector<Item> &it, size_t lo, size_t hi, int k, int nv, unsigned sq, NdProgram &G) {
+    if (lo == hi) {
+        G.words.push_back(0);
+        return;
+    }
+    const int top = it[lo].e[k];
+    const int step = (sq >> k) & 1 ? 2 : 1, e0 = step == 2 ? top & 1 : 0;
+    G.words.push_back((uint32_t)((top - e0) / step + 1) | (e0 ? kNdOdd : 0u));
+    size_t at = lo;
+    for (int e = top; e >= e0; e -= step) {
+        size_t end = at;
+        while (end < hi && it[end].e[k] == e) ++end;
+        if (k == nv - 1)
+            G.slot.push_back(end > at ? it[at].entry : -1);
+        else
+            emit(it, at, end, k + 1, nv, sq, G);
+        at = end;
+    }
+}
+
+}  // namespace
+
+void nd_order(const std::vector<Mono> &mono, int nv, int *order) {
+    // greedily the variable that splits the monomials into the fewest groups
+    std::vector<int> group(mono.size(), 0);
+    std::vector<bool> used((size_t)nv, false);
+    for (int k = 0; k < nv; ++k) {
+        int best = -1;
+        size_t least = 0;
+        for (int v = 0; v < nv; ++v) {
+            if (used[v]) continue;
+            std::set<std::pair<int, int>> s;
+            for (size_t i = 0; i < mono.size(); ++i) s.emplace(group[i], mono[i][v]);
+            if (best < 0 || s.size() < least) {
+                best = v;
+                least = s.size();
+            }
+        }
+        order[k] = best;
+        used[best] = true;
+        std::set<std::pair<int, int>> s;
+        for (size_t i = 0; i < mono.size(); ++i) s.emplace(group[i], mono[i][best]);
+        for (size_t i = 0; i < mono.size(); ++i)
+            group[i] = (int)std::distance(s.begin(), s.find({group[i], mono[i][best]}));
+    }
+}
+
+void nd_program(const std::vector<Mono> &mono, const std::vector<int> &pick, int nv, const int *order, NdProgram &G) {
+    std::vector<Mono> e(pick.size(), Mono((size_t)nv));
+    std::vector<Item> it;
+    for (size_t i = 0; i < pick.size(); ++i) {
+        for (int k = 0; k < nv; ++k) e[i][k] = mono[(size_t)pick[i]][(size_t)order[k]];
+        it.push_back({e[i].data(), pick[i]});
+    }
+    std::sort(it.begin(), it.end(), [&](const Item &a, const Item &b) {
+        for (int k = 0; k < nv; ++k)
+            if (a.e[k] != b.e[k]) return a.e[k] > b.e[k];
+        return false;
+    });
+    // depths whose powers keep their parity inside every polynomial
+    G.sq = 0;
+    for (int k = 0; k < nv; ++k) {
+        bool even = true;
+        for (size_t i = 1; i < it.size(); ++i) {
+            bool same = true;
+            for (int j = 0; j < k; ++j) same = same && it[i].e[j] == it[i - 1].e[j];
+            if (same && ((it[i].e[k] ^ it[i - 1].e[k]) & 1)) even = false;
+        }
+        if (even) G.sq |= 1u << k;
+    }
+    G.words.clear();
+    G.slot.clear();
+    emit(it, 0, it.size(), 0, nv, G.sq, G);
+}
+
+// root mean squares of x_c^e (averaged over the bridge's times), e = 0..top
+static std::vector<double> moments(double a, double b, double T, int top) {
+    std::vector<double> m((size_t)top + 1, 0.0);
+    for (int k = 1; k < 16; ++k) {
+        const double u = k / 16.0, mean = a + (b - a) * u, sd = std::sqrt(T * u * (1 - u));
+        for (int g = -24; g <= 24; ++g) {
+            const double x = mean + sd * g * 0.25;
+            double w = std::exp(-0.5 * g * g * 0.0625) * (0.25 / std::sqrt(2 * 3.14159265358979323846)) / 15;
+            for (int e = 0; e <= top; ++e, w *= x * x) m[(size_t)e] += w;
+        }
+    }
+    for (double &v : m) v = std::sqrt(v);
+    return m;
+}
+
+void nd_split(const std::vector<Mono> &mono, int D, const double *a, const double *b, double T, int n,
+              const std::vector<double> &table, std::vector<int> &heads) {
+    const double N = std::ldexp(1.0, n), eps = T / N;
+    std::vector<std::vector<double>> mx((size_t)D), mb((size_t)D);
+    for (int c = 0; c < D; ++c) {
+        int tx = 0, tb = 0;
+        for (const Mono &m : mono) {
+            tx = std::max(tx, (int)m[(size_t)c]);
+            tb = std::max(tb, (int)m[(size_t)(D + c)]);
+        }
+        mx[c] = moments(a[c], b[c], T, tx);
+        const double s2 = 0.25 * (eps + (b[c] - a[c]) * (b[c] - a[c]) / (N * N));
+        mb[c].assign((size_t)tb + 1, 1.0);
+        for (int f = 1; f <= tb; ++f) mb[c][f] = mb[c][f - 1] * std::sqrt(s2 * (2.0 * f - 1));   // E g^2f = (2f - 1)!!
+    }
+    std::vector<std::pair<double, int>> r;
+    double all = 0;
+    for (size_t i = 0; i < mono.size(); ++i) {
+        double v = std::fabs(table[i]);
+        for (int c = 0; c < D; ++c) v *= mx[c][mono[i][(size_t)c]] * mb[c][mono[i][(size_t)(D + c)]];
+        r.emplace_back(v, (int)i);
+        all += v;
+    }
+    std::sort(r.begin(), r.end());
+    // N 2^-25 rest <= 2^-55 min(1, N all)
+    const double most = 0x1p-30 * std::min(1.0, N * all) / N;
+    double rest = 0;
+    heads.clear();
+    size_t k = 0;
+    for (; k < r.size() && rest + r[k].first <= most; ++k) rest += r[k].first;
+    for (; k < r.size(); ++k) heads.push_back(r[k].second);
+}
+
+}  // namespace su

@@ -179,15 +179,43 @@ cudaError_t launch_vectors(int B, const double *X, int n, int nev, double scale,
 // thread, every coordinate an exact Brownian bridge (coordinate c of heap
 // midpoint j takes normal j D + c of the sample's stream), built and weighed
 // in segments of 2^kNdSeg slices (segment endpoints in a global scratch, one
-// segment's points in local memory); W(x, xb; eps) per slice from the monomial program of
-// NdEffective (nodes as GeneralNode; entries = powers of z_H), several
-// slices at a time (two in double, eight in single precision); weights and
-// per-item tuples as the one-dimensional sampler's.
+// segment's points in local memory); W(x, xb; eps) per slice by nested Horner
+// (nd_plan.cpp), several slices at a time; weights and per-item tuples as the
+// one-dimensional sampler's.
 constexpr int kNdSeg = 5;     // the several-coordinates path in segments of 2^5 slices
+constexpr uint32_t kNdOdd = 1u << 16;   // program word: the polynomial has a factor z_k
+// The nested-Horner program of a set of monomials (nd_plan.cpp).
+struct NdProgram {
+    std::vector<uint32_t> words;
+    std::vector<int> slot;    // table entry of each coefficient in program order, -1: zero
+    unsigned sq = 0;          // depths whose Horner variable is z_k^2
+};
+// the order of the variables for these monomials (nv exponents each)
+void nd_order(const std::vector<std::vector<unsigned char>> &mono, int nv, int *order);
+void nd_program(const std::vector<std::vector<unsigned char>> &mono, const std::vector<int> &pick, int nv,
+                const int *order, NdProgram &G);
+// the entries of a level's table that need double precision
+void nd_split(const std::vector<std::vector<unsigned char>> &mono, int D, const double *a, const double *b, double T,
+              int n, const std::vector<double> &table, std::vector<int> &heads);
+
 struct NdParams {
-    SamplerParams base;       // S, levels, tables (per level, global), M, sigma, stream, items, outputs
-    int D, H, G, n_nodes;     // Horner in z_H^G
-    const GeneralNode *nodes; // device
+    SamplerParams base;       // S, levels, M = coefficients of the program per level, sigma, stream, items, outputs
+    int D;
+    int order[2 * kNdMaxDim]; // variable of each depth: x_c = c, xb_c = D + c
+    unsigned sq;              // depths whose Horner variable is z_k^2
+    int n_words;
+    const uint32_t *words;    // device: the program
+    // base.tables: [S][M], pairs {c, c} in single precision
+    // double precision: the single-precision part's pairs [S][M], and per level the program and entries of
+    // the double part (heads = 0: the whole program in double)
+    const float2 *tail;
+    const uint32_t *hwords;   // all levels' words
+    const double *hcoef;
+    int n_hwords, n_hcoef;
+    int heads[SU_MAX_S], hw[SU_MAX_S], hc[SU_MAX_S];   // row d: its double entries, first word, first coefficient
+    unsigned hsq[SU_MAX_S];
+    double reach[kNdMaxDim];  // |q_c| beyond which the path is weighed in double
+    int staged;               // program and tables in shared memory
     double a[kNdMaxDim], b[kNdMaxDim];
     void *paths;              // device (double or float): segment endpoint i, coordinate c of slot t
                               // at [(i D + c) pstride + t]
