@@ -677,54 +677,102 @@ void general_wp_points(const GeneralEffective &G, const GeneralPotential &V, dou
 namespace {
 
 using NM = std::array<unsigned char, 2 * kNdMaxDim>;   // exponents of x_1..x_d, xb_1..xb_d
-using NPoly = std::map<NM, DD>;
+// A polynomial: monomials in lexicographic order as 64-bit keys (exponents as
+// bytes, the first variable's the highest: keys add where monomials multiply).
+// (As std::map<NM, DD> the recursion of a three-dimensional quartic at p = 8
+// took 9 ms of a 25 ms call.)
+using NKey = uint64_t;
+using NPoly = std::vector<std::pair<NKey, DD>>;
+
+NKey nkey(const NM &m) {
+    NKey k = 0;
+    for (size_t j = 0; j < 8; ++j) k = (k << 8) | (j < m.size() ? m[j] : 0u);
+    return k;
+}
+NM nmono(NKey k) {
+    NM m{};
+    for (size_t j = 0; j < m.size(); ++j) m[j] = (unsigned char)(k >> (8 * (7 - j)));
+    return m;
+}
+NKey nvar(int i) { return (NKey)1 << (8 * (7 - i)); }
+int nexp(NKey k, int i) { return (int)((k >> (8 * (7 - i))) & 255u); }
+static_assert(2 * kNdMaxDim <= 8, "a monomial's exponents in one 64-bit key");
+
+// x += v; false where the sum cancels to rounding residue
+bool nsum(DD &x, DD v) {
+    const double scale = std::max(std::fabs(x.hi), std::fabs(v.hi));
+    x = add(x, v);
+    return std::fabs(x.hi) > 1e-26 * scale;
+}
 
 // acc += s * b, dropping sums that cancel to rounding residue
 void nadd(NPoly &acc, const NPoly &b, DD s) {
+    NPoly out;
+    out.reserve(acc.size() + b.size());
+    size_t i = 0;
     for (const auto &kv : b) {
+        while (i < acc.size() && acc[i].first < kv.first) out.push_back(acc[i++]);
         const DD v = mul(kv.second, s);
-        auto it = acc.find(kv.first);
-        if (it == acc.end()) {
-            acc.emplace(kv.first, v);
+        if (i < acc.size() && acc[i].first == kv.first) {
+            DD x = acc[i++].second;
+            if (nsum(x, v)) out.emplace_back(kv.first, x);
         } else {
-            const double scale = std::max(std::fabs(it->second.hi), std::fabs(v.hi));
-            it->second = add(it->second, v);
-            if (std::fabs(it->second.hi) <= 1e-26 * scale) acc.erase(it);
+            out.emplace_back(kv.first, v);
         }
     }
+    out.insert(out.end(), acc.begin() + (long)i, acc.end());
+    acc.swap(out);
 }
 
-void nadd_term(NPoly &acc, const NM &m, DD v) {
-    auto it = acc.find(m);
-    if (it == acc.end()) {
-        acc.emplace(m, v);
-    } else {
-        const double scale = std::max(std::fabs(it->second.hi), std::fabs(v.hi));
-        it->second = add(it->second, v);
-        if (std::fabs(it->second.hi) <= 1e-26 * scale) acc.erase(it);
-    }
-}
-
+// the product, its terms summed in the order of a, then b
 NPoly nmul(const NPoly &a, const NPoly &b) {
-    NPoly out;
+    struct Slot {
+        NKey key;
+        DD v;
+        int state;   // 0 free, 1 a term, 2 a term that has cancelled
+    };
+    size_t cap = 64;
+    while (cap < 2 * std::min(a.size() * b.size(), (size_t)1 << 20)) cap *= 2;
+    std::vector<Slot> h(cap, Slot{0, dd(0), 0});
+    size_t used = 0;
+    auto at = [&](std::vector<Slot> &t, NKey k) -> Slot & {
+        size_t i = (size_t)((k * 0x9E3779B97F4A7C15ULL) >> 20) & (t.size() - 1);
+        while (t[i].state && t[i].key != k) i = (i + 1) & (t.size() - 1);
+        return t[i];
+    };
     for (const auto &x : a)
         for (const auto &y : b) {
-            NM m;
-            for (size_t j = 0; j < m.size(); ++j) m[j] = (unsigned char)(x.first[j] + y.first[j]);
-            nadd_term(out, m, mul(x.second, y.second));
+            const NKey k = x.first + y.first;
+            const DD v = mul(x.second, y.second);
+            Slot &s = at(h, k);
+            if (s.state == 1) {
+                if (!nsum(s.v, v)) s.state = 2;
+                continue;
+            }
+            if (s.state == 0 && 2 * ++used > h.size()) {
+                std::vector<Slot> g(2 * h.size(), Slot{0, dd(0), 0});
+                for (const Slot &o : h)
+                    if (o.state) at(g, o.key) = o;
+                h.swap(g);
+                at(h, k) = Slot{k, v, 1};
+                continue;
+            }
+            s = Slot{k, v, 1};
         }
+    NPoly out;
+    out.reserve(used);
+    for (const Slot &s : h)
+        if (s.state == 1) out.emplace_back(s.key, s.v);
+    std::sort(out.begin(), out.end(), [](const auto &p, const auto &q) { return p.first < q.first; });
     return out;
 }
 
-// d/dz_i
+// d/dz_i (the order of the monomials stays)
 NPoly nder(const NPoly &a, int i) {
     NPoly out;
-    for (const auto &x : a) {
-        if (!x.first[(size_t)i]) continue;
-        NM m = x.first;
-        m[(size_t)i] -= 1;
-        nadd_term(out, m, mul_d(x.second, (double)x.first[(size_t)i]));
-    }
+    out.reserve(a.size());
+    for (const auto &x : a)
+        if (const int e = nexp(x.first, i)) out.emplace_back(x.first - nvar(i), mul_d(x.second, (double)e));
     return out;
 }
 
@@ -764,7 +812,7 @@ int build_nd(int d, const int *exps, const double *coefs, int n_terms, int p, Nd
             err = "non-finite potential coefficient";
             return SU_EINVAL;
         }
-        if (coefs[t] != 0.0) nadd_term(V, m, dd(coefs[t]));
+        if (coefs[t] != 0.0) nadd(V, NPoly{{nkey(m), dd(coefs[t])}}, dd(1.0));
     }
     // W[m][k] and its gradients in x and in xb
     std::vector<std::vector<NPoly>> W((size_t)p, std::vector<NPoly>((size_t)p));
@@ -789,11 +837,8 @@ int build_nd(int d, const int *exps, const double *coefs, int n_terms, int p, Nd
                 NPoly nxt;
                 for (int i = 0; i < d; ++i) {
                     NPoly t = nder(diag, i);
-                    for (const auto &x : t) {
-                        NM mm = x.first;
-                        mm[(size_t)(d + i)] += 1;
-                        nadd_term(nxt, mm, x.second);
-                    }
+                    for (auto &x : t) x.first += nvar(d + i);
+                    nadd(nxt, t, dd(1.0));
                 }
                 diag = std::move(nxt);
             }
@@ -823,7 +868,7 @@ int build_nd(int d, const int *exps, const double *coefs, int n_terms, int p, Nd
     for (int m = 0; m < p; ++m)
         for (int k = 0; k <= m; ++k)
             for (const auto &kv : W[(size_t)m][(size_t)k]) {
-                auto &v = terms[kv.first];
+                auto &v = terms[nmono(kv.first)];
                 if (v.empty()) v.assign((size_t)p, dd(0));
                 v[(size_t)(m - k)] = add(v[(size_t)(m - k)], kv.second);
             }
@@ -876,16 +921,21 @@ int build_nd(int d, const int *exps, const double *coefs, int n_terms, int p, Nd
     for (int H = 0; H < nv; ++H) {
         int G = 1;
         const auto grp = spans_of(H, G);
-        std::map<std::vector<int>, int> trie;   // every prefix of every group's prefix
-        size_t entries = 0;
+        std::vector<std::vector<int>> seqs;
+        size_t entries = 0, nodes = 1;   // nodes: the distinct prefixes of the sequences, the empty one first
         for (const auto &g : grp) {
             entries += (size_t)((g.second.hi - g.second.lo) / G + 1);
-            const std::vector<int> seq = seq_of(g.first, H, g.second.lo);
-            for (size_t len = 0; len <= seq.size(); ++len)
-                trie.emplace(std::vector<int>(seq.begin(), seq.begin() + (long)len), 0);
+            seqs.push_back(seq_of(g.first, H, g.second.lo));
         }
-        if (trie.size() + entries < best) {
-            best = trie.size() + entries;
+        std::sort(seqs.begin(), seqs.end());
+        for (size_t i = 0; i < seqs.size(); ++i) {
+            size_t same = 0;
+            if (i)
+                while (same < seqs[i].size() && same < seqs[i - 1].size() && seqs[i][same] == seqs[i - 1][same]) ++same;
+            nodes += seqs[i].size() - same;
+        }
+        if (nodes + entries < best) {
+            best = nodes + entries;
             bestH = H;
             bestG = G;
         }

@@ -21,7 +21,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <set>
 
 #include "sampler.h"
 
@@ -61,26 +60,31 @@ void emit(const std::vector<Item> &it, size_t lo, size_t hi, int k, int nv, unsi
 
 void nd_order(const std::vector<Mono> &mono, int nv, int *order) {
     // greedily the variable that splits the monomials into the fewest groups
-    std::vector<int> group(mono.size(), 0);
+    std::vector<int> group(mono.size(), 0), key(mono.size()), uniq;
     std::vector<bool> used((size_t)nv, false);
+    auto split = [&](int v) {
+        for (size_t i = 0; i < mono.size(); ++i) key[i] = group[i] * 256 + mono[i][(size_t)v];
+        uniq = key;
+        std::sort(uniq.begin(), uniq.end());
+        uniq.erase(std::unique(uniq.begin(), uniq.end()), uniq.end());
+        return uniq.size();
+    };
     for (int k = 0; k < nv; ++k) {
         int best = -1;
         size_t least = 0;
         for (int v = 0; v < nv; ++v) {
-            if (used[v]) continue;
-            std::set<std::pair<int, int>> s;
-            for (size_t i = 0; i < mono.size(); ++i) s.emplace(group[i], mono[i][v]);
-            if (best < 0 || s.size() < least) {
+            if (used[(size_t)v]) continue;
+            const size_t n = split(v);
+            if (best < 0 || n < least) {
                 best = v;
-                least = s.size();
+                least = n;
             }
         }
         order[k] = best;
-        used[best] = true;
-        std::set<std::pair<int, int>> s;
-        for (size_t i = 0; i < mono.size(); ++i) s.emplace(group[i], mono[i][best]);
+        used[(size_t)best] = true;
+        split(best);
         for (size_t i = 0; i < mono.size(); ++i)
-            group[i] = (int)std::distance(s.begin(), s.find({group[i], mono[i][best]}));
+            group[i] = (int)(std::lower_bound(uniq.begin(), uniq.end(), key[i]) - uniq.begin());
     }
 }
 
