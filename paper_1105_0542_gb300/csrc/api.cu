@@ -106,11 +106,61 @@ cudaError_t dmalloc(void **p, size_t bytes) {
     return cudaMalloc(p, bytes);
 }
 
+// The memory pool of the calls' own scratch, one per device and context: it
+// keeps up to 32 MB between calls, where the device's default pool (left as it
+// is, it may be shared) hands every byte back at the next synchronisation,
+// 90 us to unmap and map again per call.  The context is told by its id, so that a
+// pool of a context that was torn down is never used.  Null where the driver
+// cannot say: the default pool then.
+cudaMemPool_t call_pool() {
+    using GetCurrent = int (*)(void **);
+    using GetId = int (*)(void *, unsigned long long *);
+    static std::mutex mu;
+    static GetCurrent get_current = nullptr;
+    static GetId get_id = nullptr;
+    static bool asked = false;
+    static std::map<std::pair<int, unsigned long long>, cudaMemPool_t> pools;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!asked) {
+        asked = true;
+        void *f = nullptr, *g = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess &&
+            cudaGetDriverEntryPointByVersion("cuCtxGetId", &g, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess) {
+            get_current = reinterpret_cast<GetCurrent>(f);
+            get_id = reinterpret_cast<GetId>(g);
+        }
+        cudaGetLastError();
+    }
+    void *ctx = nullptr;
+    unsigned long long id = 0;
+    int dev = 0;
+    if (!get_id || cudaGetDevice(&dev) != cudaSuccess || get_current(&ctx) || !ctx || get_id(ctx, &id)) return nullptr;
+    auto it = pools.find({dev, id});
+    if (it != pools.end()) return it->second;
+    cudaMemPool_t pool = nullptr;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    uint64_t keep = (uint64_t)32 << 20;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        pool = nullptr;
+    }
+    pools.emplace(std::make_pair(dev, id), pool);
+    return pool;
+}
+
 cudaError_t dmalloc_async(void **p, size_t bytes, cudaStream_t st) {
     if (take_alloc_fault()) {
         *p = nullptr;
         return cudaErrorMemoryAllocation;
     }
+    if (cudaMemPool_t pool = call_pool()) return cudaMallocFromPoolAsync(p, bytes, pool, st);
     return cudaMallocAsync(p, bytes, st);
 }
 
@@ -153,6 +203,7 @@ struct su_plan {
     int64_t n_blocks = 1;
     su::SamplerParams P{};
     void *d_tables = nullptr;
+    bool tables_async = false;   // d_tables is stream-ordered on opt.stream (a plan inside one call)
     int device = 0;
     int grid = 0;
     size_t smem = 0;
@@ -342,6 +393,30 @@ static int general_image(const su::GeneralEffective &G, const su::GeneralPotenti
 
 static int upload_general(su_plan &pl) { return general_image(*pl.G, pl.V, &pl.d_general); }
 
+// The plan's device block of tables: stream-ordered for a plan that lives
+// inside one call, else allocated and uploaded when the plan is made.
+static int upload_tables(su_plan &pl, const std::vector<unsigned char> &blob) {
+    if (pl.tables_async) {
+        cudaStream_t st = (cudaStream_t)pl.opt.stream;
+        CU(dmalloc_async(&pl.d_tables, blob.size(), st), "device allocation (tables)");
+        CU(cudaMemcpyAsync(pl.d_tables, blob.data(), blob.size(), cudaMemcpyHostToDevice, st), "upload tables");
+        return SU_OK;
+    }
+    CU(dmalloc(&pl.d_tables, blob.size()), "device allocation (tables)");
+    CU(cudaMemcpy(pl.d_tables, blob.data(), blob.size(), cudaMemcpyHostToDevice), "upload tables");
+    return SU_OK;
+}
+
+static void free_tables(su_plan &pl) {
+    if (pl.d_tables && pl.tables_async)
+        cudaFreeAsync(pl.d_tables, (cudaStream_t)pl.opt.stream);
+    else if (pl.d_tables)
+        cudaFree(pl.d_tables);
+    pl.d_tables = nullptr;
+    if (pl.d_general) cudaFree(pl.d_general);
+    pl.d_general = nullptr;
+}
+
 // The level tables of a plan (rows d = 0..S-1 for levels n = S..1), each
 // scaled for the kernel and rounded to its precision: host work only.
 static int plan_tables(su_plan &pl, std::vector<unsigned char> &blob) {
@@ -504,8 +579,8 @@ static int configure(su_plan &pl) {
     if (rc) return rc;
     rc = plan_shape(pl, sms, smem_max, blob);
     if (rc) return rc;
-    CU(dmalloc(&pl.d_tables, blob.size()), "device allocation (tables)");
-    CU(cudaMemcpy(pl.d_tables, blob.data(), blob.size(), cudaMemcpyHostToDevice), "upload tables");
+    rc = upload_tables(pl, blob);
+    if (rc) return rc;
     if (pl.model == SU_GENERAL) {
         rc = upload_general(pl);
         if (rc) return rc;
@@ -549,8 +624,10 @@ static int plan_init(su_plan &pl, int model, const double *params, int n_params,
     return SU_OK;
 }
 
-int su_plan_create(int model, const double *params, int n_params, double a, double b, double T,
-                   int p, int s, int64_t n_mc, uint64_t seed, const su_options *opt, su_plan **out) {
+// in_call: the plan's device block is ordered on the options' stream, and so
+// are all uses of it and its release (a plan inside one entry point).
+static int plan_create(int model, const double *params, int n_params, double a, double b, double T, int p, int s,
+                       int64_t n_mc, uint64_t seed, const su_options *opt, su_plan **out, bool in_call) {
     if (!out) return fail(SU_EINVAL, "plan pointer missing");
     *out = nullptr;
     su_options o;
@@ -560,14 +637,19 @@ int su_plan_create(int model, const double *params, int n_params, double a, doub
     if (!pl) return fail(SU_ENOMEM, "host allocation failed");
     int rc = plan_init(*pl, model, params, n_params, a, b, T, p, s, n_mc, seed, o);
     if (rc) return rc;
+    pl->tables_async = in_call;
     rc = configure(*pl);
     if (rc) {
-        if (pl->d_tables) cudaFree(pl->d_tables);
-        if (pl->d_general) cudaFree(pl->d_general);
+        free_tables(*pl);
         return rc;
     }
     *out = pl.release();
     return SU_OK;
+}
+
+int su_plan_create(int model, const double *params, int n_params, double a, double b, double T,
+                   int p, int s, int64_t n_mc, uint64_t seed, const su_options *opt, su_plan **out) {
+    return plan_create(model, params, n_params, a, b, T, p, s, n_mc, seed, opt, out, false);
 }
 
 // Tables, program and launch shape of a system of several coordinates.
@@ -654,8 +736,8 @@ static int configure_nd(su_plan &pl) {
     const size_t o_hc = put(hcoef.data(), hcoef.size() * sizeof(double));
     const size_t o_hw = put(hwords.data(), hwords.size() * sizeof(uint32_t));
     const size_t o_w = put(G.words.data(), G.words.size() * sizeof(uint32_t));
-    CU(dmalloc(&pl.d_tables, blob.size()), "device allocation (tables)");
-    CU(cudaMemcpy(pl.d_tables, blob.data(), blob.size(), cudaMemcpyHostToDevice), "upload tables");
+    rc = upload_tables(pl, blob);
+    if (rc) return rc;
     unsigned char *dev = static_cast<unsigned char *>(pl.d_tables);
 
     SamplerParams &P = pl.P;
@@ -710,8 +792,9 @@ static int configure_nd(su_plan &pl) {
     return SU_OK;
 }
 
-int su_plan_create_nd(int d, const int *exps, const double *coefs, int n_terms, const double *a, const double *b,
-                      double T, int p, int s, int64_t n_mc, uint64_t seed, const su_options *opt, su_plan **out) {
+static int plan_create_nd(int d, const int *exps, const double *coefs, int n_terms, const double *a, const double *b,
+                          double T, int p, int s, int64_t n_mc, uint64_t seed, const su_options *opt, su_plan **out,
+                          bool in_call) {
     if (!out) return fail(SU_EINVAL, "plan pointer missing");
     *out = nullptr;
     if (d < 1 || d > su::kNdMaxDim) return fail(SU_EINVAL, "d must be in 1..%d", su::kNdMaxDim);
@@ -755,20 +838,24 @@ int su_plan_create_nd(int d, const int *exps, const double *coefs, int n_terms, 
     pl->w0 = -T * su::nd_wp_host(pl->N, xm, xh, T);
     if (!std::isfinite(pl->w0) && !(std::isinf(pl->w0) && pl->w0 < 0))
         return fail(SU_ENONFINITE, "level-0 weight is not finite");
+    pl->tables_async = in_call;
     rc = configure_nd(*pl);
     if (rc) {
-        if (pl->d_tables) cudaFree(pl->d_tables);
-        if (pl->d_general) cudaFree(pl->d_general);
+        free_tables(*pl);
         return rc;
     }
     *out = pl.release();
     return SU_OK;
 }
 
+int su_plan_create_nd(int d, const int *exps, const double *coefs, int n_terms, const double *a, const double *b,
+                      double T, int p, int s, int64_t n_mc, uint64_t seed, const su_options *opt, su_plan **out) {
+    return plan_create_nd(d, exps, coefs, n_terms, a, b, T, p, s, n_mc, seed, opt, out, false);
+}
+
 int su_plan_destroy(su_plan *pl) {
     if (!pl) return SU_OK;
-    if (pl->d_tables) cudaFree(pl->d_tables);
-    if (pl->d_general) cudaFree(pl->d_general);
+    free_tables(*pl);
     delete pl;
     return SU_OK;
 }
@@ -950,25 +1037,23 @@ static int amplitude_of_plan(su_plan *pl, su_level_result *out, float *ms = null
     void *dbuf = nullptr;
     const int64_t tb = pl->tuple_bytes, sb = pl->scratch_bytes;
     CU(dmalloc_async(&dbuf, (size_t)(tb + sb), st), "cudaMallocAsync");
+    // scratch, whose last 256 bytes hold the flag word, then the tuples: one copy reads both
     std::vector<double> h((size_t)(tb / sizeof(double)) + 32);
-    void *d_tup = dbuf;
-    void *d_scr = static_cast<char *>(dbuf) + tb;
+    void *d_scr = dbuf;
+    void *d_tup = static_cast<char *>(dbuf) + sb;
     int rc = ms ? su_plan_execute_timed(pl, d_tup, d_scr, st, nullptr, ms) : su_plan_execute(pl, d_tup, d_scr, st, nullptr);
     cudaError_t e = cudaSuccess;
     if (rc == SU_OK) {
-        e = cudaMemcpyAsync(h.data(), d_tup, (size_t)tb, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(h.data() + tb / sizeof(double), static_cast<char *>(d_scr) + sb - 256,
-                                sizeof(int), cudaMemcpyDeviceToHost, st);
+        e = cudaMemcpyAsync(h.data(), static_cast<char *>(d_tup) - 256, (size_t)tb + 256, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
     cudaFreeAsync(dbuf, st);
     if (rc) return rc;
     if (e != cudaSuccess) return cuda_fail(e, "sampling");
     int flags = 0;
-    std::memcpy(&flags, h.data() + tb / sizeof(double), sizeof(int));
+    std::memcpy(&flags, h.data(), sizeof(int));
     if (flags & 1) return fail(SU_ENONFINITE, "a per-sample weight was NaN or +Inf");
-    return su_plan_finalize(pl, h.data(), nullptr, out);
+    return su_plan_finalize(pl, h.data() + 32, nullptr, out);
 }
 
 int speedup_amplitude(int model, const double *params, int n_params, double a, double b, double T,
@@ -976,7 +1061,7 @@ int speedup_amplitude(int model, const double *params, int n_params, double a, d
                       su_level_result *out) {
     if (!out) return fail(SU_EINVAL, "output missing");
     su_plan *pl = nullptr;
-    int rc = su_plan_create(model, params, n_params, a, b, T, p, s, n_mc, seed, opt, &pl);
+    int rc = plan_create(model, params, n_params, a, b, T, p, s, n_mc, seed, opt, &pl, true);
     if (rc) return rc;
     std::unique_ptr<su_plan, int (*)(su_plan *)> guard(pl, su_plan_destroy);
     return amplitude_of_plan(pl, out);
@@ -987,7 +1072,7 @@ int speedup_amplitude_nd(int d, const int *exps, const double *coefs, int n_term
                          su_level_result *out) {
     if (!out) return fail(SU_EINVAL, "output missing");
     su_plan *pl = nullptr;
-    int rc = su_plan_create_nd(d, exps, coefs, n_terms, a, b, T, p, s, n_mc, seed, opt, &pl);
+    int rc = plan_create_nd(d, exps, coefs, n_terms, a, b, T, p, s, n_mc, seed, opt, &pl, true);
     if (rc) return rc;
     std::unique_ptr<su_plan, int (*)(su_plan *)> guard(pl, su_plan_destroy);
     return amplitude_of_plan(pl, out);
@@ -1006,7 +1091,7 @@ int speedup_logweights_nd(int d, const int *exps, const double *coefs, int n_ter
     o.hierarchy = 1;
     o.n_blocks = 1;
     su_plan *pl = nullptr;
-    int rc = su_plan_create_nd(d, exps, coefs, n_terms, a, b, T, p, s, n_samples, seed, &o, &pl);
+    int rc = plan_create_nd(d, exps, coefs, n_terms, a, b, T, p, s, n_samples, seed, &o, &pl, true);
     if (rc) return rc;
     std::unique_ptr<su_plan, int (*)(su_plan *)> guard(pl, su_plan_destroy);
     cudaStream_t st = (cudaStream_t)o.stream;
@@ -1480,7 +1565,7 @@ int speedup_logweights(int model, const double *params, int n_params, double a, 
     o.hierarchy = 1;
     o.n_blocks = 1;
     su_plan *pl = nullptr;
-    int rc = su_plan_create(model, params, n_params, a, b, T, p, s, n_samples, seed, &o, &pl);
+    int rc = plan_create(model, params, n_params, a, b, T, p, s, n_samples, seed, &o, &pl, true);
     if (rc) return rc;
     std::unique_ptr<su_plan, int (*)(su_plan *)> guard(pl, su_plan_destroy);
     cudaStream_t st = (cudaStream_t)o.stream;
@@ -2451,7 +2536,7 @@ extern "C" int speedup_proposal_logweights(int model, const double *params, int 
     int rc = proposal_check(o, s, pr);
     if (rc) return rc;
     su_plan *pl = nullptr;
-    rc = su_plan_create(model, params, n_params, a, b, T, p, s, n_samples, seed, &o, &pl);
+    rc = plan_create(model, params, n_params, a, b, T, p, s, n_samples, seed, &o, &pl, true);
     if (rc) return rc;
     std::unique_ptr<su_plan, int (*)(su_plan *)> guard(pl, su_plan_destroy);
     su::ProposalParams Q;

@@ -60,34 +60,40 @@ static const FixedEntry kFxFixed[kFixedGroups] = {
 namespace {
 
 // ----------------------------------------------------------- combine
-__global__ void combine_kernel(const double *__restrict__ partial, double *__restrict__ tuples, int64_t b0,
-                               int64_t n_blocks, int L, int64_t ipb) {
-    const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= n_blocks * L) return;
+// The tuple of each (block, level) from its items' tuples: one warp each, lanes
+// over the items (the largest M first, then the sums scaled to it, lanes folded
+// by butterfly: a fixed order).  Latency bound: with one thread walking the
+// items in turn (a load and a double exponential each) 79 items took 0.1 ms
+// and 2441 items 1.7 ms, a fifth of a short single-precision run.
+__global__ void __launch_bounds__(128) combine_kernel(const double *__restrict__ partial, double *__restrict__ tuples,
+                                                      int64_t b0, int64_t n_blocks, int L, int64_t ipb) {
+    const int64_t id = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+    const int lane = threadIdx.x & 31;
+    if (id >= n_blocks * L) return;   // whole warps
     const int64_t b = b0 + id / L;
     const int d = (int)(id - (id / L) * L);
+    const double *p = partial + 4 * (b * ipb * L + d);
     double M = -INFINITY, S = 0, Q = 0, n = 0;
-    for (int64_t r = 0; r < ipb; ++r) {
-        const double *p = partial + 4 * ((b * ipb + r) * L + d);
-        const double m2 = p[0];
-        n += p[3];
-        if (!(m2 > -INFINITY)) continue;
-        if (m2 > M) {
-            const double f = exp(M - m2);  // 0 when M = -inf
-            S = S * f + p[1];
-            Q = Q * f * f + p[2];
-            M = m2;
-        } else {
-            const double f = exp(m2 - M);
-            S += p[1] * f;
-            Q += p[2] * f * f;
-        }
+    for (int64_t r = lane; r < ipb; r += 32) M = fmax(M, p[4 * L * r]);
+    M = warp_max(M);
+    for (int64_t r = lane; r < ipb; r += 32) {
+        const double *t = p + 4 * L * r;
+        n += t[3];
+        if (!(t[0] > -INFINITY)) continue;
+        const double f = exp(t[0] - M);
+        S = fma(t[1], f, S);
+        Q = fma(t[2], f * f, Q);
     }
-    double *o = tuples + 4 * (b * L + d);
-    o[0] = M;
-    o[1] = S;
-    o[2] = Q;
-    o[3] = n;
+    S = warp_sum(S);
+    Q = warp_sum(Q);
+    n = warp_sum(n);
+    if (lane == 0) {
+        double *o = tuples + 4 * (b * L + d);
+        o[0] = M;
+        o[1] = S;
+        o[2] = Q;
+        o[3] = n;
+    }
 }
 
 // ------------------------------------------------------- raw Philox words
@@ -291,7 +297,7 @@ cudaError_t launch_combine(const double *partial, double *tuples, int64_t b0, in
     if (n == 0) return cudaSuccess;
     const int th = 128;
     cudaGetLastError();
-    combine_kernel<<<(unsigned)((n + th - 1) / th), th, 0, st>>>(partial, tuples, b0, n_blocks, levels,
+    combine_kernel<<<(unsigned)((n + th / 32 - 1) / (th / 32)), th, 0, st>>>(partial, tuples, b0, n_blocks, levels,
                                                                items_per_block);
     return cudaGetLastError();
 }
