@@ -172,6 +172,27 @@ cudaError_t launch_cheb(const double *part, int splits, int64_t nb, const double
 // op 2: out[chunk][B] = sum (A - Q[c] C)^2 over the chunk's rows (Q: B Ritz values)
 cudaError_t launch_block_op(int op, int B, const double *A, const double *C, const double *Q, int n, int chunks,
                             double *out, cudaStream_t st);
+// The same product on the tensor cores from digit planes (spectrum_mma.cu):
+// Ynew = alpha U X + beta Ycur + gamma Yprev for the columns col0..col0+15 of X
+// (n x B), xmax their largest magnitudes as bits; ymax (or null) receives Ynew's.
+struct BandMma {
+    int n, w;                          // elements beyond w diagonals have no digits
+    int ea;                            // exponent of the largest element
+    unsigned char *A, *Xd;
+    unsigned long long *scratch_max;
+    int *status;                       // bit 0: a wait ran out
+};
+int band_exponent(unsigned long long bits);   // e of |v| = m 2^e, m in [1/2, 1), from v's bits
+cudaError_t launch_diag_max(const double *D, int64_t pitch, int n, int w, unsigned long long *dmax, cudaStream_t st);
+int64_t band_mma_bytes_a(int n, int w);
+int64_t band_mma_bytes_x(int n);
+cudaError_t launch_band_digits(const BandMma &M, const double *D, int64_t pitch, cudaStream_t st);
+cudaError_t launch_col_max(const double *X, int n, int B, int col0, unsigned long long *xmax, cudaStream_t st);
+cudaError_t launch_band_mma(const BandMma &M, const double *X, const unsigned long long *xmax, unsigned long long *ymax,
+                            int B, int col0, const double *Ycur, const double *Yprev, double *Ynew, double alpha,
+                            double beta, double gamma, cudaStream_t st);
+// one Lanczos step after wv = U v (alpha and beta into al[j] and be[j])
+cudaError_t launch_lanczos(int n, int j, double *v, double *vp, double *wv, double *al, double *be, cudaStream_t st);
 // vec[k n + i] = scale X[i][k], k < nev
 cudaError_t launch_vectors(int B, const double *X, int n, int nev, double scale, double *vec, cudaStream_t st);
 

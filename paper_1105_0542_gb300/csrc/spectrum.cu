@@ -21,9 +21,10 @@
 // The block width (8, 16 or 32 columns) holds nev wanted pairs plus at least
 // six guard vectors, so nearly degenerate pairs (a tunnelling doublet) sit
 // inside the block and are separated by the Rayleigh-Ritz step, not by the
-// filter.  Device work: the band matrix-block product (FP64 FMA bound,
-// 2B multiply-adds per stored element and row), the Chebyshev update, Gram
-// products and rotations; host work: B x B Cholesky and Jacobi.
+// filter.  Device work: the band matrix-block product with the Chebyshev update
+// (on the tensor cores in exact digits, spectrum_mma.cu; in double, FP64 bound,
+// where the digit planes have no room), Gram products and rotations; host work:
+// B x B Cholesky and Jacobi.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -39,6 +40,11 @@
 
 namespace su {
 namespace {
+
+// least n w B for the tensor-core product: at n = 1201, w = 158, B = 8 a product
+// takes 0.023 ms there and 0.013 in double, at n = 2001, w = 212, B = 16 0.029
+// and 0.050, at n = 16 385, w = 1297, B = 16 0.090 and 1.16
+constexpr int64_t kMmaLeast = 3000000;
 
 // symmetric eigenpairs of the k x k matrix A (row-major) by cyclic Jacobi
 // rotations; eigenvalues descending in ev, eigenvectors in the columns of V
@@ -91,6 +97,43 @@ void jacobi_eig(std::vector<double> A, int k, std::vector<double> &ev, std::vect
     V.swap(W);
 }
 
+// The smallest and largest eigenvalue of the symmetric tridiagonal matrix with
+// diagonal al and off-diagonal be, by bisection on the Sturm sequence's count of
+// negative pivots (Golub and Van Loan, Sec. 8.4).
+void tridiagonal_ends(const std::vector<double> &al, const std::vector<double> &be, double &least, double &most) {
+    const size_t k = al.size();
+    double lo = al[0], hi = al[0];
+    for (size_t i = 0; i < k; ++i) {   // Gershgorin
+        const double r = (i ? std::fabs(be[i - 1]) : 0.0) + (i + 1 < k ? std::fabs(be[i]) : 0.0);
+        lo = std::min(lo, al[i] - r);
+        hi = std::max(hi, al[i] + r);
+    }
+    auto below = [&](double x) {   // eigenvalues smaller than x
+        size_t n = 0;
+        double d = 1.0;
+        for (size_t i = 0; i < k; ++i) {
+            d = al[i] - x - (i ? be[i - 1] * be[i - 1] / d : 0.0);
+            if (d == 0.0) d = -1e-300;
+            n += d < 0.0;
+        }
+        return n;
+    };
+    auto find = [&](size_t want) {   // the eigenvalue that has `want` below it
+        double a = lo, b = hi;
+        for (int it = 0; it < 200 && a < b; ++it) {
+            const double m = 0.5 * (a + b);
+            if (m <= a || m >= b) break;
+            if (below(m) > want)
+                b = m;
+            else
+                a = m;
+        }
+        return 0.5 * (a + b);
+    };
+    least = find(0);
+    most = find(k - 1);
+}
+
 // lower Cholesky factor of the k x k matrix G (row-major); false if not
 // positive definite
 bool cholesky(const std::vector<double> &G, int k, std::vector<double> &Lf) {
@@ -124,6 +167,22 @@ std::vector<double> inverse_upper(const std::vector<double> &Lf, int k) {
     return X;
 }
 
+// device buffers, freed together
+struct Bufs {
+    std::vector<void *> v;
+    ~Bufs() {
+        for (void *p : v) cudaFree(p);
+    }
+    template <typename T>
+    cudaError_t get(T **p, size_t count) {
+        void *q = nullptr;
+        cudaError_t e = cudaMalloc(&q, count * sizeof(T));
+        if (e == cudaSuccess) v.push_back(q);
+        *p = static_cast<T *>(q);
+        return e;
+    }
+};
+
 struct Work {
     double *D = nullptr;
     int64_t pitch = 0;
@@ -132,6 +191,9 @@ struct Work {
     double *part = nullptr;      // splits x n x B
     double *gpart = nullptr;     // chunks x B x B
     double *dQ = nullptr;        // B x B (or B values)
+    bool mma = false;            // block products on the tensor cores
+    BandMma M{};
+    unsigned long long *mx[2] = {nullptr, nullptr};   // column maxima (32 each) of a product's input and output
     std::vector<double> hpart;
     int64_t matvecs = 0;         // vector products with U
     std::vector<cudaEvent_t> ev; // pairs around the block products (their device time)
@@ -146,27 +208,33 @@ struct Work {
         if (e_ != cudaSuccess) return e_;       \
     } while (0)
 
-// part = the split partial sums of U X; block products (B = W.B) are
-// bracketed by a pair of events for their device time
-cudaError_t matvec(Work &W, int B, const double *X) {
+// Ynew = alpha U X + beta Ycur + gamma Yprev for the block: on the tensor cores
+// (in: which of W.mx holds X's column maxima; the other receives Ynew's), or in
+// double from split partial sums.  Bracketed by a pair of events for its device time.
+cudaError_t product(Work &W, const double *X, const double *Ycur, const double *Yprev, double *Ynew, double alpha,
+                    double beta, double gamma, int in) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (B == W.B) {
-        SPC(cudaEventCreate(&e0));
-        W.ev.push_back(e0);
-        SPC(cudaEventCreate(&e1));
-        W.ev.push_back(e1);
-        SPC(cudaEventRecord(e0, W.st));
+    SPC(cudaEventCreate(&e0));
+    W.ev.push_back(e0);
+    SPC(cudaEventCreate(&e1));
+    W.ev.push_back(e1);
+    SPC(cudaEventRecord(e0, W.st));
+    if (W.mma) {
+        for (int c = 0; c < W.B; c += 16)
+            SPC(launch_band_mma(W.M, X, W.mx[in] + c, W.mx[in ^ 1] + c, W.B, c, Ycur, Yprev, Ynew, alpha, beta, gamma, W.st));
+    } else {
+        SPC(launch_band_matvec(W.B, W.D, W.pitch, W.n, W.w, W.splits, X, W.part, W.st));
+        SPC(launch_cheb(W.part, W.splits, (int64_t)W.n * W.B, Ycur, Yprev, Ynew, alpha, beta, gamma, W.st));
     }
-    SPC(launch_band_matvec(B, W.D, W.pitch, W.n, W.w, W.splits, X, W.part, W.st));
-    if (e1) SPC(cudaEventRecord(e1, W.st));
+    SPC(cudaEventRecord(e1, W.st));
+    W.matvecs += W.B;
     return cudaSuccess;
 }
 
-// Y = U X (block of W.B columns, or one column with B = 1)
-cudaError_t apply(Work &W, int B, const double *X, double *Y) {
-    SPC(matvec(W, B, X));
-    SPC(launch_cheb(W.part, W.splits, (int64_t)W.n * B, nullptr, nullptr, Y, 1.0, 0.0, 0.0, W.st));
-    W.matvecs += B;
+// W.mx[0] = the column maxima of X
+cudaError_t maxima(Work &W, const double *X) {
+    if (W.mma)
+        for (int c = 0; c < W.B; c += 16) SPC(launch_col_max(X, W.n, W.B, c, W.mx[0] + c, W.st));
     return cudaSuccess;
 }
 
@@ -249,44 +317,38 @@ int band_spectrum(const double *D, int64_t pitch, int n, int w, int nev, int deg
     // resident: the FP64 multiply-adds need the warps to hide load latency
     W.splits = std::max(1, std::min(w + 1, (32 * std::max(sms, 1) + rblocks - 1) / rblocks));
     W.chunks = std::max(1, std::min(std::max(sms, 1), (n + 31) / 32));
-    struct Bufs {
-        std::vector<void *> v;
-        ~Bufs() {
-            for (void *p : v) cudaFree(p);
-        }
-        cudaError_t get(double **p, size_t count) {
-            void *q = nullptr;
-            cudaError_t e = cudaMalloc(&q, count * sizeof(double));
-            if (e == cudaSuccess) v.push_back(q);
-            *p = static_cast<double *>(q);
-            return e;
-        }
-    } bufs;
+    Bufs bufs;
     const size_t nb = (size_t)n * B;
-    double *X, *Y0, *Y1, *Y2, *Z, *UX, *T;
+    const int steps = std::min(40, n);
+    double *X, *Y0, *Y1, *Y2, *Z, *UX, *T, *ab;
+    unsigned long long *dmax = nullptr;
     cudaError_t e = cudaSuccess;
     for (double **p : {&X, &Y0, &Y1, &Y2, &Z, &UX, &T})
         if (e == cudaSuccess) e = bufs.get(p, nb);
-    if (e == cudaSuccess) e = bufs.get(&W.part, (size_t)W.splits * nb);
     if (e == cudaSuccess) e = bufs.get(&W.gpart, (size_t)W.chunks * B * B);
     if (e == cudaSuccess) e = bufs.get(&W.dQ, (size_t)B * B);
-    if (e != cudaSuccess) {
+    if (e == cudaSuccess) e = bufs.get(&ab, (size_t)2 * steps);
+    if (e == cudaSuccess) e = bufs.get(&dmax, (size_t)w + 1 + 4 * 32);
+    if (e == cudaSuccess) e = bufs.get(&W.part, (size_t)W.splits * n);
+    auto no_buffers = [&] {
         cudaGetLastError();
         err = std::string("eigensolver buffers: ") + cudaGetErrorString(e);
         return e == cudaErrorMemoryAllocation ? SU_ENOMEM : SU_ECUDA;
-    }
+    };
+    if (e != cudaSuccess) return no_buffers();
     auto cuda_err = [&](cudaError_t c, const char *what) {
         err = std::string(what) + ": " + cudaGetErrorString(c);
         cudaGetLastError();
         return SU_ECUDA;
     };
 
-    // ---- the lower end of the spectrum: Lanczos steps on one vector
+    // ---- the lower end of the spectrum: Lanczos steps on one vector, all on
+    // the device; the host draws the start block meanwhile
     std::mt19937_64 rng(seed);
     std::normal_distribution<double> nd(0.0, 1.0);
+    std::vector<double> v((size_t)n), h(nb), hab((size_t)2 * steps);
+    std::vector<unsigned long long> dm((size_t)w + 1);
     {
-        const int steps = std::min(40, n);
-        std::vector<double> v((size_t)n), vp((size_t)n, 0.0), wv((size_t)n), al, be;
         double nrm = 0;
         for (double &x : v) {
             x = nd(rng);
@@ -294,42 +356,60 @@ int band_spectrum(const double *D, int64_t pitch, int n, int w, int nev, int deg
         }
         nrm = std::sqrt(nrm);
         for (double &x : v) x /= nrm;
-        double beta = 0.0;
+    }
+    if ((e = cudaMemcpyAsync(X, v.data(), (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st)) ||
+        (e = launch_diag_max(D, pitch, n, w, dmax, st)))
+        return cuda_err(e, "Lanczos bounds");
+    for (int j = 0; j < steps; ++j) {
+        if ((e = launch_band_matvec(1, W.D, W.pitch, n, w, W.splits, X, W.part, st)) ||
+            (e = launch_cheb(W.part, W.splits, n, nullptr, nullptr, Y2, 1.0, 0.0, 0.0, st)) ||
+            (e = launch_lanczos(n, j, X, Y1, Y2, ab, ab + steps, st)))
+            return cuda_err(e, "Lanczos bounds");
+        W.matvecs += 1;
+    }
+    for (double &x : h) x = nd(rng);
+    if ((e = cudaMemcpyAsync(dm.data(), dmax, dm.size() * sizeof(dm[0]), cudaMemcpyDeviceToHost, st)) ||
+        (e = cudaMemcpyAsync(hab.data(), ab, hab.size() * sizeof(double), cudaMemcpyDeviceToHost, st)) ||
+        (e = cudaStreamSynchronize(st)))
+        return cuda_err(e, "Lanczos bounds");
+    {
+        std::vector<double> al, be;
         for (int j = 0; j < steps; ++j) {
-            if ((e = cudaMemcpyAsync(X, v.data(), (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st)) ||
-                (e = apply(W, 1, X, Y0)) ||
-                (e = cudaMemcpyAsync(wv.data(), Y0, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, st)) ||
-                (e = cudaStreamSynchronize(st)))
-                return cuda_err(e, "Lanczos bounds");
-            double a = 0;
-            for (int i = 0; i < n; ++i) a += v[(size_t)i] * wv[(size_t)i];
-            double b2 = 0;
-            for (int i = 0; i < n; ++i) {
-                wv[(size_t)i] -= a * v[(size_t)i] + beta * vp[(size_t)i];
-                b2 += wv[(size_t)i] * wv[(size_t)i];
-            }
-            al.push_back(a);
-            beta = std::sqrt(b2);
-            be.push_back(beta);
-            if (!(beta > 0)) break;
-            vp = v;
-            for (int i = 0; i < n; ++i) v[(size_t)i] = wv[(size_t)i] / beta;
+            al.push_back(hab[(size_t)j]);
+            be.push_back(hab[(size_t)(steps + j)]);
+            if (!(be.back() > 0)) break;
         }
-        const int k = (int)al.size();
-        std::vector<double> Tm((size_t)k * k, 0.0), ev, V;
-        for (int i = 0; i < k; ++i) {
-            Tm[(size_t)i * k + i] = al[(size_t)i];
-            if (i + 1 < k) Tm[(size_t)i * k + i + 1] = Tm[(size_t)(i + 1) * k + i] = be[(size_t)i];
+        double least = 0, most = 0;
+        tridiagonal_ends(al, be, least, most);
+        res.upper = most + be.back();
+        res.lower = least - be.back();
+    }
+    // ---- digit planes for the tensor-core product, where the band's values
+    // are finite and the planes fit the device
+    {
+        const unsigned long long top = *std::max_element(dm.begin(), dm.end());
+        W.M.n = n;
+        W.M.ea = band_exponent(top);
+        // diagonals whose elements all round to zero digits (below 2^-48 of the largest's power of two)
+        W.M.w = w;
+        while (W.M.w > 0 && band_exponent(dm[(size_t)W.M.w]) < W.M.ea - 48) --W.M.w;
+        if (W.M.ea > -400 && W.M.ea < 400 && (int64_t)n * w * B >= kMmaLeast) {
+            W.mx[0] = dmax + w + 1;
+            W.mx[1] = W.mx[0] + 32;
+            W.M.scratch_max = W.mx[1] + 32;
+            W.M.status = reinterpret_cast<int *>(W.M.scratch_max + 32);
+            W.mma = bufs.get(&W.M.A, (size_t)band_mma_bytes_a(n, W.M.w)) == cudaSuccess &&
+                    bufs.get(&W.M.Xd, (size_t)band_mma_bytes_x(n)) == cudaSuccess;
+            if (!W.mma) cudaGetLastError();
         }
-        jacobi_eig(Tm, k, ev, V);
-        res.upper = ev.front() + be.back();
-        res.lower = ev.back() - be.back();
+        // (in double the split partial sums of the whole block)
+        if (!W.mma && (e = bufs.get(&W.part, (size_t)W.splits * nb)) != cudaSuccess) return no_buffers();
+        if (W.mma && ((e = cudaMemsetAsync(W.M.status, 0, sizeof(int), st)) || (e = launch_band_digits(W.M, D, pitch, st))))
+            return cuda_err(e, "digit planes");
     }
     const double lo = res.lower;
 
     // ---- a random block, orthonormalized, and its Rayleigh-Ritz pairs
-    std::vector<double> h(nb);
-    for (double &x : h) x = nd(rng);
     if ((e = cudaMemcpyAsync(Y0, h.data(), nb * sizeof(double), cudaMemcpyHostToDevice, st)) ||
         (e = cudaStreamSynchronize(st)))
         return cuda_err(e, "initial block");
@@ -342,7 +422,8 @@ int band_spectrum(const double *D, int64_t pitch, int n, int w, int nev, int deg
             err = "the block lost rank (Cholesky QR failed)";
             return SU_ECUDA;
         }
-        if ((e = apply(W, B, X, Z)) || (e = gram(W, X, Z, H))) return cuda_err(e, "Rayleigh-Ritz");
+        if ((e = maxima(W, X)) || (e = product(W, X, nullptr, nullptr, Z, 1.0, 0.0, 0.0, 0)) || (e = gram(W, X, Z, H)))
+            return cuda_err(e, "Rayleigh-Ritz");
         for (int i = 0; i < B; ++i)   // symmetrize the projection's rounding
             for (int j = i + 1; j < B; ++j)
                 H[(size_t)i * B + j] = H[(size_t)j * B + i] = 0.5 * (H[(size_t)i * B + j] + H[(size_t)j * B + i]);
@@ -354,9 +435,15 @@ int band_spectrum(const double *D, int64_t pitch, int n, int w, int nev, int deg
             (e = launch_block_op(2, B, UX, X, W.dQ, n, W.chunks, W.gpart, st)))
             return cuda_err(e, "residuals");
         std::vector<double> rp((size_t)W.chunks * B);
+        int waits = 0;
         if ((e = cudaMemcpyAsync(rp.data(), W.gpart, rp.size() * sizeof(double), cudaMemcpyDeviceToHost, st)) ||
+            (W.mma && (e = cudaMemcpyAsync(&waits, W.M.status, sizeof(int), cudaMemcpyDeviceToHost, st))) ||
             (e = cudaStreamSynchronize(st)))
             return cuda_err(e, "residuals");
+        if (waits) {
+            err = "a block product's wait ran out";
+            return SU_ETIMEOUT;
+        }
         double worst = 0.0;
         for (int c = 0; c < B; ++c) {
             double s = 0;
@@ -373,15 +460,9 @@ int band_spectrum(const double *D, int64_t pitch, int n, int w, int nev, int deg
         const double c0 = 0.5 * (cut + lo), e0 = 0.5 * (cut - lo);
         const int m = it == 0 ? std::min(4, degree) : degree;
         double *ym1 = X, *y = Y0, *yp = Y1;
-        if ((e = matvec(W, B, X)) ||
-            (e = launch_cheb(W.part, W.splits, (int64_t)nb, X, nullptr, Y0, 1.0 / e0, -c0 / e0, 0.0, st)))
-            return cuda_err(e, "filter");
-        W.matvecs += B;
+        if ((e = maxima(W, X)) || (e = product(W, X, X, nullptr, Y0, 1.0 / e0, -c0 / e0, 0.0, 0))) return cuda_err(e, "filter");
         for (int j = 1; j < m; ++j) {
-            if ((e = matvec(W, B, y)) ||
-                (e = launch_cheb(W.part, W.splits, (int64_t)nb, y, ym1, yp, 2.0 / e0, -2.0 * c0 / e0, -1.0, st)))
-                return cuda_err(e, "filter");
-            W.matvecs += B;
+            if ((e = product(W, y, y, ym1, yp, 2.0 / e0, -2.0 * c0 / e0, -1.0, j & 1))) return cuda_err(e, "filter");
             // rotate the three buffers: the oldest becomes the next output
             double *old = ym1;
             ym1 = y;
