@@ -19,7 +19,8 @@ LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libspeedup_gb300.so")
 CLI = os.path.join(LIBDIR, "speedup")
 SOURCES = ["sampler.cu", "api.cu", "generator.cpp", "peaks.cu", "proposal.cu", "train.cu", "evolution.cu", "nd.cu", "spectrum.cu",
-           "sampler_fx.cu", "fx_plan.cpp", "nd_plan.cpp", "spectrum_mma.cu"]
+           "sampler_fx.cu", "fx_plan.cpp", "nd_plan.cpp", "spectrum_mma.cu",
+           "general.cu", "general_plan.cpp"]
 # the sampler kernel, once per (precision, ring): compiled in parallel
 INSTANCES = [(prec, ring, 0) for prec in (64, 32) for ring in (0, 1, 2)] + [(64, 3, 0)]
 # double-precision samplers that read tables too large for shared memory from global memory

@@ -379,6 +379,16 @@ static int general_image(const su::GeneralEffective &G, const su::GeneralPotenti
         }
     }
     for (int n = 1; n <= kGenMaxSym; ++n) D.inv[n] = 1.0 / (double)n;
+    for (int n = 1; n <= kGenMaxSym + 1; ++n) D.invf[n] = (float)(1.0 / (double)n);
+    for (int i = 0; i <= 8; ++i)
+        if (V.a[i] != 0.0) D.deg = i;
+    for (int j = 0; j <= 8; ++j) {
+        double f = 1.0;
+        for (int r = 2; r <= j; ++r) f *= (double)r;
+        for (int i = j; i <= 8; ++i) D.poly_tay[j][i] = (float)(j <= G.J ? D.poly_der[j][i] / f : 0.0);
+    }
+    for (int q = 0; q < V.ns; ++q)
+        for (int n = 0; n <= G.J; ++n) D.sech_tay[q][n] = (float)(V.sech[q][0] * std::pow(V.sech[q][1], n) * (n + 1));
     const size_t o_nodes = (sizeof(GeneralDev) + 15) & ~(size_t)15;
     const size_t bytes = o_nodes + nodes.size() * sizeof(GeneralNode);
     CU(dmalloc(d_out, bytes), "device allocation (general program)");
@@ -470,6 +480,80 @@ static int plan_rounds(su_plan &pl, int rounds, int sms, int smem_max) {
     return occ;
 }
 
+// The general potential's program split by size (general_split): the level's
+// single-precision entries (times the factorials that the kernel's derivatives
+// are short of), and its double part's nodes and entries, behind the tables.
+static void split_general(su_plan &pl, std::vector<unsigned char> &blob, int smem_max) {
+    using namespace su;
+    SamplerParams &P = pl.P;
+    const GeneralEffective &G = *pl.G;
+    const int S = pl.s, M = P.M;
+    const size_t nn = G.depth.size();
+    const std::vector<double> tab(reinterpret_cast<const double *>(blob.data()),
+                                  reinterpret_cast<const double *>(blob.data()) + (size_t)S * M);
+    std::vector<double> ms, fact(nn, 1.0), fs((size_t)G.J + 1, 1.0), stk((size_t)G.J + 3 * G.p + 2, 1.0);
+    general_moments(G, pl.V, pl.a, pl.b, pl.T, ms);
+    for (int j = 2; j <= G.J; ++j) fs[(size_t)j] = fs[(size_t)j - 1] * j;
+    for (size_t t = 1; t < nn; ++t) {
+        fact[t] = stk[(size_t)G.depth[t] - 1] * fs[(size_t)G.sym[t]];
+        stk[(size_t)G.depth[t]] = fact[t];
+    }
+    std::vector<float> tail((size_t)S * M, 0.0f);
+    std::vector<GeneralNode> hnodes;
+    std::vector<double> hcoef;
+    std::vector<int> head;
+    bool any = false;
+    for (int d = 0; d < pl.levels; ++d) {
+        const double *t = tab.data() + (size_t)d * M;
+        general_split(G, ms, pl.a, pl.b, pl.T, S - d, t, head);
+        int total = 0;
+        bool fits = true;
+        for (size_t k = 0; k < nn; ++k) {
+            total += head[k];
+            for (int e = head[k]; e < G.count[k]; ++e) {
+                const double c = t[G.first[k] + e] * fact[k];
+                fits = fits && std::fabs(c) < 1e30;
+                tail[(size_t)d * M + G.first[k] + e] = (float)c;
+            }
+        }
+        if (!fits || total == 0 || 2 * total > M) continue;
+        // the nodes with entries and their ancestors, in order
+        std::vector<char> keep(nn, 0);
+        std::vector<size_t> path((size_t)kGenMaxDepth + 1, 0);
+        for (size_t k = 0; k < nn; ++k) {
+            path[(size_t)G.depth[k]] = k;
+            if (head[k])
+                for (int q = 0; q <= G.depth[k]; ++q) keep[path[(size_t)q]] = 1;
+        }
+        P.gs.h0[d] = (int)hnodes.size();
+        P.gs.hc[d] = (int)hcoef.size();
+        for (size_t k = 0; k < nn; ++k) {
+            if (!keep[k] && k) continue;
+            hnodes.push_back({(unsigned char)G.depth[k], (unsigned char)G.sym[k], (unsigned short)head[k],
+                              (int)hcoef.size() - P.gs.hc[d]});
+            for (int e = 0; e < head[k]; ++e) hcoef.push_back(t[G.first[k] + e]);
+            if (k) P.gs.hj[d] = std::max(P.gs.hj[d], G.sym[k]);
+        }
+        P.gs.hn[d] = (int)hnodes.size() - P.gs.h0[d];
+        any = true;
+    }
+    if (!any) return;
+    auto put = [&](const void *src, size_t bytes) {
+        const size_t at = (blob.size() + 15) / 16 * 16;
+        blob.resize(at + bytes);
+        if (bytes) std::memcpy(blob.data() + at, src, bytes);
+        return (int64_t)at;
+    };
+    P.gs.on = 1;
+    P.gs.n_nodes = (int)nn;
+    P.gs.tail = put(tail.data(), tail.size() * sizeof(float));
+    P.gs.hnodes = put(hnodes.data(), hnodes.size() * sizeof(GeneralNode));
+    P.gs.hcoef = put(hcoef.data(), hcoef.size() * sizeof(double));
+    // program and entries in shared memory where four CTAs still fit an SM
+    P.gs.staged = 1;
+    if (sampler_smem_bytes(P, SU_FP64) > (size_t)std::min(smem_max, 56 * 1024)) P.gs.staged = 0;
+}
+
 // The sampler's parameters and launch shape of a plan (everything but the
 // device pointers): host work and occupancy queries only, no allocation.  The
 // fixed-point sampler's images go behind the level tables in blob.
@@ -531,6 +615,8 @@ static int plan_shape(su_plan &pl, int sms, int smem_max, std::vector<unsigned c
             std::memcpy(blob.data() + P.fx.tail_off, tail.data(), tail.size() * sizeof(float));
         }
     }
+    if (general && prec == SU_FP64 && S >= 1 && !P.wf_on && !P.generic && pl.opt.seg_log2 == 0 && pl.opt.rounds == 0)
+        split_general(pl, blob, smem_max);
     // launch shape: one path per thread, persistent grid over items of
     // 128 * rounds samples
     const int occ1 = plan_rounds(pl, 1, sms, smem_max);

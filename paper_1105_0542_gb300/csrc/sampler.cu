@@ -30,6 +30,9 @@ const void *batch_entry_f32_1();
 const void *batch_entry_f32_2();
 // the double sampler in fixed point (sampler_fx.cu)
 const void *sampler_fx_entry(int ring);
+// the general potential's split sampler (general.cu)
+const void *general_entry();
+size_t general_smem_bytes(const SamplerParams &P);
 size_t sampler_fx_smem_bytes(const SamplerParams &P);
 // the compiled-shape kernels of group g = k % kFixedGroups (sampler_inst.cu, SU_FIXED = g)
 #define SU_FIXED_GROUP(g)                        \
@@ -179,6 +182,7 @@ const void *pick(const SamplerParams &P, int precision) {
         return k < 0 ? sampler_fx_entry(P.ring) : kFxFixed[k % kFixedGroups](k);
     }
     if (const void *fn = pick_fixed(P, precision)) return fn;
+    if (P.gs.on) return general_entry();
     if (P.ring == RING_GENERAL) return precision == SU_FP64 ? sampler_entry_f64_3() : nullptr;
     if (P.tab_global) {
         if (precision != SU_FP64) return nullptr;
@@ -224,6 +228,7 @@ size_t batch_smem_bytes(const BatchParams &B, int precision) {
 
 size_t sampler_smem_bytes(const SamplerParams &P, int precision) {
     if (P.fx.on) return sampler_fx_smem_bytes(P);
+    if (P.gs.on) return general_smem_bytes(P);
     const size_t rs = precision == SU_FP32 ? sizeof(float) : sizeof(double);
     const int C = 1 << (P.S - P.F);
     size_t off = P.w_out ? 0 : rs * (size_t)P.levels * kThreads * P.rounds;

@@ -37,6 +37,11 @@ struct GeneralDev {
     double sech_scale[4][kGenMaxSym];          // B alpha^n (n+1)!
     double expo[4][3];                         // E, kappa, x0
     double inv[kGenMaxSym + 1];                // 1 / n
+    // single precision, derivatives over j!
+    int deg;                                   // degree of the polynomial part
+    float poly_tay[9][9];                      // a_i C(i, j)
+    float sech_tay[4][kGenMaxSym];             // B alpha^n (n+1)
+    float invf[kGenMaxSym + 2];
 };
 
 // The fixed-point sampler's plan (sampler_fx.cuh; built by fx_plan).  Path
@@ -60,6 +65,15 @@ struct FxParams {
     double q_unit;
     FxLevel lv[SU_MAX_S];
     int64_t head_off, tail_off;   // from the tables: [S][hrow] int64, [S][M] float
+};
+
+// The split general program (general.cu; built by general_split): byte offsets
+// from the tables, and per level (row d) the double part's nodes, entries and
+// highest derivative (hn = 0: the whole program in double).
+struct GeneralSplit {
+    int on, staged, n_nodes;
+    int64_t tail, hnodes, hcoef;
+    int hn[SU_MAX_S], h0[SU_MAX_S], hc[SU_MAX_S], hj[SU_MAX_S];
 };
 
 struct SamplerParams {
@@ -95,8 +109,16 @@ struct SamplerParams {
     float *q_out;             // device: per-sample mode, single precision only: path points [sample][N+1] (or null)
     int *flags;               // device: bit 0 = non-finite weight seen
     const GeneralDev *general;  // device: RING_GENERAL only
+    GeneralSplit gs;            // RING_GENERAL: the split program where gs.on
     FxParams fx;                // double precision: the fixed-point sampler where fx.on
 };
+
+// root mean squares of the general program's monomials over the bridge
+void general_moments(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T,
+                     std::vector<double> &ms);
+// head[t] = the leading entries of node t that need double precision on level n
+void general_split(const GeneralEffective &G, const std::vector<double> &ms, double a, double b, double T, int n,
+                   const double *table, std::vector<int> &head);
 
 // The fixed-point plan of a double-precision plan's tables (rows of M entries,
 // kernel_table's, for levels n = S..1): fills P.fx (on = 0 where the ranges do

@@ -148,13 +148,13 @@ __device__ __forceinline__ R ring_var(R us, R alpha) {
 // polynomial table; Gaussians through the Hermite recurrence; sech^2 = tanh'
 // through the Taylor coefficients a_k of tanh, (n+1) a_{n+1} = -sum_k a_k a_{n-k}
 // from tanh' = 1 - tanh^2, which stay accurate where tanh is near +-1.
-__device__ __forceinline__ void general_derivatives(double x, const GeneralDev *__restrict__ G,
+__device__ __forceinline__ void general_derivatives(double x, const GeneralDev *__restrict__ G, int J,
                                                     double (&V)[kGenMaxSym]) {
-    const int J = G->J;
+    const int deg = G->deg;
     for (int j = 0; j <= J; ++j) {
         double v = 0.0;
-        if (j <= 8)
-            for (int i = 8; i >= j; --i) v = fma(v, x, G->poly_der[j][i]);
+        if (j <= deg)
+            for (int i = deg; i >= j; --i) v = fma(v, x, G->poly_der[j][i]);
         V[j] = v;
     }
     for (int g = 0; g < G->ng; ++g) {
@@ -206,21 +206,20 @@ __device__ __forceinline__ void general_derivatives(double x, const GeneralDev *
 // times the monomial.  Two slices share every node and coefficient load.
 template <int B>
 __device__ __noinline__ double2 slice_general(double ql0, double qr0, double ql1, double qr1,
-                                              const double *__restrict__ coef,
-                                              const GeneralDev *__restrict__ G) {
+                                              const double *__restrict__ coef, const GeneralDev *__restrict__ G,
+                                              const GeneralNode *__restrict__ nodes, int nn, int J) {
     const double ql[2] = {ql0, ql1}, qr[2] = {qr0, qr1};
     double V[B][kGenMaxSym], Y[B], stk[B][kGenMaxDepth + 1], w[B];
 #pragma unroll
     for (int b = 0; b < B; ++b) {
-        general_derivatives(0.5 * (ql[b] + qr[b]), G, V[b]);
+        general_derivatives(0.5 * (ql[b] + qr[b]), G, J, V[b]);
         const double vs = qr[b] - ql[b];
         Y[b] = vs * vs;
         stk[b][0] = 1.0;
         w[b] = 0.0;
     }
-    const int nn = G->n_nodes;
     for (int t = 0; t < nn; ++t) {
-        const GeneralNode nd = G->nodes[t];
+        const GeneralNode nd = nodes[t];
         double mu[B];
 #pragma unroll
         for (int b = 0; b < B; ++b) {
@@ -262,7 +261,7 @@ template <typename R, int RING, typename TT, typename SP>
 __device__ __forceinline__ R slice(R ql, R qr, const TT *__restrict__ tab, const SP &P, R alpha) {
     if constexpr (RING == RING_GENERAL) {
         static_assert(sizeof(R) == 8, "the general potential is evaluated in double");
-        return slice_general<1>(ql, qr, ql, qr, tab, P.general).x;
+        return slice_general<1>(ql, qr, ql, qr, tab, P.general, P.general->nodes, P.general->n_nodes, P.general->J).x;
     }
     const R us = ql + qr;
     const R vs = qr - ql;
@@ -383,12 +382,14 @@ __device__ __forceinline__ R level_sum(const R (&q)[NQ], const TT *__restrict__ 
     if constexpr (RING == RING_GENERAL) {
         R total = 0;
         if constexpr (NS == 1) {
-            total = slice_general<1>(q[0], q[STR], q[0], q[STR], tab, P.general).x;
+            total = slice_general<1>(q[0], q[STR], q[0], q[STR], tab, P.general, P.general->nodes, P.general->n_nodes,
+                                     P.general->J).x;
         } else {
 #pragma unroll
             for (int k = 0; k < NS; k += 2) {   // unrolled: q stays in registers
                 const double2 r = slice_general<2>(q[k * STR], q[(k + 1) * STR], q[(k + 1) * STR],
-                                                   q[(k + 2) * STR], tab, P.general);
+                                                   q[(k + 2) * STR], tab, P.general, P.general->nodes,
+                                                   P.general->n_nodes, P.general->J);
                 total += r.x + r.y;
             }
         }
