@@ -2668,9 +2668,8 @@ extern "C" int su_mlp_loss_grad(const float *theta, const float *d_X, const floa
                                 int64_t n, double *loss, float *grad) {
     if (!theta || !d_X || !d_u || !d_rw || !loss || !grad || n < 1 || n > (1 << 22))
         return fail(SU_EINVAL, "bad arguments");
-    const int R = (int)((n + 31) / 32 * 32);
     su::train::Workspace ws;
-    CU(ws.reserve(R), "training workspace");
+    CU(ws.make((int)n), "training workspace");
     cudaStream_t st = nullptr;
     double norm = 0;
     {
@@ -2680,8 +2679,8 @@ extern "C" int su_mlp_loss_grad(const float *theta, const float *d_X, const floa
     }
     if (!(norm > 0)) return fail(SU_EINVAL, "row weights must have a positive sum");
     CU(cudaMemcpyAsync(ws.theta, theta, (size_t)su::mlp::kParams * 4, cudaMemcpyHostToDevice, st), "upload theta");
-    CU(su::train::rows_from_features(ws, d_X, d_u, d_rw, (int)n, R, st), "rows");
-    CU(su::train::loss_grad(ws, R, 1.0 / norm, true, st), "loss and gradient");
+    CU(su::train::pack(ws, st), "operands");
+    CU(su::train::loss_grad(ws, d_X, d_u, d_rw, (int)n, 1.0 / norm, st), "loss and gradient");
     CU(cudaMemcpyAsync(grad, ws.grad, (size_t)su::mlp::kParams * 4, cudaMemcpyDeviceToHost, st), "read gradient");
     CU(cudaMemcpyAsync(loss, ws.loss, 8, cudaMemcpyDeviceToHost, st), "read loss");
     int tstat = 0;
@@ -2728,7 +2727,9 @@ extern "C" int speedup_train_proposal(int model, const double *params, int n_par
     fr.v.push_back(d_w);
     CU(dmalloc(&d_flag, 4), "device allocation (flag)");
     fr.v.push_back(d_flag);
-    CU(dmalloc(&d_ids, (size_t)to.batch_paths * 4), "device allocation (ids)");
+    // minibatch ids, drawn ahead for as many steps as 4 MB of them make
+    const int drawn = std::min(to.steps, std::max(1, (1 << 20) / to.batch_paths));
+    CU(dmalloc(&d_ids, (size_t)to.batch_paths * drawn * 4), "device allocation (ids)");
     fr.v.push_back(d_ids);
     CU(dmalloc(&d_sig, 16 * 4), "device allocation (sigma)");
     fr.v.push_back(d_sig);
@@ -2741,13 +2742,15 @@ extern "C" int speedup_train_proposal(int model, const double *params, int n_par
     if (su::sampler_occupancy(P, SU_FP32, smem) < 1) return fail(SU_ECUDA, "sampler not resident");
     CU(cudaMemset(d_flag, 0, 4), "clear flag");
     CU(su::launch_sampler(P, SU_FP32, pl->grid, smem, nullptr), "path sampling");
-    std::vector<double> w((size_t)to.n_train * s);
-    CU(cudaMemcpy(w.data(), d_w, w.size() * 8, cudaMemcpyDeviceToHost), "read weights");
+    double *d_cdf = nullptr;
+    CU(dmalloc(&d_cdf, (size_t)to.n_train * sizeof(double)), "device allocation (cdf)");
+    fr.v.push_back(d_cdf);
+    CU(su::train::top_weights(d_w, to.n_train, s, d_cdf, nullptr), "top-level weights");
     // 2. training weights: top-level log-weights clipped at a quantile (the
     //    weighted likelihood of rare huge weights would fit one path), then
     //    minibatches drawn in proportion to them
     std::vector<double> wt((size_t)to.n_train);
-    for (int64_t i = 0; i < to.n_train; ++i) wt[(size_t)i] = w[(size_t)i * s + (s - 1)];
+    CU(cudaMemcpy(wt.data(), d_cdf, wt.size() * 8, cudaMemcpyDeviceToHost), "read weights");
     std::vector<double> srt = wt;
     const size_t qi = std::min(srt.size() - 1, (size_t)(to.clip_quantile * (double)(srt.size() - 1)));
     std::nth_element(srt.begin(), srt.begin() + qi, srt.end());
@@ -2766,20 +2769,14 @@ extern "C" int speedup_train_proposal(int model, const double *params, int n_par
     }
     if (!(acc > 0)) return fail(SU_ENONFINITE, "all training weights vanish");
     // 3. Adam on minibatches of batch_paths paths x (N-1) midpoints, drawn on
-    //    the device from the running sums of the weights; one step (draw, rows,
-    //    loss and gradient, Adam, loss record) is captured as a CUDA graph on a
+    //    the device from the running sums of the weights; one step (rows, loss
+    //    and gradient; Adam, loss record) is captured as a CUDA graph on a
     //    stream of its own and replayed `steps` times
-    const int R = to.batch_paths * (N - 1);
     su::train::Workspace ws;
-    CU(ws.reserve(R), "training workspace");
-    double *d_cdf = nullptr, *d_losses = nullptr;
-    int *d_step = nullptr;
-    CU(dmalloc(&d_cdf, cdf.size() * sizeof(double)), "device allocation (cdf)");
-    fr.v.push_back(d_cdf);
+    CU(ws.make(to.batch_paths * (N - 1)), "training workspace");
+    double *d_losses = nullptr;
     CU(dmalloc(&d_losses, (size_t)to.steps * sizeof(double)), "device allocation (losses)");
     fr.v.push_back(d_losses);
-    CU(dmalloc(&d_step, sizeof(int)), "device allocation (step)");
-    fr.v.push_back(d_step);
     struct GraphRes {
         cudaStream_t st = nullptr;
         cudaGraph_t g = nullptr;
@@ -2796,24 +2793,24 @@ extern "C" int speedup_train_proposal(int model, const double *params, int n_par
     CU(cudaMemcpy(d_sig, sig, sizeof sig, cudaMemcpyHostToDevice), "upload sigma");
     CU(cudaMemcpy(d_cdf, cdf.data(), cdf.size() * sizeof(double), cudaMemcpyHostToDevice), "upload cdf");
     CU(cudaMemcpy(ws.theta, theta, (size_t)su::mlp::kParams * 4, cudaMemcpyHostToDevice), "upload theta");
-    CU(cudaMemset(ws.m, 0, (size_t)su::mlp::kParams * 8), "clear moments");   // m and v are adjacent
-    CU(cudaMemset(d_step, 0, sizeof(int)), "clear step");
-    CU(su::train::fill(ws.rw, 1.0f, R, nullptr), "row weights");
+    CU(su::train::pack(ws, nullptr), "operands");
     CU(cudaDeviceSynchronize(), "training set-up");
     const int64_t n_train = to.n_train;
     CU(cudaStreamBeginCapture(gr.st, cudaStreamCaptureModeThreadLocal), "begin capture");
-    cudaError_t ce = su::train::sample_ids(d_cdf, n_train, acc, to.seed, d_step, to.batch_paths, d_ids, gr.st);
-    if (ce == cudaSuccess)
-        ce = su::train::build_rows(ws, d_paths, np1, d_ids, to.batch_paths, (float)a, (float)b, (float)T, s, d_sig,
-                                   gr.st);
-    if (ce == cudaSuccess) ce = su::train::loss_grad(ws, R, 1.0 / R, true, gr.st);
-    if (ce == cudaSuccess) ce = su::train::adam_step_dev(ws, d_step, (float)to.lr, gr.st);
-    if (ce == cudaSuccess) ce = su::train::step_tail(d_step, ws.loss, d_losses, gr.st);
+    cudaError_t ce = su::train::path_step(ws, d_paths, np1, d_ids, drawn, to.batch_paths, (float)a, (float)b, (float)T, s,
+                                          d_sig, gr.st);
+    if (ce == cudaSuccess) ce = su::train::adam_step(ws, (float)to.lr, d_losses, gr.st);
     const cudaError_t ee = cudaStreamEndCapture(gr.st, &gr.g);
     if (ce != cudaSuccess) return cuda_fail(ce, "capturing the training step");
     CU(ee, "end capture");
     CU(cudaGraphInstantiate(&gr.ge, gr.g, 0), "instantiate the training step");
-    for (int t = 0; t < to.steps; ++t) CU(cudaGraphLaunch(gr.ge, gr.st), "training step");
+    for (int t = 0; t < to.steps; ++t) {
+        if (t % drawn == 0)
+            CU(su::train::sample_ids(d_cdf, n_train, acc, to.seed, t, std::min(drawn, to.steps - t), to.batch_paths, d_ids,
+                                     gr.st),
+               "minibatch draws");
+        CU(cudaGraphLaunch(gr.ge, gr.st), "training step");
+    }
     CU(cudaStreamSynchronize(gr.st), "training");
     if (loss_out)
         CU(cudaMemcpy(loss_out, d_losses, (size_t)to.steps * sizeof(double), cudaMemcpyDeviceToHost), "read losses");

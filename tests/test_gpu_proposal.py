@@ -154,6 +154,28 @@ def test_training_gradient_matches_oracle():
             assert np.linalg.norm(blk - ref) <= 0.06 * np.linalg.norm(ref) + 1e-7, (o, i, size)
 
 
+@pytest.mark.parametrize("n", [1, 127, 129, 50_001])
+def test_training_gradient_at_tile_edges(n):
+    """One row, a tile short of and past its 128 rows, several tiles per thread
+    block: the bounds of test_training_gradient_matches_oracle."""
+    th = _theta(22, 1.0)
+    rng = np.random.default_rng(n)
+    X = np.stack([np.full(n, 0.5), np.full(n, -1.0), np.full(n, 2.0), rng.integers(1, 7, n) / 6,
+                  rng.normal(0, 1.2, n), rng.normal(0, 1.2, n)], axis=1)
+    u, rw = rng.normal(0, 1.0, n), rng.uniform(0.2, 2.0, n)
+    dev = lambda v: torch.tensor(v, dtype=torch.float32, device="cuda").contiguous()
+    L, g = su.su_mlp_loss_grad(th, dev(X), dev(u), dev(rw))
+    f32 = lambda v: np.asarray(v, dtype=np.float32).astype(np.float64)
+    Lr, gr = pr.loss_and_grad(f32(th), f32(X), f32(u), f32(rw))
+    assert L == pytest.approx(Lr, rel=2e-2, abs=2e-3)
+    k = 0
+    for o, i in pr.SIZES:
+        for size in (o * i, o):
+            blk, ref = g[k:k + size].astype(np.float64), gr[k:k + size]
+            k += size
+            assert np.linalg.norm(blk - ref) <= 0.06 * np.linalg.norm(ref) + 1e-7, (o, i, size)
+
+
 def test_training_lowers_the_loss():
     th0 = pr.init(5).astype(np.float32)
     th, losses = su.speedup_train_proposal("dw", [5.0], -1.0, 1.0, 5.0, 12, 6, 77, th0, n_train=200_000,
