@@ -20,10 +20,13 @@
 // rows 2..15 of W4 zero) issued by one thread into tensor-memory columns
 // [0, 128) (outputs: [128, 144)), a commit to an mbarrier, and an epilogue
 // in which warp w reads tensor-memory lanes 32 (w % 4) .. +31 (its rows) and
-// a quarter of the columns of its quadrant's rows (16 warps: 32 columns each),
-// adds the bias, applies GELU (erf by a polynomial, two values per packed
-// multiply-add) and writes the bfloat16 activations back into the A tile for
-// the next layer.
+// half of the columns of its quadrant's rows, adds the bias, applies GELU (erf
+// by a polynomial, two values per packed multiply-add) and writes the bfloat16
+// activations back into the A tile for the next layer.
+//
+// A tile belongs to a group of eight warps with its own accumulators, A tiles,
+// named barrier and mbarrier; a CTA runs two groups on one copy of the weights,
+// so that one group's epilogue fills the other's wait for its MMAs (@FIG@).
 #include <cuda_bf16.h>
 #include <cstdint>
 
@@ -37,9 +40,11 @@ constexpr int kParams = kHid * kIn + kHid + 2 * (kHid * kHid + kHid) + kOut * kH
 constexpr int kK1 = 16;        // layer-1 K: the 6 features, zero-padded
 constexpr int kNOut = 16;      // output-layer N: 2 outputs, zero-padded
 constexpr int kRows = 128;     // rows per tile = the MMA's M
-constexpr int kThreads = 512;  // 16 warps: four per tensor-memory lane quadrant
-constexpr int kColsPerWarp = kHid * 4 / (kThreads / 32);   // epilogue columns of a warp
-constexpr int kTmemCols = 256; // [0, 128) hidden accumulator, [128, 144) outputs
+constexpr int kGroups = 2;     // groups of a CTA
+constexpr int kGroup = 256;    // threads of a group: two warps per tensor-memory lane quadrant
+constexpr int kThreads = kGroups * kGroup;
+constexpr int kColsPerWarp = kHid * 4 / (kGroup / 32);     // epilogue columns of a warp
+constexpr int kTmemCols = 256; // a group's: [0, 128) hidden accumulator, [128, 144) outputs
 
 // byte offset of element (r, k) of an operand with K columns
 __host__ __device__ constexpr int cm_off(int r, int k, int K) {
@@ -74,20 +79,18 @@ __device__ __forceinline__ float erf_sqrt2(float v) {
     return x * p;
 }
 
-// GELU of two values, v (1 + erf(v/sqrt 2))/2, with erf(v/sqrt 2) from the
+// GELU of two values, v (1/2 + erf(v/sqrt 2)/2), with erf(v/sqrt 2) from the
 // odd polynomial v Q(v^2) of erf_poly.h (v clamped to [-3 sqrt 2, 3 sqrt 2],
-// error <= 1e-4, below the bfloat16 rounding the epilogue applies) evaluated
-// on the pair by packed multiply-adds (fma.rn.f32x2): one instruction for
-// both values.
+// error <= 1e-4, below the bfloat16 rounding the epilogue applies; the halves
+// of its coefficients are exact) evaluated on the pair by packed multiply-adds
+// (fma.rn.f32x2): one instruction for both values.
 __device__ __forceinline__ float2 gelu2(float2 v) {
     const float2 x = make_float2(fminf(fmaxf(v.x, -kErfClamp), kErfClamp), fminf(fmaxf(v.y, -kErfClamp), kErfClamp));
     const float2 z = __fmul2_rn(x, x);
-    float2 p = make_float2(erf_poly(kErfTerms - 1), erf_poly(kErfTerms - 1));
+    float2 p = make_float2(0.5f * erf_poly(kErfTerms - 1), 0.5f * erf_poly(kErfTerms - 1));
 #pragma unroll
-    for (int k = kErfTerms - 2; k >= 0; --k) p = __ffma2_rn(p, z, make_float2(erf_poly(k), erf_poly(k)));
-    const float2 e = __fmul2_rn(x, p);                                   // erf(v/sqrt 2)
-    const float2 h = __fmul2_rn(v, make_float2(0.5f, 0.5f));
-    return __ffma2_rn(h, e, h);                                           // v/2 + v/2 erf
+    for (int k = kErfTerms - 2; k >= 0; --k) p = __ffma2_rn(p, z, make_float2(0.5f * erf_poly(k), 0.5f * erf_poly(k)));
+    return __fmul2_rn(v, __ffma2_rn(x, p, make_float2(0.5f, 0.5f)));
 }
 
 // ---- tcgen05 plumbing
@@ -114,13 +117,31 @@ struct Tc {
     uint32_t ncols;    // allocated columns
 };
 
-// All threads: mbarrier init (thread 0), allocation of ncols tensor-memory
-// columns (warp 0; a power of two >= 32).  slot and bar are shared-memory
-// words of the CTA.
-__device__ __forceinline__ Tc tc_begin(uint32_t *slot, uint64_t *bar, uint32_t ncols = kTmemCols) {
+// A group of a CTA: its threads, named barrier and tensor-core state (tmem and
+// mbar its own)
+struct Group {
+    int tid;           // thread within the group
+    uint32_t bar;      // named barrier
+    Tc tc;
+    // every thread of the group; false on all where any came with !ok
+    __device__ __forceinline__ bool sync(bool ok) const {
+        uint32_t all;
+        asm volatile(
+            "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.and.pred q, %2, %3, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+            : "=r"(all)
+            : "r"((uint32_t)ok), "r"(bar), "n"(kGroup)
+            : "memory");
+        return all != 0;
+    }
+};
+
+// All threads: initialisation of n mbarriers (thread 0), allocation of ncols
+// tensor-memory columns (warp 0; a power of two >= 32).  slot and bar are
+// shared-memory words of the CTA.
+__device__ __forceinline__ Tc tc_begin(uint32_t *slot, uint64_t *bar, uint32_t ncols, int n = 1) {
     const int tid = threadIdx.x;
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)));
+        for (int k = 0; k < n; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar + k)));
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if ((tid >> 5) == 0) {
@@ -139,6 +160,19 @@ __device__ __forceinline__ Tc tc_begin(uint32_t *slot, uint64_t *bar, uint32_t n
     return t;
 }
 
+// The group of this thread, of a CTA of blockDim.x / kGroup groups (bar: one
+// mbarrier each; the CTA's allocation is kTmemCols columns each)
+__device__ __forceinline__ Group group_begin(uint32_t *slot, uint64_t *bar) {
+    const int n = (int)blockDim.x / kGroup, g = (int)threadIdx.x / kGroup;
+    Group r;
+    r.tid = (int)threadIdx.x % kGroup;
+    r.bar = 1u + (uint32_t)g;
+    r.tc = tc_begin(slot, bar, (uint32_t)(n * kTmemCols), n);
+    r.tc.tmem += (uint32_t)(g * kTmemCols);
+    r.tc.mbar += (uint32_t)(g * 8);
+    return r;
+}
+
 // All threads, after the last use: warp 0 frees the tensor memory.
 __device__ __forceinline__ void tc_end(const Tc &t) {
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -148,13 +182,21 @@ __device__ __forceinline__ void tc_end(const Tc &t) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(t.tmem), "r"(t.ncols));
 }
 
-// One layer's MMAs, D[:, col..col+N) = A[128][K] B[N][K]^T, issued by thread
-// 0 after the other threads' shared-memory writes (fenced for the async
+// All threads of the CTA, after its groups' last use
+__device__ __forceinline__ void group_end(const Group &g) {
+    Tc t = g.tc;
+    t.tmem -= (threadIdx.x / kGroup) * kTmemCols;
+    tc_end(t);
+}
+
+// One layer's MMAs, D[:, col..col+N) = A[128][K] B[N][K]^T, issued by the
+// group's thread 0 after the other threads' shared-memory writes (fenced for the async
 // proxy and synchronised by the caller), then committed to the mbarrier.
 // withhold (fault injection): issue nothing, so the wait runs out.
-__device__ __forceinline__ void tc_layer(const Tc &t, uint32_t a, uint32_t b, int K, int N, uint32_t col,
+__device__ __forceinline__ void tc_layer(const Group &g, uint32_t a, uint32_t b, int K, int N, uint32_t col,
                                          bool withhold = false) {
-    if (threadIdx.x == 0 && !withhold) {
+    const Tc &t = g.tc;
+    if (g.tid == 0 && !withhold) {
         asm volatile("tcgen05.fence::after_thread_sync;");
         const uint32_t sbo = (uint32_t)(K / 8) * 128;
         const uint32_t id = instr_desc(kRows, N);
@@ -205,81 +247,96 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&v)[16]) {
     for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
+__device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
+        "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;");
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t *>(&h);
 }
 
 // Epilogue of a hidden layer: bias + GELU of the accumulator, bfloat16, into
-// the A tile H ([128][128], operand layout); then fenced for the next MMA.
-__device__ __forceinline__ void tc_store_gelu(const Tc &t, const float *bias, unsigned char *H) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// the A tile H ([128][128], operand layout); fenced for the next MMA.
+__device__ __forceinline__ void tc_store_gelu(const Group &g, const float *bias, unsigned char *H) {
+    const int warp = g.tid >> 5, lane = g.tid & 31;
     const int row = 32 * (warp & 3) + lane;
     const int c0 = kColsPerWarp * (warp >> 2);
-    const uint32_t base = t.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
+    const uint32_t base = g.tc.tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
+    unsigned char *h = H + cm_off(row, c0, kHid);
+#pragma unroll 1
+    for (int cc = 0; cc < kColsPerWarp; cc += 32) {
+        uint32_t v[32];
+        tmem_ld32(base + (uint32_t)cc, v);
 #pragma unroll
-    for (int cc = 0; cc < kColsPerWarp; cc += 16) {
-        float v[16];
-        tmem_ld16(base + (uint32_t)cc, v);
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int c = c0 + cc + 8 * half;
-            // the eight columns' biases (16-byte aligned: the blob's bias block is)
-            const float4 b0 = *reinterpret_cast<const float4 *>(bias + c);
-            const float4 b1 = *reinterpret_cast<const float4 *>(bias + c + 4);
-            const float *u = v + 8 * half;
-            const float2 g0 = gelu2(__fadd2_rn(make_float2(u[0], u[1]), make_float2(b0.x, b0.y)));
-            const float2 g1 = gelu2(__fadd2_rn(make_float2(u[2], u[3]), make_float2(b0.z, b0.w)));
-            const float2 g2 = gelu2(__fadd2_rn(make_float2(u[4], u[5]), make_float2(b1.x, b1.y)));
-            const float2 g3 = gelu2(__fadd2_rn(make_float2(u[6], u[7]), make_float2(b1.z, b1.w)));
+        for (int q = 0; q < 4; ++q) {
+            // eight columns' biases (16-byte aligned: the blob's bias block is)
+            const float4 b0 = *reinterpret_cast<const float4 *>(bias + c0 + cc + 8 * q);
+            const float4 b1 = *reinterpret_cast<const float4 *>(bias + c0 + cc + 8 * q + 4);
+            auto act = [&](int k, float x, float y) {
+                const float2 u = make_float2(__uint_as_float(v[8 * q + k]), __uint_as_float(v[8 * q + k + 1]));
+                const float2 a = gelu2(__fadd2_rn(u, make_float2(x, y)));
+                return pack_bf16(a.x, a.y);
+            };
             uint4 w;
-            w.x = pack_bf16(g0.x, g0.y);
-            w.y = pack_bf16(g1.x, g1.y);
-            w.z = pack_bf16(g2.x, g2.y);
-            w.w = pack_bf16(g3.x, g3.y);
-            *reinterpret_cast<uint4 *>(H + cm_off(row, c, kHid)) = w;
+            w.x = act(0, b0.x, b0.y);
+            w.y = act(2, b0.z, b0.w);
+            w.z = act(4, b1.x, b1.y);
+            w.w = act(6, b1.z, b1.w);
+            *reinterpret_cast<uint4 *>(h + cm_off(0, cc + 8 * q, kHid)) = w;
         }
     }
     asm volatile("fence.proxy.async.shared::cta;");
     asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
 }
 
-// The whole network on one 128-row tile.  X0: the features in operand layout
-// ([128][16], columns 6..15 zero), written and synchronised by the caller
-// (fence.proxy.async by the writers, then __syncthreads); H: the hidden tile;
-// out[row * 2 + {0, 1}] = (shift, ls).  All kThreads threads; returns false on
-// all threads if an MMA never completed (the tile's outputs are then invalid
-// and the caller must stop).  withhold: fault injection (see tc_layer).
-__device__ __forceinline__ bool tile_forward(Tc &t, const unsigned char *blob, const unsigned char *X0,
-                                             unsigned char *H, float *out, bool withhold = false) {
+// The whole network on the group's 128-row tile.  X0: the features in operand
+// layout ([128][16], columns 6..15 zero), written by the caller's threads; H: the
+// hidden tile.  (sh, ls) = outputs of row tid on the group's first 128 threads.
+// All threads of the group.  A thread whose MMA never completed clears its ok and
+// goes on to the group's next barrier (a layer on the sums of an unfinished MMA
+// computes what is thrown away); from there all return false, and the caller stops
+// (after the last tile: sync(ok)).  withhold: fault injection (see tc_layer).
+__device__ __forceinline__ bool tile_forward(Group &g, const unsigned char *blob, const unsigned char *X0,
+                                             unsigned char *H, float &sh, float &ls, bool &ok, bool withhold = false) {
     const float *B = reinterpret_cast<const float *>(blob + kOffB);
-    const uint32_t sb = smem_u32(blob), sx = smem_u32(X0), sh = smem_u32(H);
-    // each wait's outcome agreed by the whole CTA before the epilogue reads
-    tc_layer(t, sx, sb + kOffW1, kK1, kHid, 0, withhold);
-    if (!__syncthreads_and(tc_wait(t) ? 1 : 0)) return false;
-    tc_store_gelu(t, B, H);
-    tc_layer(t, sh, sb + kOffW2, kHid, kHid, 0);
-    if (!__syncthreads_and(tc_wait(t) ? 1 : 0)) return false;
-    tc_store_gelu(t, B + kHid, H);
-    tc_layer(t, sh, sb + kOffW3, kHid, kHid, 0);
-    if (!__syncthreads_and(tc_wait(t) ? 1 : 0)) return false;
-    tc_store_gelu(t, B + 2 * kHid, H);
-    tc_layer(t, sh, sb + kOffW4, kHid, kNOut, kHid);
-    if (!__syncthreads_and(tc_wait(t) ? 1 : 0)) return false;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp < 4) {   // the output columns of the warp's 32 rows
+    const uint32_t sb = smem_u32(blob), sx = smem_u32(X0), ah = smem_u32(H);
+    asm volatile("fence.proxy.async.shared::cta;");
+    if (!g.sync(ok)) return false;
+    tc_layer(g, sx, sb + kOffW1, kK1, kHid, 0, withhold);
+    ok = tc_wait(g.tc);
+    tc_store_gelu(g, B, H);
+    if (!g.sync(ok)) return false;
+    tc_layer(g, ah, sb + kOffW2, kHid, kHid, 0);
+    ok = tc_wait(g.tc);
+    tc_store_gelu(g, B + kHid, H);
+    if (!g.sync(ok)) return false;
+    tc_layer(g, ah, sb + kOffW3, kHid, kHid, 0);
+    ok = tc_wait(g.tc);
+    tc_store_gelu(g, B + 2 * kHid, H);
+    if (!g.sync(ok)) return false;
+    tc_layer(g, ah, sb + kOffW4, kHid, kNOut, kHid);
+    if (g.tid < kRows) {   // the other threads' next wait comes after a barrier that these reach later
+        ok = tc_wait(g.tc);
         uint32_t r0, r1;
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];"
                      : "=r"(r0), "=r"(r1)
-                     : "r"(t.tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)kHid));
+                     : "r"(g.tc.tmem + ((uint32_t)(g.tid & ~31) << 16) + (uint32_t)kHid));
         asm volatile("tcgen05.wait::ld.sync.aligned;");
-        const int row = 32 * warp + lane;
-        out[2 * row] = __uint_as_float(r0) + B[3 * kHid];
-        out[2 * row + 1] = __uint_as_float(r1) + B[3 * kHid + 1];
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        sh = __uint_as_float(r0) + B[3 * kHid];
+        ls = __uint_as_float(r1) + B[3 * kHid + 1];
+    } else {
+        g.tc.phase ^= 1u;
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
     return true;
 }
 

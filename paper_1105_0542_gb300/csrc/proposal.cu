@@ -1,7 +1,7 @@
 // The learned bisection proposal on the device (single-precision path).
 //
-// proposal_kernel -- 128 paths per work item, one per thread of the first
-// four warps; all eight warps evaluate the network.  For bisection level
+// proposal_kernel -- 128 paths per work item of a group of eight warps (mlp.cuh),
+// one per thread of the first four; all eight evaluate the network.  For bisection level
 // n = 1..S and midpoint index i, the 128 paths' features
 // (a, b, T, n/S, q_L, q_R) form one 128-row tile; the network gives every
 // path (shift, ls); the path's thread draws its normal z (the plain
@@ -81,9 +81,7 @@ using mlp::kX0Bytes;
 using mlp::kHBytes;
 using mlp::kRows;
 using mlp::kIn;
-using mlp::Tc;
 using mlp::tile_forward;
-constexpr int kT = mlp::kThreads;
 
 __device__ __forceinline__ void copy16(void *dst, const void *src, int bytes, int tid, int nth) {
     const uint4 *s = reinterpret_cast<const uint4 *>(src);
@@ -91,7 +89,11 @@ __device__ __forceinline__ void copy16(void *dst, const void *src, int bytes, in
     for (int i = tid; i < bytes / 16; i += nth) d[i] = s[i];
 }
 
-// shared memory: blob | X0 | H | out[128][2] | qs[(N+1)][128] | tab[S][M] | sig[11] | corr[S+1][128] | sw[S][128]
+// shared memory: blob | tab[S][M] (+ pad) | sig[16] | per group: X0 | H | qs[(N+1)][128] | corr[S+1][128];
+// the levels' weights sw[S][128] in H once the network is done with it
+size_t group_bytes(int S) { return kX0Bytes + kHBytes + (size_t)((1 << S) + S + 2) * kRows * 4; }
+size_t shared_bytes(const SamplerParams &P) { return kBlobBytes + (size_t)(P.S * P.M + 3) / 4 * 16 + 16 * 4; }
+
 template <int RING>
 __global__ void __launch_bounds__(mlp::kThreads, 1) proposal_kernel(const __grid_constant__ ProposalParams Q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -99,53 +101,49 @@ __global__ void __launch_bounds__(mlp::kThreads, 1) proposal_kernel(const __grid
     const int tid = threadIdx.x;
     const int S = P.S, N = 1 << S, L = P.levels;
     __shared__ uint32_t tmem_slot;
-    __shared__ __align__(8) uint64_t mma_bar;
+    __shared__ __align__(8) uint64_t mma_bar[mlp::kGroups];
+    const int group = tid / mlp::kGroup;
     unsigned char *blob = smem_raw;
-    size_t off = kBlobBytes;
-    unsigned char *X0 = smem_raw + off;
-    off += kX0Bytes;
-    unsigned char *H = smem_raw + off;
-    off += kHBytes;
-    float *out = reinterpret_cast<float *>(smem_raw + off);
-    off += kRows * 2 * 4;
-    float *qs = reinterpret_cast<float *>(smem_raw + off);
-    off += (size_t)(N + 1) * kRows * 4;
-    float *tab = reinterpret_cast<float *>(smem_raw + off);
-    off += (size_t)S * P.M * 4;
-    float *sig = reinterpret_cast<float *>(smem_raw + off);
-    off += 16 * 4;
-    float *corr = reinterpret_cast<float *>(smem_raw + off);
-    off += (size_t)(S + 1) * kRows * 4;
-    float *sw = reinterpret_cast<float *>(smem_raw + off);
+    float *tab = reinterpret_cast<float *>(smem_raw + kBlobBytes);
+    float *sig = tab + (S * P.M + 3) / 4 * 4;
+    unsigned char *own = reinterpret_cast<unsigned char *>(sig + 16) +
+                         (size_t)group * (kX0Bytes + kHBytes + (size_t)(N + S + 2) * kRows * 4);
+    unsigned char *X0 = own, *H = X0 + kX0Bytes;
+    float *qs = reinterpret_cast<float *>(H + kHBytes);
+    float *corr = qs + (size_t)(N + 1) * kRows;
+    float *sw = reinterpret_cast<float *>(H);
 
-    copy16(blob, Q.blob, kBlobBytes, tid, kT);
+    copy16(blob, Q.blob, kBlobBytes, tid, blockDim.x);
     {
         const float *g = reinterpret_cast<const float *>(P.tables);
-        for (int i = tid; i < S * P.M; i += kT) tab[i] = g[i];
-        for (int i = tid; i <= SU_MAX_S; i += kT) sig[i] = (float)P.sigma[i];
-        for (int i = tid; i < kX0Bytes / 16; i += kT) reinterpret_cast<uint4 *>(X0)[i] = make_uint4(0, 0, 0, 0);
+        for (int i = tid; i < S * P.M; i += blockDim.x) tab[i] = g[i];
+        for (int i = tid; i <= SU_MAX_S; i += blockDim.x) sig[i] = (float)P.sigma[i];
+        for (int i = tid % mlp::kGroup; i < kX0Bytes / 16; i += mlp::kGroup)
+            reinterpret_cast<uint4 *>(X0)[i] = make_uint4(0, 0, 0, 0);
     }
-    Tc tc = mlp::tc_begin(&tmem_slot, &mma_bar);   // contains __syncthreads
-    bool alive = true;
+    mlp::Group gr = mlp::group_begin(&tmem_slot, mma_bar);   // contains __syncthreads
+    bool alive = true, ok = true;   // alive: the same for the whole group
 
     const float fa = (float)P.a, fb = (float)P.b, fT = (float)Q.T;
     const __nv_bfloat16 ba = __float2bfloat16_rn(fa), bb = __float2bfloat16_rn(fb), bT = __float2bfloat16_rn(fT);
     const float alpha = (float)P.alpha;
-    const int warp = tid >> 5, lane = tid & 31;
-    const bool owner = tid < kRows;
+    const int p = gr.tid, warp = p >> 5, lane = p & 31;
+    const bool owner = p < kRows;
     Stream<float> st;
     st.key = make_uint2((uint32_t)P.seed, (uint32_t)(P.seed >> 32));
     st.inst = P.instance;
     st.bm = nullptr;
 
-    for (int64_t item = blockIdx.x; alive && item < P.n_items; item += gridDim.x) {
+    // the groups run on their own; a grid of at most n_items CTAs gives every one work
+    const int groups = (int)blockDim.x / mlp::kGroup;
+    for (int64_t item = blockIdx.x + (int64_t)group * gridDim.x; alive && item < P.n_items;
+         item += (int64_t)groups * gridDim.x) {
         const int64_t bk = item / P.items_per_block;
         const int64_t r = item - bk * P.items_per_block;
         const int64_t lo = bk * P.n_mc / P.n_blocks;
         const int64_t hi = (bk + 1) * P.n_mc / P.n_blocks;
         const int64_t start = lo + r * kRows;
         const int cnt = (int)max((int64_t)0, min((int64_t)kRows, hi - start));
-        const int p = tid;
         const bool valid = owner && p < cnt;
         float quad[4] = {0.f, 0.f, 0.f, 0.f}, c = 0.f;
         if (owner) {
@@ -164,20 +162,14 @@ __global__ void __launch_bounds__(mlp::kThreads, 1) proposal_kernel(const __grid
                 if (owner)
                     mlp::store_features(X0, p, ba, bb, bT, bn, __float2bfloat16_rn(qs[kL * kRows + p]),
                                         __float2bfloat16_rn(qs[kR * kRows + p]));
-                asm volatile("fence.proxy.async.shared::cta;");
-                __syncthreads();
-                if (!tile_forward(tc, blob, X0, H, out, Q.withhold != 0)) {
-                    if (tid == 0) atomicOr(P.flags, 4);   // an MMA never completed
-                    alive = false;
-                    break;
-                }
+                float sh = 0.f, ls = 0.f;
+                if (!(alive = tile_forward(gr, blob, X0, H, sh, ls, ok, Q.withhold != 0))) break;
                 if (owner) {
                     const uint32_t j = (1u << (n - 1)) - 1u + (uint32_t)i;
                     // the plain single-precision stream: slot j' & 3 of call j' >> 2, j' = j + 1
                     const uint32_t jp = j + 1;
                     if (j == 0 || (jp & 3u) == 0) st.quad(jp >> 2, quad);
                     const float z = pick4(quad, jp);
-                    const float sh = out[2 * p], ls = out[2 * p + 1];
                     const float t = fmaf(__expf(ls), z, sh);
                     const float mid = 0.5f * (qs[kL * kRows + p] + qs[kR * kRows + p]);
                     qs[kM * kRows + p] = fmaf(sig[n], t, mid);
@@ -191,7 +183,7 @@ __global__ void __launch_bounds__(mlp::kThreads, 1) proposal_kernel(const __grid
             }
             if (owner) corr[n * kRows + p] = c;
         }
-        if (!alive) break;
+        if (!alive || !(alive = gr.sync(ok))) break;
         // W_p on every level of the path, plus the proposal weight
         if (owner) {
             for (int d = 0; d < L; ++d) {
@@ -207,9 +199,9 @@ __global__ void __launch_bounds__(mlp::kThreads, 1) proposal_kernel(const __grid
                 if (valid && P.w_out) P.w_out[(start + p) * (int64_t)S + (n - 1)] = (double)w;
             }
         }
-        __syncthreads();
+        gr.sync(true);
         if (!P.w_out) {
-            for (int d = warp; d < L; d += kT / 32) {
+            for (int d = warp; d < L; d += mlp::kGroup / 32) {
                 const float *v = sw + d * kRows;
                 float m = -INFINITY;
                 for (int t = lane; t < cnt; t += 32) m = fmaxf(m, v[t]);
@@ -233,9 +225,10 @@ __global__ void __launch_bounds__(mlp::kThreads, 1) proposal_kernel(const __grid
                 }
             }
         }
-        __syncthreads();
+        gr.sync(true);
     }
-    mlp::tc_end(tc);
+    if (!alive && p == 0) atomicOr(P.flags, 4);   // an MMA never completed
+    mlp::group_end(gr);
 }
 
 // rows of features X (n x 6 floats) -> Y (n x 2); a tile whose MMAs never
@@ -245,35 +238,34 @@ __global__ void __launch_bounds__(mlp::kThreads, 1) mlp_forward_kernel(const uns
                                                                        float *Y) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t tmem_slot;
-    __shared__ __align__(8) uint64_t mma_bar;
+    __shared__ __align__(8) uint64_t mma_bar[mlp::kGroups];
     unsigned char *blob = smem_raw;
-    unsigned char *X0 = smem_raw + kBlobBytes;
-    unsigned char *H = smem_raw + kBlobBytes + kX0Bytes;
-    float *out = reinterpret_cast<float *>(smem_raw + kBlobBytes + kX0Bytes + kHBytes);
-    const int tid = threadIdx.x;
-    copy16(blob, gblob, kBlobBytes, tid, kT);
-    for (int i = tid; i < kX0Bytes / 16; i += kT) reinterpret_cast<uint4 *>(X0)[i] = make_uint4(0, 0, 0, 0);
-    Tc tc = mlp::tc_begin(&tmem_slot, &mma_bar);
-    for (int64_t t0 = (int64_t)blockIdx.x * kRows; t0 < n; t0 += (int64_t)gridDim.x * kRows) {
-        if (tid < kRows) {
-            const int64_t r = t0 + tid;
+    const int tid = threadIdx.x, group = tid / mlp::kGroup;
+    unsigned char *X0 = smem_raw + kBlobBytes + group * (kX0Bytes + kHBytes);
+    unsigned char *H = X0 + kX0Bytes;
+    copy16(blob, gblob, kBlobBytes, tid, blockDim.x);
+    for (int i = tid % mlp::kGroup; i < kX0Bytes / 16; i += mlp::kGroup)
+        reinterpret_cast<uint4 *>(X0)[i] = make_uint4(0, 0, 0, 0);
+    mlp::Group gr = mlp::group_begin(&tmem_slot, mma_bar);
+    const int64_t stride = (int64_t)gridDim.x * kRows;
+    bool alive = true, ok = true;
+    for (int64_t t0 = (int64_t)blockIdx.x * kRows + group * stride; alive && t0 < n; t0 += mlp::kGroups * stride) {
+        const int64_t r = t0 + gr.tid;
+        if (gr.tid < kRows) {
             float f[kIn];
             for (int c = 0; c < kIn; ++c) f[c] = r < n ? X[r * kIn + c] : 0.f;
-            mlp::store_features(X0, tid, __float2bfloat16_rn(f[0]), __float2bfloat16_rn(f[1]),
+            mlp::store_features(X0, gr.tid, __float2bfloat16_rn(f[0]), __float2bfloat16_rn(f[1]),
                                 __float2bfloat16_rn(f[2]), __float2bfloat16_rn(f[3]), __float2bfloat16_rn(f[4]),
                                 __float2bfloat16_rn(f[5]));
         }
-        asm volatile("fence.proxy.async.shared::cta;");
-        __syncthreads();
-        const bool ok = tile_forward(tc, blob, X0, H, out);
-        if (tid < kRows && t0 + tid < n) {
-            Y[(t0 + tid) * 2] = ok ? out[2 * tid] : NAN;
-            Y[(t0 + tid) * 2 + 1] = ok ? out[2 * tid + 1] : NAN;
+        float sh, ls;
+        alive = tile_forward(gr, blob, X0, H, sh, ls, ok);
+        if (gr.tid < kRows && r < n) {
+            Y[r * 2] = alive && ok ? sh : NAN;
+            Y[r * 2 + 1] = alive && ok ? ls : NAN;
         }
-        __syncthreads();
-        if (!ok) break;
     }
-    mlp::tc_end(tc);
+    mlp::group_end(gr);
 }
 
 const void *proposal_fn(int ring) {
@@ -290,15 +282,14 @@ cudaError_t allow_smem(const void *fn, size_t smem) {
 
 }  // namespace
 
+// two groups' tiles where they fit, else one's
+static int proposal_groups(const ProposalParams &Q) {
+    const size_t most = 227 * 1024 - 64;   // of a CTA, with the static words
+    return shared_bytes(Q.base) + mlp::kGroups * group_bytes(Q.base.S) <= most ? mlp::kGroups : 1;
+}
+
 size_t proposal_smem_bytes(const ProposalParams &Q) {
-    const SamplerParams &P = Q.base;
-    const int N = 1 << P.S;
-    size_t off = mlp::kBlobBytes + mlp::kX0Bytes + mlp::kHBytes + mlp::kRows * 2 * 4;
-    off += (size_t)(N + 1) * mlp::kRows * 4;
-    off += (size_t)P.S * P.M * 4 + 16 * 4;
-    off += (size_t)(P.S + 1) * mlp::kRows * 4;
-    off += (size_t)P.S * mlp::kRows * 4;
-    return off;
+    return shared_bytes(Q.base) + proposal_groups(Q) * group_bytes(Q.base.S);
 }
 
 int proposal_occupancy(const ProposalParams &Q, size_t smem) {
@@ -308,7 +299,7 @@ int proposal_occupancy(const ProposalParams &Q, size_t smem) {
         return 0;
     }
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, mlp::kThreads, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, proposal_groups(Q) * mlp::kGroup, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -321,12 +312,12 @@ cudaError_t launch_proposal(const ProposalParams &Q, int grid, size_t smem, cuda
     cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     void *args[] = {const_cast<ProposalParams *>(&Q)};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(mlp::kThreads), args, smem, st);
+    return cudaLaunchKernel(fn, dim3(grid), dim3(proposal_groups(Q) * mlp::kGroup), args, smem, st);
 }
 
 cudaError_t launch_mlp_forward(const unsigned char *blob, const float *X, int64_t n, float *Y, int sms,
                                cudaStream_t st) {
-    const size_t smem = mlp::kBlobBytes + mlp::kX0Bytes + mlp::kHBytes + mlp::kRows * 2 * 4;
+    const size_t smem = mlp::kBlobBytes + mlp::kGroups * (mlp::kX0Bytes + mlp::kHBytes);
     cudaGetLastError();
     cudaError_t e = allow_smem((const void *)mlp_forward_kernel, smem);
     if (e != cudaSuccess) return e;
