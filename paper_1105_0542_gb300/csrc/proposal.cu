@@ -1,7 +1,7 @@
 // The learned bisection proposal on the device (single-precision path).
 //
-// proposal_kernel -- 128 paths per work item of a group of eight warps (mlp.cuh),
-// one per thread of the first four; all eight evaluate the network.  For bisection level
+// proposal_kernel -- 128 paths per work item of a group of sixteen warps (mlp.cuh),
+// one per thread of the first four; all evaluate the network.  For bisection level
 // n = 1..S and midpoint index i, the 128 paths' features
 // (a, b, T, n/S, q_L, q_R) form one 128-row tile; the network gives every
 // path (shift, ls); the path's thread draws its normal z (the plain
