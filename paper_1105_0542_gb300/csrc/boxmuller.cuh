@@ -16,39 +16,55 @@
 // (a 49-node logarithm, quadrant-reduced 33-node sin/cos), were a few units
 // in the last place accurate but cost about 55 instructions per pair, the
 // largest item of the issue-bound single-precision sampler after the W_p
-// Horner; this one costs about 25.
+// Horner; this one costs about 25, and with two pairs side by side in packed
+// operations about 18 (the anharmonic oscillator's 48 x 48 amplitude matrix at p = 10, 54.0 ->
+// 52.2 ms; the anharmonic oscillator at p = 18, N = 1024, 17.5 -> 17.2 ms).
 #include <cstdint>
 
 namespace su {
 namespace bm32 {
 
-// z0 = R cos(2 pi u2), z1 = R sin(2 pi u2), R = sqrt(-2 ln u1)
-__device__ __forceinline__ void pair(uint32_t a, uint32_t b, float &z0, float &z1) {
+// z[0], z[1] = R cos(2 pi u2), R sin(2 pi u2), R = sqrt(-2 ln u1), of the words
+// w.x, w.y, and z[2], z[3] of w.z, w.w.  Both pairs at once: a packed operation
+// occupies the two FMA pipes of a scheduler for as long as a single one holds up
+// the packed Horner of W_p beside it.  The approximations in their ftz forms, with
+// no code for subnormal arguments (u1 >= 2^-25, v = 0 or >= 2^-24).
+__device__ __forceinline__ void quad(uint4 w, float (&z)[4]) {
+    auto both = [](float c) { return make_float2(c, c); };
     // ((w >> 8) + 1/2) 2^-24 in one rounding: the scaling is exact
-    const float u1 = fmaf((float)(a >> 8), 0x1p-24f, 0x1p-25f);
-    const float u2 = fmaf((float)(b >> 8), 0x1p-24f, 0x1p-25f);
+    const float2 u1 = __ffma2_rn(make_float2((float)(w.x >> 8), (float)(w.z >> 8)), both(0x1p-24f), both(0x1p-25f));
+    const float2 u2 = __ffma2_rn(make_float2((float)(w.y >> 8), (float)(w.w >> 8)), both(0x1p-24f), both(0x1p-25f));
 
-    // ---- v = -2 ln u1
-    const float t = 1.0f - u1;
-    float lg;
-    asm("lg2.approx.f32 %0, %1;" : "=f"(lg) : "f"(u1));
-    float ser = fmaf(t, 1.0f / 7.0f, 1.0f / 6.0f);
-    ser = fmaf(t, ser, 0.2f);
-    ser = fmaf(t, ser, 0.25f);
-    ser = fmaf(t, ser, 0.333333343f);
-    ser = fmaf(t, ser, 0.5f);
-    ser = fmaf(t, ser, 1.0f);
-    const float v = t < 0.0625f ? 2.0f * t * ser : -1.38629436f * lg;   // -2 ln 2 = -1.38629436
+    // ---- v = -2 ln u1; the series with its coefficients doubled
+    const float2 t = __ffma2_rn(u1, both(-1.0f), both(1.0f));
+    float2 ser = __ffma2_rn(t, both(2.0f / 7.0f), both(2.0f / 6.0f));
+    ser = __ffma2_rn(t, ser, both(0.4f));
+    ser = __ffma2_rn(t, ser, both(0.5f));
+    ser = __ffma2_rn(t, ser, both(2.0f * 0.333333343f));
+    ser = __ffma2_rn(t, ser, both(1.0f));
+    ser = __ffma2_rn(t, ser, both(2.0f));
+    const float2 near = __fmul2_rn(t, ser);
+    float2 lg;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg.x) : "f"(u1.x));
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg.y) : "f"(u1.y));
+    const float2 far = __fmul2_rn(lg, both(-1.38629436f));   // -2 ln 2
+    const float va = t.x < 0.0625f ? near.x : far.x, vb = t.y < 0.0625f ? near.y : far.y;
 
     // ---- R = sqrt(v), v in {0} u [2^-24, 35]
-    float R;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(R) : "f"(v));
+    float Ra, Rb;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(Ra) : "f"(va));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(Rb) : "f"(vb));
 
     // ---- cos, sin of 2 pi u2
-    float sn, cs;
-    __sincosf(6.28318530718f * (u2 - 0.5f), &sn, &cs);
-    z0 = -R * cs;
-    z1 = -R * sn;
+    const float2 x = __fmul2_rn(__fadd2_rn(u2, both(-0.5f)), both(6.28318530718f));
+    float2 ca, cb;   // (cos, sin)
+    __sincosf(x.x, &ca.y, &ca.x);
+    __sincosf(x.y, &cb.y, &cb.x);
+    const float2 za = __fmul2_rn(ca, both(-Ra)), zb = __fmul2_rn(cb, both(-Rb));
+    z[0] = za.x;
+    z[1] = za.y;
+    z[2] = zb.x;
+    z[3] = zb.y;
 }
 
 }  // namespace bm32

@@ -73,8 +73,7 @@ struct Normal<float> {
     // ((w >> 8) + 1/2) 2^-24 of (w0, w1), (z2, z3) from (w2, w3), through the
     // single-precision routine of boxmuller.cuh (hardware approximations)
     static __device__ __forceinline__ void quad(uint4 w, float (&z)[4]) {
-        bm32::pair(w.x, w.y, z[0], z[1]);
-        bm32::pair(w.z, w.w, z[2], z[3]);
+        bm32::quad(w, z);
     }
 };
 
