@@ -762,6 +762,7 @@ static int configure_nd(su_plan &pl) {
     const int nv = 2 * pl.nd;
     NdParams &Q = pl.Q;
     std::memset(&Q, 0, sizeof Q);
+    Q.one = 1;
     NdProgram G;
     std::vector<int> every((size_t)M), heads;
     for (int i = 0; i < M; ++i) every[(size_t)i] = i;

@@ -3,6 +3,7 @@
 // level-p effective potential W(x, xb; eps) of a polynomial potential per
 // slice, per-sample log-weights of every level, per-item log-sum-exp tuples.
 #include <cstdint>
+#include <type_traits>
 
 #include "sampler_impl.cuh"
 
@@ -22,7 +23,9 @@ __device__ __forceinline__ void vzero(double &a) { a = 0.0; }
 template <typename VT, int NV, int B>
 struct Vars {
     VT z[NV][B], m[NV][B];
-    __device__ __forceinline__ void close(unsigned sq) {
+    unsigned one;   // 1, not known to the compiler (double)
+    __device__ __forceinline__ void close(unsigned sq, unsigned once) {
+        one = once;
 #pragma unroll
         for (int k = 0; k < NV; ++k)
 #pragma unroll
@@ -30,10 +33,17 @@ struct Vars {
     }
 };
 
+// Steps that only some polynomials have -- the factor z_k, and a Horner chain's
+// multiply-add after the first -- are loops of no or one pass in double, where an
+// operation holds the pipe for 16 cycles: written as conditions the compiler
+// computed both for all and selected (102 double operations a slice, two coordinates
+// at p = 10; 54 now: 47.3 -> 29.7 ms for 100 003 paths of 1024 slices), and kept
+// from that it left them to predicates, which hold the pipe too (37.4 ms).
 // t = the polynomial in z_K.. at w (words) and c (coefficients), both moved past it
 template <int K, typename VT, int NV, int B>
 __device__ __forceinline__ void nd_poly(const uint32_t *__restrict__ &w, const VT *__restrict__ &c,
                                         const Vars<VT, NV, B> &v, VT (&t)[B]) {
+    constexpr bool kSkip = std::is_same<VT, double>::value;
     const uint32_t hd = *w++;
     const int n = (int)(hd & 0xffffu);
     if constexpr (K == NV - 1) {
@@ -58,11 +68,25 @@ __device__ __forceinline__ void nd_poly(const uint32_t *__restrict__ &w, const V
         for (int e = 0; e < n; ++e) {
             VT u[B];
             nd_poly<K + 1>(w, c, v, u);
+            if constexpr (kSkip) {
+#pragma unroll 1
+                for (unsigned o = e ? v.one : 0u; o; --o)
 #pragma unroll
-            for (int i = 0; i < B; ++i) t[i] = vfma(t[i], v.m[K][i], u[i]);
+                    for (int i = 0; i < B; ++i) u[i] = vfma(t[i], v.m[K][i], u[i]);
+#pragma unroll
+                for (int i = 0; i < B; ++i) t[i] = u[i];
+            } else {
+#pragma unroll
+                for (int i = 0; i < B; ++i) t[i] = vfma(t[i], v.m[K][i], u[i]);
+            }
         }
     }
-    if (hd & kNdOdd) {
+    if constexpr (kSkip) {
+#pragma unroll 1
+        for (uint32_t o = hd >> 16; o; --o)   // kNdOdd
+#pragma unroll
+            for (int i = 0; i < B; ++i) t[i] = vmul(t[i], v.z[K][i]);
+    } else if (hd & kNdOdd) {
 #pragma unroll
         for (int i = 0; i < B; ++i) t[i] = vmul(t[i], v.z[K][i]);
     }
@@ -94,7 +118,7 @@ __device__ __forceinline__ float nd_single(const NdParams &Q, const uint32_t *w,
             l = b;
         }
     }
-    v.close(Q.sq);
+    v.close(Q.sq, Q.one);
     float2 t[BP];
     nd_poly<0>(w, c, v, t);
     float s = 0;
@@ -116,7 +140,7 @@ __device__ __forceinline__ double nd_double(const NdParams &Q, unsigned sq, cons
         v.z[k][0] = fma(sg, a, b);
         v.z[k][1] = fma(sg, b, e);
     }
-    v.close(sq);
+    v.close(sq, Q.one);
     double t[2];
     nd_poly<0>(w, c, v, t);
     return t[0] + t[1];
@@ -130,7 +154,8 @@ __device__ __forceinline__ double nd_double(const NdParams &Q, unsigned sq, cons
 //
 // What bounds it.  Single precision: instruction issue, most of it the packed
 // multiply-adds of the nest and the loops around them.  Double: the FP64 pipe
-// (2 lanes a cycle) in the double part, a tenth of the entries on fine levels.
+// (2 lanes a cycle; 58 % busy) in the double part, a tenth of the entries on fine
+// levels, and the latency of its short chains.
 template <typename R, int D>
 __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __grid_constant__ NdParams Q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -259,6 +259,7 @@ struct NdParams {
     unsigned hsq[SU_MAX_S];
     double reach[kNdMaxDim];  // |q_c| beyond which the path is weighed in double
     int staged;               // program and tables in shared memory
+    unsigned one;             // 1
     double a[kNdMaxDim], b[kNdMaxDim];
     void *paths;              // device (double or float): segment endpoint i, coordinate c of slot t
                               // at [(i D + c) pstride + t]
