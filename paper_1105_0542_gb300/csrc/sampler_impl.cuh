@@ -152,37 +152,36 @@ __device__ __forceinline__ void general_derivatives(double x, const GeneralDev *
     const int deg = G->deg;
     for (int j = 0; j <= J; ++j) {
         double v = 0.0;
-        if (j <= deg)
-            for (int i = deg; i >= j; --i) v = fma(v, x, G->poly_der[j][i]);
+        if (j <= deg) {
+            v = G->poly_der[j][deg];
+            for (int i = deg - 1; i >= j; --i) v = fma(v, x, G->poly_der[j][i]);
+        }
         V[j] = v;
     }
     for (int g = 0; g < G->ng; ++g) {
-        const double u = x - G->gauss[g][2], sb = G->gauss[g][3];
-        const double y = sb * u, e = G->gauss[g][0] * exp(-G->gauss[g][1] * u * u);
-        double h0 = 1.0, h1 = 2.0 * y, f = 1.0;
+        // D_n = (d/dx)^n A e^{-beta u^2}: D_{n+1} = -2 beta (u D_n + n D_{n-1})
+        const double u = x - G->gauss[g][2], b2 = -2.0 * G->gauss[g][1], y = b2 * u;
+        double d0 = 0.0, d1 = G->gauss[g][0] * exp(0.5 * y * u), c = 0.0;
         for (int n = 0; n <= J; ++n) {
-            V[n] = fma(f * (n == 0 ? h0 : h1), e, V[n]);
-            f *= -sb;
-            if (n >= 1) {
-                const double h2 = fma(2.0 * y, h1, -2.0 * n * h0);
-                h0 = h1;
-                h1 = h2;
-            }
+            V[n] += d1;
+            const double d2 = fma(y, d1, c * d0);
+            d0 = d1;
+            d1 = d2;
+            c += b2;
         }
     }
     for (int q = 0; q < G->ns; ++q) {
         const double w = G->sech[q][1] * (x - G->sech[q][2]);
         const double em = expm1(-2.0 * fabs(w)), e = exp(-2.0 * fabs(w));
-        const double den = 2.0 + em;               // 1 + e^{-2|w|}
+        const double r = 1.0 / (2.0 + em);         // 1 / (1 + e^{-2|w|})
         double a[kGenMaxSym + 1];
-        a[0] = copysign(-em / den, w);             // tanh w
-        a[1] = 4.0 * e / (den * den);              // sech^2 w
+        a[0] = copysign(-em * r, w);               // tanh w
+        a[1] = 4.0 * e * (r * r);                  // sech^2 w
         V[0] = fma(G->sech_scale[q][0], a[1], V[0]);
         for (int n = 1; n <= J; ++n) {
-            double acc = 0.0;
-            for (int k = 0; k < (n + 1) / 2; ++k) acc = fma(a[k], a[n - k], acc);
-            acc += acc;
-            if (!(n & 1)) acc = fma(a[n >> 1], a[n >> 1], acc);
+            double acc = a[0] * a[n];
+            for (int k = 1; k < (n + 1) / 2; ++k) acc = fma(a[k], a[n - k], acc);
+            acc = (n & 1) ? acc + acc : fma(a[n >> 1], a[n >> 1], acc + acc);
             a[n + 1] = -acc * G->inv[n + 1];
             V[n] = fma(G->sech_scale[q][n], a[n + 1], V[n]);
         }
