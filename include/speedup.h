@@ -111,8 +111,10 @@ typedef struct {
                              In double precision 0 also takes the fixed-point
                              sampler where the ranges of a, b, T and the tables
                              allow it (even polynomial potentials, automatic
-                             segments); 1 never does.  The two agree to a
-                             double's rounding. */
+                             segments), and several-coordinates and general
+                             potentials evaluate the small entries of their
+                             programs in single precision; 1 never does.
+                             They agree to a double's rounding. */
 } su_options;
 
 /* per bisection level n = 0..s (N = 2^n slices) */

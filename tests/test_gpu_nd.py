@@ -196,3 +196,24 @@ def test_nd_edge_cases():
     on = su.speedup_amplitude_nd(V, a, b, T, p, 7, 5000, 9, n_blocks=10)
     off = su.speedup_amplitude_nd(V, a, b, T, p, 7, 5000, 9, n_blocks=10, hierarchy=False)
     assert off[7]["amp"] == on[7]["amp"] and off[7]["err"] == on[7]["err"]
+
+
+@pytest.mark.parametrize("V,a,b,T,p,s", [
+    ({(3,): 0.1, (2,): 0.5}, (0.2,), (-0.4,), 0.5, 5, 3),                          # odd powers
+    ({(2, 0): 0.5, (1, 2): 0.2, (0, 4): 0.1}, (0.0, 0.3), (0.5, 0.0), 0.7, 6, 6),  # odd in one coordinate
+    ({(2, 0): 0.5, (4, 0): 0.2, (0, 2): 1.0}, (0.0, 0.0), (1.0, 0.5), 3.0, 4, 1),  # one step, paths past the reach
+    ({(2, 0, 0): 0.5, (0, 2, 0): 0.5, (0, 0, 2): 0.5, (1, 1, 1): 0.3}, (0.0,) * 3, (0.3,) * 3, 0.5, 5, 7),
+    ({(2, 0, 0, 0): 0.5, (1, 1, 0, 0): 0.2, (0, 0, 2, 2): 0.1}, (0.1,) * 4, (0.2,) * 4, 0.4, 4, 5)])
+def test_split_program_matches_the_whole_program(V, a, b, T, p, s):
+    """The program split by the size of its entries against the whole program in
+    double (kernel="generic") on the same samples, a partial last item: the
+    split's rounding is 2^-55 a level of O(1), both programs' own a few 2^-53 a
+    slice, so 1e-12 of max(1, |w|)."""
+    w = []
+    for kernel in ("auto", "generic"):
+        out = torch.zeros((333, s), dtype=torch.float64, device="cuda")
+        su.speedup_logweights_nd(V, a, b, T, p, s, 3, 333, 41, out, precision="fp64", kernel=kernel)
+        torch.cuda.synchronize()
+        w.append(out.cpu().numpy())
+    assert np.isfinite(w[0]).all()
+    assert np.all(np.abs(w[0] - w[1]) <= 1e-12 * np.maximum(1.0, np.abs(w[1])))
