@@ -615,7 +615,12 @@ static int plan_shape(su_plan &pl, int sms, int smem_max, std::vector<unsigned c
             std::memcpy(blob.data() + P.fx.tail_off, tail.data(), tail.size() * sizeof(float));
         }
     }
-    if (general && prec == SU_FP64 && S >= 1 && !P.wf_on && !P.generic && pl.opt.seg_log2 == 0 && pl.opt.rounds == 0)
+    // the split pays for its preparation (0.1 to 0.3 ms) from some 1.5e8 entries
+    // evaluated (about 0.5 ms as a whole program)
+    constexpr double kSplitLeast = 1.5e8;
+    const double entries = (double)pl.n_mc * ((pl.levels > 1 ? 2.0 : 1.0) * (double)((int64_t)1 << S)) * P.M;
+    if (general && prec == SU_FP64 && S >= 1 && !P.wf_on && !P.generic && pl.opt.seg_log2 == 0 && pl.opt.rounds == 0 &&
+        entries >= kSplitLeast)
         split_general(pl, blob, smem_max);
     // launch shape: one path per thread, persistent grid over items of
     // 128 * rounds samples

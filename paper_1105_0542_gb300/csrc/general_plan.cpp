@@ -17,9 +17,8 @@ namespace su {
 void general_moments(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T,
                      std::vector<double> &ms) {
     const size_t nn = G.depth.size();
-    // fewer positions for the long programs (p > 12)
-    const int times = nn > 800 ? 8 : 16, half = nn > 800 ? 8 : 24;
-    const double dg = 6.0 / half;
+    constexpr int times = 8, half = 8;   // 7 times, 17 positions to 6 standard deviations
+    constexpr double dg = 6.0 / half;
     ms.assign(nn, 0.0);
     std::vector<double> D((size_t)G.J + 1), stk((size_t)G.J + 3 * G.p + 2, 1.0);
     for (int k = 1; k < times; ++k) {
@@ -46,24 +45,43 @@ void general_split(const GeneralEffective &G, const std::vector<double> &ms, dou
     std::vector<double> my((size_t)G.K, 1.0);
     for (int k = 1; k < G.K; ++k) my[(size_t)k] = my[(size_t)k - 1] * s2 * std::sqrt((4.0 * k - 1) * (4.0 * k - 3));
     const size_t nn = G.depth.size();
-    std::vector<std::pair<double, std::pair<int, int>>> r;   // size, (node, power)
+    std::vector<double> size(G.entry_k.size());
     double all = 0;
     for (size_t t = 0; t < nn; ++t)
         for (int k = 0; k < G.count[t]; ++k) {
-            const double v = std::fabs(table[G.first[t] + k]) * ms[t] * my[(size_t)k];
-            r.push_back({v, {(int)t, k}});
-            all += v;
+            const size_t e = (size_t)G.first[t] + (size_t)k;
+            all += size[e] = std::fabs(table[e]) * ms[t] * my[(size_t)k];
         }
-    std::sort(r.begin(), r.end());
-    const double most = 0x1p-33 * std::min(1.0, N * all) / N;
-    double rest = 0;
-    size_t i = 0;
-    for (; i < r.size() && rest + r[i].first <= most; ++i) rest += r[i].first;
-    head.assign(nn, 0);
-    for (; i < r.size(); ++i) {
-        int &h = head[(size_t)r[i].second.first];
-        h = std::max(h, r[i].second.second + 1);
+    if (!std::isfinite(all)) {   // sizes beyond a double: nothing to split by
+        head.assign(G.count.begin(), G.count.end());
+        return;
     }
+    // the smallest entries up to the sum: whole octaves, then the last one's in order
+    const double most = 0x1p-33 * std::min(1.0, N * all) / N;
+    constexpr int kOctaves = 400;
+    auto octave = [](double v) { return v > 0 ? std::max(0, std::min(kOctaves - 1, std::ilogb(v) + 300)) : 0; };
+    std::vector<double> sum(kOctaves, 0.0);
+    for (double v : size) sum[(size_t)octave(v)] += v;
+    double rest = 0;
+    int oct = 0;
+    while (oct < kOctaves && rest + sum[(size_t)oct] <= most) rest += sum[(size_t)oct++];
+    std::vector<double> last;
+    for (double v : size)
+        if (octave(v) == oct) last.push_back(v);
+    std::sort(last.begin(), last.end());
+    double least = 0;   // of the large ones
+    for (double v : last) {
+        least = v;
+        if (rest + v > most) break;
+        rest += v;
+    }
+    head.assign(nn, 0);
+    for (size_t t = 0; t < nn; ++t)
+        for (int k = 0; k < G.count[t]; ++k) {
+            const double v = size[(size_t)G.first[t] + (size_t)k];
+            const int o = octave(v);
+            if (o > oct || (o == oct && v >= least)) head[t] = k + 1;
+        }
 }
 
 }  // namespace su

@@ -197,18 +197,19 @@ def test_morse_amplitude_matches_dvr():
     assert abs(top["amp"] - ref) <= 4 * sig, (top["amp"], ref, sig)
 
 
-@pytest.mark.parametrize("gauss,sech,expo,p,s", [((), (), (), 4, 1), (((1.5, 2.0, 0.3),), ((-1.0, 2.0, 0.0),), (), 10, 6),
-                                                 (((2.0, 80.0, 0.1),), (), (), 7, 8), ((), (), ((3.0, 1.0, 0.0),), 12, 4)])
-def test_split_program_matches_the_whole_program(gauss, sech, expo, p, s):
-    """The split sampler (small entries in single precision) against the whole
-    program in double (kernel="generic") on the same samples, with narrow
-    features, two slices and a partial last item: 1e-12 of the weight, or of its
-    largest terms' scale where they cancel (the weights are O(1) here)."""
+@pytest.mark.parametrize("gauss,sech,expo,p,s,n", [((), (), (), 4, 10, 5003), (((1.5, 2.0, 0.3),), ((-1.0, 2.0, 0.0),), (), 10, 6, 2501),
+                                                   (((2.0, 80.0, 0.1),), (), (), 7, 8, 5003), ((), (), ((3.0, 1.0, 0.0),), 12, 1, 23011)])
+def test_split_program_matches_the_whole_program(gauss, sech, expo, p, s, n):
+    """The split sampler (small entries in single precision; from 1.5e8 entries
+    evaluated) against the whole program in double (kernel="generic") on the same
+    samples, with narrow features, two slices and a partial last item: 1e-12 of
+    the weight, or of its largest terms' scale where they cancel (the weights are
+    O(1) here)."""
     par = list(su.general_params((0.1, 0.0, 0.5, 0.0, 0.2), list(gauss), list(sech), list(expo)))
     w = []
     for kernel in ("auto", "generic"):
-        out = torch.zeros((333, s), dtype=torch.float64, device="cuda")
-        su.speedup_logweights("general", par, -0.4, 0.6, 0.2, p, s, 5, 333, 99, out, precision="fp64", kernel=kernel)
+        out = torch.zeros((n, s), dtype=torch.float64, device="cuda")
+        su.speedup_logweights("general", par, -0.4, 0.6, 0.2, p, s, 5, n, 99, out, precision="fp64", kernel=kernel)
         torch.cuda.synchronize()
         w.append(out.cpu().numpy())
     assert np.isfinite(w[0]).all()
