@@ -425,14 +425,16 @@ def run_ours(args):
     fma32 = su.su_fma_peak("fp32")
     peak64 = 2 * fma64 / 1e12
     achieved32 = chosen["flops"] / (chosen["total_ms"] / 1e3) / 1e12
-    roofline = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved / FP64_PEAK_TFLOPS,
+    roofline = {"bound": "alu", "achieved": achieved, "peak": 2 * fma32 / 1e12, "unit": "TFLOP/s",
+                "frac": achieved / (2 * fma32 / 1e12),
                 "traffic": FP64_TRAFFIC_BYTES * n_mc / FP64_TRAFFIC_SAMPLES,
                 "traffic_note": "bytes per launch: DRAM read+write of the 2e5-sample ncu capture of the same "
                                 "kernel (p = 10) scaled by samples; the algorithmic bytes per slice-action are 0",
-                "kernel": "sampler_kernel<double, RING_EVEN> (+ its combine)",
-                "peak_source": "152 SMs x 2 FP64 FMA/clock x 2 flop x 2.07 GHz (MEASURED_PEAKS.json has no "
-                               "FP64 figure); measured_fma_peak_tflops is this GPU's FMA loop (su_fma_peak)",
+                "kernel": "sampler_fx_kernel (+ its combine): 64-bit fixed point on the integer and FP32 pipes",
+                "peak_source": "this GPU's FP32 FMA loop (su_fma_peak): the pipes that the kernel runs on, where a "
+                               "64-bit product is several 32-bit ones; the FP64 pipe's own peak is 152 SMs x 2 "
+                               "FMA/clock x 2 flop x 2.07 GHz",
+                "fp64_pipe_peak": FP64_PEAK_TFLOPS,
                 "measured_fma_peak_tflops": {"fp64": peak64, "fp32": 2 * fma32 / 1e12},
                 "frac_of_measured_fp64": achieved / peak64,
                 "fp32_sampler": {"kernel": "sampler_kernel<float, RING_EVEN, false, K> (the compiled table shape K of each p)",
@@ -453,6 +455,8 @@ def run_ours(args):
         "config": {"workload": "convergence sweep: AHO g=10 T=1 a=0 b=1, s=10 (N=1..1024 via hierarchy), "
                                "1e7 samples/100 blocks per rank, p=k mod 18+1 per step, plain method: W_p and "
                                "log-sum-exp in fp64",
+                   "arithmetic": "double precision: normals, path and the leading part of W_p in 64-bit fixed point, "
+                                 "the part of W_p below 2^-29 of it in single precision, reductions in double",
                    "l2": "flushed (256 MB write) before every step", "seed": inst.seed},
         "chosen_fp32": {"value": chosen["sa"] * world / (chosen["total_ms"] / 1e3), "unit": UNIT,
                         "ms_per_step": chosen["total_ms"] / max(args.steps, 1), "dtype": "f32 W_p, f64 reductions",
