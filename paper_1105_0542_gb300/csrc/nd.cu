@@ -127,23 +127,30 @@ __device__ __forceinline__ float nd_single(const NdParams &Q, const uint32_t *w,
     return s;
 }
 
-// two slices' -eps W in double
-template <int D, typename PT>
+// B slices' -eps W in double
+template <int D, int B, typename PT>
 __device__ __forceinline__ double nd_double(const NdParams &Q, unsigned sq, const uint32_t *w, const double *c, PT &&pt,
                                             int k0, int stp) {
-    Vars<double, 2 * D, 2> v;
+    Vars<double, 2 * D, B> v;
 #pragma unroll
     for (int k = 0; k < 2 * D; ++k) {
         const int var = Q.order[k], cc = var >= D ? var - D : var;
         const double sg = var >= D ? -1.0 : 1.0;
-        const double a = pt(k0 * stp, cc), b = pt((k0 + 1) * stp, cc), e = pt((k0 + 2) * stp, cc);
-        v.z[k][0] = fma(sg, a, b);
-        v.z[k][1] = fma(sg, b, e);
+        double l = pt(k0 * stp, cc);
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            const double e = pt((k0 + i + 1) * stp, cc);
+            v.z[k][i] = fma(sg, l, e);
+            l = e;
+        }
     }
     v.close(sq, Q.one);
-    double t[2];
+    double t[B];
     nd_poly<0>(w, c, v, t);
-    return t[0] + t[1];
+    double s = 0;
+#pragma unroll
+    for (int i = 0; i < B; i += 2) s += t[i] + t[i + 1];
+    return s;
 }
 
 // R = double or float (the path and the per-level sums; the item's log-sum-exp
@@ -154,8 +161,10 @@ __device__ __forceinline__ double nd_double(const NdParams &Q, unsigned sq, cons
 //
 // What bounds it.  Single precision: instruction issue, most of it the packed
 // multiply-adds of the nest and the loops around them.  Double: the FP64 pipe
-// (2 lanes a cycle; 58 % busy) in the double part, a tenth of the entries on fine
-// levels, and the latency of its short chains.
+// (2 lanes a cycle; 56 % busy) in the double part, a tenth of the entries on fine
+// levels, and the latency of its short chains: four slices a pass instead of two,
+// where their variables fit the registers (D <= 2), took the case above from 29.7 to
+// 24.4 ms.
 template <typename R, int D>
 __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __grid_constant__ NdParams Q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -203,6 +212,7 @@ __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __gr
     R *q = reinterpret_cast<R *>(Q.paths) + (int64_t)blockIdx.x * kThreads + tid;
     auto co = [&](int i, int c) -> R & { return q[((int64_t)i * D + c) * ps]; };
     R seg[((1 << kNdSeg) + 1) * D];
+    constexpr int kBD = D <= 2 ? 4 : 2;          // slices per pass of the double part
     constexpr int kBP = D == 4 ? 2 : 4;          // pairs of slices per pass of the single-precision program
 
     for (int64_t item = P.item0 + blockIdx.x; item < P.n_items; item += gridDim.x) {
@@ -290,14 +300,20 @@ __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __gr
 #pragma unroll 1
                             for (int k = 0; k < ns; k += 2) tail += nd_single<R, D, 1>(Q, words, c, pt, k, stp);
                         }
+                        if (kBD > 2 && ns >= kBD) {
 #pragma unroll 1
-                        for (int k = 0; k < ns; k += 2)
-                            w += nd_double<D>(Q, Q.hsq[dl], hwords + Q.hw[dl], hcoef + Q.hc[dl], pt, k, stp);
+                            for (int k = 0; k < ns; k += kBD)
+                                w += nd_double<D, kBD>(Q, Q.hsq[dl], hwords + Q.hw[dl], hcoef + Q.hc[dl], pt, k, stp);
+                        } else {
+#pragma unroll 1
+                            for (int k = 0; k < ns; k += 2)
+                                w += nd_double<D, 2>(Q, Q.hsq[dl], hwords + Q.hw[dl], hcoef + Q.hc[dl], pt, k, stp);
+                        }
                         w += (double)tail;
                     } else {
 #pragma unroll 1
                         for (int k = 0; k < ns; k += 2)
-                            w += nd_double<D>(Q, Q.sq, words, reinterpret_cast<const double *>(P.tables) + (size_t)dl * P.M, pt, k, stp);
+                            w += nd_double<D, 2>(Q, Q.sq, words, reinterpret_cast<const double *>(P.tables) + (size_t)dl * P.M, pt, k, stp);
                     }
                     wloc[dl] += w;
                 };
