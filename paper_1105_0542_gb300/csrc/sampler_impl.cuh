@@ -147,52 +147,100 @@ __device__ __forceinline__ R ring_var(R us, R alpha) {
 // polynomial table; Gaussians through the Hermite recurrence; sech^2 = tanh'
 // through the Taylor coefficients a_k of tanh, (n+1) a_{n+1} = -sum_k a_k a_{n-k}
 // from tanh' = 1 - tanh^2, which stay accurate where tanh is near +-1.
-__device__ __forceinline__ void general_derivatives(double x, const GeneralDev *__restrict__ G, int J,
-                                                    double (&V)[kGenMaxSym]) {
+// Of B slices side by side: the recurrences are chains, and B of them share the
+// loops and the constants' loads (two features, p = 10, N = 64, 200 001 samples:
+// 27.7 -> 24.7 ms, with the steps of odd and even order apart).
+template <int B>
+__device__ __forceinline__ void general_derivatives(const double (&x)[B], const GeneralDev *__restrict__ G, int J,
+                                                    double (&V)[kGenMaxSym][B]) {
     const int deg = G->deg;
     for (int j = 0; j <= J; ++j) {
-        double v = 0.0;
+        double v[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) v[b] = 0.0;
         if (j <= deg) {
-            v = G->poly_der[j][deg];
-            for (int i = deg - 1; i >= j; --i) v = fma(v, x, G->poly_der[j][i]);
+            const double top = G->poly_der[j][deg];
+#pragma unroll
+            for (int b = 0; b < B; ++b) v[b] = top;
+            for (int i = deg - 1; i >= j; --i) {
+                const double c = G->poly_der[j][i];
+#pragma unroll
+                for (int b = 0; b < B; ++b) v[b] = fma(v[b], x[b], c);
+            }
         }
-        V[j] = v;
+#pragma unroll
+        for (int b = 0; b < B; ++b) V[j][b] = v[b];
     }
     for (int g = 0; g < G->ng; ++g) {
         // D_n = (d/dx)^n A e^{-beta u^2}: D_{n+1} = -2 beta (u D_n + n D_{n-1})
-        const double u = x - G->gauss[g][2], b2 = -2.0 * G->gauss[g][1], y = b2 * u;
-        double d0 = 0.0, d1 = G->gauss[g][0] * exp(0.5 * y * u), c = 0.0;
+        const double b2 = -2.0 * G->gauss[g][1], A = G->gauss[g][0], c0 = G->gauss[g][2];
+        double y[B], d0[B], d1[B], c = 0.0;
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const double u = x[b] - c0;
+            y[b] = b2 * u;
+            d0[b] = 0.0;
+            d1[b] = A * exp(0.5 * y[b] * u);
+        }
         for (int n = 0; n <= J; ++n) {
-            V[n] += d1;
-            const double d2 = fma(y, d1, c * d0);
-            d0 = d1;
-            d1 = d2;
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                V[n][b] += d1[b];
+                const double d2 = fma(y[b], d1[b], c * d0[b]);
+                d0[b] = d1[b];
+                d1[b] = d2;
+            }
             c += b2;
         }
     }
     for (int q = 0; q < G->ns; ++q) {
-        const double w = G->sech[q][1] * (x - G->sech[q][2]);
-        const double em = expm1(-2.0 * fabs(w)), e = exp(-2.0 * fabs(w));
-        const double r = 1.0 / (2.0 + em);         // 1 / (1 + e^{-2|w|})
-        double a[kGenMaxSym + 1];
-        a[0] = copysign(-em * r, w);               // tanh w
-        a[1] = 4.0 * e * (r * r);                  // sech^2 w
-        V[0] = fma(G->sech_scale[q][0], a[1], V[0]);
-        for (int n = 1; n <= J; ++n) {
-            double acc = a[0] * a[n];
-            for (int k = 1; k < (n + 1) / 2; ++k) acc = fma(a[k], a[n - k], acc);
-            acc = (n & 1) ? acc + acc : fma(a[n >> 1], a[n >> 1], acc + acc);
-            a[n + 1] = -acc * G->inv[n + 1];
-            V[n] = fma(G->sech_scale[q][n], a[n + 1], V[n]);
+        double a[kGenMaxSym + 1][B];
+        const double s0 = G->sech_scale[q][0];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const double w = G->sech[q][1] * (x[b] - G->sech[q][2]);
+            const double em = expm1(-2.0 * fabs(w)), e = exp(-2.0 * fabs(w));
+            const double r = 1.0 / (2.0 + em);         // 1 / (1 + e^{-2|w|})
+            a[0][b] = copysign(-em * r, w);            // tanh w
+            a[1][b] = 4.0 * e * (r * r);               // sech^2 w
+            V[0][b] = fma(s0, a[1][b], V[0][b]);
+        }
+        // odd and even n in turn: as a condition the square was computed for both
+        auto next = [&](int n, auto even) {
+            double acc[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) acc[b] = a[0][b] * a[n][b];
+            for (int k = 1; k < (n + 1) / 2; ++k)
+#pragma unroll
+                for (int b = 0; b < B; ++b) acc[b] = fma(a[k][b], a[n - k][b], acc[b]);
+            const double f = -G->inv[n + 1], f2 = f + f, sc = G->sech_scale[q][n];
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                if constexpr (decltype(even)::value) {
+                    const double h = a[n / 2][b];
+                    a[n + 1][b] = fma(acc[b], 2.0, h * h) * f;
+                } else {
+                    a[n + 1][b] = acc[b] * f2;
+                }
+                V[n][b] = fma(sc, a[n + 1][b], V[n][b]);
+            }
+        };
+        for (int n = 1; n <= J; n += 2) {
+            next(n, std::false_type());
+            if (n < J) next(n + 1, std::true_type());
         }
     }
     for (int q = 0; q < G->ne; ++q) {   // exponentials: (-kappa)^n E e^{-kappa (x - x0)}
         const double kap = G->expo[q][1];
-        double e = G->expo[q][0] * exp(-kap * (x - G->expo[q][2]));
-        for (int n = 0; n <= J; ++n) {
-            V[n] += e;
-            e *= -kap;
-        }
+        double e[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) e[b] = G->expo[q][0] * exp(-kap * (x[b] - G->expo[q][2]));
+        for (int n = 0; n <= J; ++n)
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                V[n][b] += e[b];
+                e[b] *= -kap;
+            }
     }
 }
 
@@ -207,15 +255,16 @@ __device__ __noinline__ double2 slice_general(double ql0, double qr0, double ql1
                                               const double *__restrict__ coef, const GeneralDev *__restrict__ G,
                                               const GeneralNode *__restrict__ nodes, int nn, int J) {
     const double ql[2] = {ql0, ql1}, qr[2] = {qr0, qr1};
-    double V[B][kGenMaxSym], Y[B], stk[B][kGenMaxDepth + 1], w[B];
+    double V[kGenMaxSym][B], x[B], Y[B], stk[kGenMaxDepth + 1][B], w[B];
 #pragma unroll
     for (int b = 0; b < B; ++b) {
-        general_derivatives(0.5 * (ql[b] + qr[b]), G, J, V[b]);
+        x[b] = 0.5 * (ql[b] + qr[b]);
         const double vs = qr[b] - ql[b];
         Y[b] = vs * vs;
-        stk[b][0] = 1.0;
+        stk[0][b] = 1.0;
         w[b] = 0.0;
     }
+    general_derivatives<B>(x, G, J, V);
     for (int t = 0; t < nn; ++t) {
         const GeneralNode nd = nodes[t];
         double mu[B];
@@ -223,8 +272,8 @@ __device__ __noinline__ double2 slice_general(double ql0, double qr0, double ql1
         for (int b = 0; b < B; ++b) {
             mu[b] = 1.0;
             if (t) {
-                mu[b] = stk[b][nd.depth - 1] * V[b][nd.sym];
-                stk[b][nd.depth] = mu[b];
+                mu[b] = stk[nd.depth - 1][b] * V[nd.sym][b];
+                stk[nd.depth][b] = mu[b];
             }
         }
         const int cnt = nd.count;
