@@ -2437,7 +2437,7 @@ extern "C" int su_mlp_forward(const su_proposal *pr, const float *d_X, int64_t n
 }
 
 // plan + proposal parameters with 128-sample items (one path per thread of
-// the first 128 threads of a 256-thread CTA)
+// the first 128 threads of a group)
 static int proposal_setup(su_plan *pl, const su_proposal *pr, su::ProposalParams &Q, int &grid, size_t &smem) {
     using namespace su;
     std::memset(&Q, 0, sizeof Q);
