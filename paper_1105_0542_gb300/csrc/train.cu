@@ -89,20 +89,26 @@ constexpr uint32_t kTD = 0, kTW2 = 128, kTW3 = 256, kTW1 = 384, kTB2 = 400, kTB3
 constexpr int kOffX0 = mlp::kBlobBytes, kOffDY = kOffX0 + kX0Bytes, kOffH = (kOffDY + kX0Bytes + 127) / 128 * 128;
 constexpr int kStepSmem = kOffH + 4 * kHBytes;
 
-// GELU(v) = v (1 + erf(v / sqrt 2)) / 2 of two values, as mlp::gelu2, and its
-// derivative from the same polynomial of erf
-__device__ __forceinline__ float2 gelu_both(float2 v, float2 &grad) {
+// GELU(v) = v (1 + erf(v / sqrt 2)) / 2 of two values and its derivative, from one
+// polynomial of erf (that of mlp::gelu2)
+__device__ __forceinline__ float2 one_plus_erf(float2 v) {
     const float c = mlp::kErfClamp;
     const float2 x = make_float2(fminf(fmaxf(v.x, -c), c), fminf(fmaxf(v.y, -c), c));
     const float2 z = __fmul2_rn(x, x);
     float2 p = make_float2(mlp::erf_poly(mlp::kErfTerms - 1), mlp::erf_poly(mlp::kErfTerms - 1));
 #pragma unroll
     for (int k = mlp::kErfTerms - 2; k >= 0; --k) p = __ffma2_rn(p, z, make_float2(mlp::erf_poly(k), mlp::erf_poly(k)));
-    const float2 half = make_float2(0.5f, 0.5f), e = __fmul2_rn(x, p), h = __fmul2_rn(v, half);
-    const float2 g = make_float2(0.39894228040143268f * __expf(-0.5f * v.x * v.x),
-                                 0.39894228040143268f * __expf(-0.5f * v.y * v.y));
-    grad = __ffma2_rn(v, g, __ffma2_rn(e, half, half));
-    return __ffma2_rn(h, e, h);
+    return __ffma2_rn(x, p, make_float2(1.0f, 1.0f));
+}
+__device__ __forceinline__ float2 gelu(float2 v) {
+    return __fmul2_rn(__fmul2_rn(v, make_float2(0.5f, 0.5f)), one_plus_erf(v));
+}
+__device__ __forceinline__ float2 gelu_both(float2 v, float2 &grad) {
+    const float2 half = make_float2(0.5f, 0.5f), o = one_plus_erf(v);
+    const float2 e = make_float2(__expf(-0.5f * v.x * v.x), __expf(-0.5f * v.y * v.y));
+    const float2 g = __fmul2_rn(__fmul2_rn(v, make_float2(0.39894228040143268f, 0.39894228040143268f)), e);
+    grad = __ffma2_rn(half, o, g);
+    return __fmul2_rn(__fmul2_rn(v, half), o);
 }
 
 __device__ __forceinline__ float2 unpack_bf16(uint32_t w) {
@@ -285,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_kernel(const StepArgs P) {
             commit(tc);
         }
         if (!(ok = arrived())) break;
-        forward(B, H, [](int, float2 x) { return mlp::gelu2(x); });
+        forward(B, H, [](int, float2 x) { return gelu(x); });
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;");
             mma(tc.tmem + kTD, k_major(aH, kHid), w2, kHid, 8, false);
