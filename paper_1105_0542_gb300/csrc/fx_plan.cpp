@@ -29,6 +29,11 @@ namespace su {
 
 // the largest integer of a chain, with room for the products' constants
 static constexpr double kFxMax = 0x1.8p62;
+// ranges for which every scale below is a normal double: path points at most
+// 1e100 and at least 1e-100 across, weights in units of 2^-900 to 2^900 (the
+// conversion of the sums puts the unit into a double's exponent)
+static constexpr double kFxLeast = 1e-100;
+static constexpr int kFxUnits = 900;
 
 void fx_plan(SamplerParams &P, double T, const double *tables, std::vector<int64_t> &head, std::vector<float> &tail) {
     FxParams &X = P.fx;
@@ -41,6 +46,7 @@ void fx_plan(SamplerParams &P, double T, const double *tables, std::vector<int64
     int qe;
     const double qm = std::frexp(std::max(std::fabs(P.a), std::fabs(P.b)) + 2.9 * std::sqrt(T), &qe);
     const double Q = std::ldexp(std::ceil(qm * 256), qe - 8);
+    if (!(Q >= kFxLeast && Q <= 1 / kFxLeast)) return;
     const bool th = P.ring == RING_TANH2;
     X.q_unit = std::ldexp(Q, -62);
     if (th) {
@@ -105,21 +111,24 @@ void fx_plan(SamplerParams &P, double T, const double *tables, std::vector<int64
         std::vector<double> my((size_t)P.ncol, 1.0);
         for (int j = 1; j < P.ncol; ++j)
             my[j] = std::min(1.0, my[j - 1] * yt * std::sqrt((4.0 * j - 1) * (4.0 * j - 3)));
-        double typ = 0;
+        double typ = 0, most = 0;
+        bool finite = true;
         for (int k = 0; k < M; ++k) {
             C[k] = t[k];
             for (int i = 0; i < row[k]; ++i) C[k] *= zs;
             for (int j = 0; j < col[k]; ++j) C[k] *= ys;
             typ += std::fabs(C[k]) * mz[row[k]] * my[col[k]];
+            most = std::max(most, std::fabs(C[k]));
+            finite = finite && std::isfinite(C[k]);
         }
+        if (!finite || !std::isfinite(typ)) continue;
         const double N = std::ldexp(1.0, n);
         const double ns = (d <= P.F && n > 0) ? std::min(4.0, std::ldexp(1.0, P.F - d)) : 1.0;   // slices per 64-bit sum
         const double tol = 0x1p-55 * std::min(1.0, N * typ);
-        if (!(tol > 0) || !std::isfinite(tol)) {
-            // W_p = 0 on the whole path: any scale will do
-            if (typ != 0) continue;
-        }
-        const int E = tol > 0 ? (int)std::ceil(std::log2(0.5 * std::sqrt(N) / tol)) : 60;
+        // W_p = 0 on the whole path: any scale will do
+        const double units = tol > 0 ? std::ceil(std::log2(0.5 * std::sqrt(N) / tol)) : most > 0 ? kFxUnits + 1 : 60;
+        if (!(std::fabs(units) <= kFxUnits)) continue;
+        const int E = (int)units;
         const double scale = std::ldexp(1.0, E);
         // entries beyond each column's heads, root mean square
         auto rest = [&](const int *h, int j) {
@@ -133,13 +142,13 @@ void fx_plan(SamplerParams &P, double T, const double *tables, std::vector<int64
         int h[kFxCols] = {1};
         bool fits = true;
         for (;;) {
-            double sum = 0, most = -1;
+            double sum = 0, top = -1;
             int at = -1;
             for (int j = 0; j < P.ncol; ++j) {
                 const double x = rest(h, j);
                 sum += x;
-                if (x > most) {
-                    most = x;
+                if (x > top) {
+                    top = x;
                     at = j;
                 }
             }
