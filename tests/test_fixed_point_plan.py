@@ -69,5 +69,5 @@ def test_plan_ends_with_scales_that_a_double_holds(plan, ring, a, T, factor):
 
 
 def test_plan_takes_ordinary_tables(plan):
-    on, levels = plan(EVEN, 0.0, 1.0, 1.0, 1.0, 10, (6, 4, 3, 1), 1e-3)
+    on, levels = plan(EVEN, 0.0, 0.5, 0.25, 1.0, 10, (6, 4, 3, 1), 1e-3)
     assert on and sum(ok for ok, _, _ in levels) >= 5
