@@ -186,6 +186,10 @@ __device__ __forceinline__ void tanh_load(TanhNode *t, int n, int tid, int nthre
 }
 #endif
 
+// |x| for the node index: a sum of two points that has left 64 bits may be
+// -2^63, whose magnitude is taken as zero (such a path is weighed again)
+SU_FX_FN int64_t magnitude(int64_t x) { return (x < 0 ? 0 - (uint64_t)x : (uint64_t)x) & 0x7FFFFFFFFFFFFFFFULL; }
+
 SU_FX_FN int64_t tanh2(int64_t w, const TanhNode *__restrict__ t) {
     const TanhNode &n = t[(int)(w >> 53)];
     const int64_t f = (int64_t)(((uint64_t)w << 11) >> 2);         // units 2^-62

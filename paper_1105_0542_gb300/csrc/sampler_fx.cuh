@@ -99,7 +99,7 @@ __device__ __forceinline__ fx::Limbs fx_ring(int64_t us, const FxParams &X, cons
     if constexpr (RING == RING_EVEN)
         return fx::limbs(fx::square(fx::limbs(us)) << 1);
     else
-        return fx::limbs(fx::tanh2(fx::mul(us < 0 ? -us : us, fx::Limbs{X.ah, X.al}), th) << 1);
+        return fx::limbs(fx::tanh2(fx::mul(fx::magnitude(us), fx::Limbs{X.ah, X.al}), th) << 1);
 }
 
 // a high word in units of 1

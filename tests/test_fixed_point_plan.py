@@ -71,3 +71,36 @@ def test_plan_ends_with_scales_that_a_double_holds(plan, ring, a, T, factor):
 def test_plan_takes_ordinary_tables(plan):
     on, levels = plan(EVEN, 0.0, 0.5, 0.25, 1.0, 10, (6, 4, 3, 1), 1e-3)
     assert on and sum(ok for ok, _, _ in levels) >= 5
+
+
+INDEX = r"""
+#include <cmath>
+#include <cstdio>
+#include "fixed_point.cuh"
+using namespace su;
+// the node of tanh^2 for sums of two points, as the sampler finds it, from the plan's limbs
+int main() {
+    double step;
+    long long us;
+    while (std::scanf("%lf %lld", &step, &us) == 2) {
+        const fx::Limbs l = fx::limbs((int64_t)std::nearbyint((long double)step * std::ldexp(1.0L, 64 + 53 - 63)));
+        std::printf("%lld\n", (long long)(fx::mul(fx::magnitude((int64_t)us), l) >> 53));
+    }
+}
+"""
+
+
+def test_every_sum_of_two_points_has_a_node(tmp_path):
+    """Sums that leave 64 bits wrap: also the most negative one finds a node
+    of those in reach, 0..int(step)."""
+    (tmp_path / "index.cpp").write_text(INDEX)
+    exe = str(tmp_path / "index")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-I", CSRC, str(tmp_path / "index.cpp"), "-o", exe], check=True)
+    steps = (1e-12, 1e-7, 2.0 ** -22, 0.3, 1.0, 5.999999, 150.25, 383.999)
+    sums = (-2 ** 63, -2 ** 63 + 1, -2 ** 62, -2 ** 32, -1, 0, 1, 2 ** 32 - 1, 2 ** 62, 2 ** 63 - 1)
+    pairs = [(step, us) for step in steps for us in sums]
+    out = subprocess.run([exe], input="\n".join(f"{a!r} {b}" for a, b in pairs), capture_output=True, text=True,
+                         check=True).stdout.split()
+    assert len(out) == len(pairs)
+    for (step, us), k in zip(pairs, out):
+        assert 0 <= int(k) <= int(step), (step, us)
