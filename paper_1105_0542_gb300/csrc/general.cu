@@ -221,12 +221,14 @@ __global__ void __launch_bounds__(kThreads, 4) general_kernel(const __grid_const
                     const GeneralNode *nd = split ? hnodes + P.gs.h0[d] : nodes;
                     const int nn = split ? P.gs.hn[d] : G->n_nodes, J = split ? P.gs.hj[d] : G->J;
                     const double *c = split ? hcoef + P.gs.hc[d] : reinterpret_cast<const double *>(P.tables) + (size_t)d * P.M;
+                    double sum = 0;   // of this segment (one running sum over the path rounds at its full size)
 #pragma unroll 1
                     for (int k = 0; k < ns; k += 2) {
                         const double2 v = slice_general<2>(q[k * stp], q[(k + 1) * stp], q[(k + 1) * stp], q[(k + 2) * stp],
                                                            c, G, nd, nn, J);
-                        w[d] += v.x + v.y;
+                        sum += v.x + v.y;
                     }
+                    w[d] += sum;
                 };
                 // coarse levels: the segment endpoints
                 co[0] = P.a;
