@@ -505,7 +505,7 @@ static void split_general(su_plan &pl, std::vector<unsigned char> &blob, int sme
     bool any = false;
     for (int d = 0; d < pl.levels; ++d) {
         const double *t = tab.data() + (size_t)d * M;
-        general_split(G, ms, pl.a, pl.b, pl.T, S - d, t, head);
+        P.gs.lim[d] = (float)(kGenReach * general_split(G, ms, pl.a, pl.b, pl.T, S - d, t, head));
         int total = 0;
         bool fits = true;
         for (size_t k = 0; k < nn; ++k) {

@@ -9,9 +9,11 @@
 // busy), most of them the derivatives that the large entries need; the packed program
 // hides behind them.  Two features, p = 10, N = 64, 200 001 samples: 62.4 -> 24.7 ms.
 //
-// A path whose single-precision part is too large against its weight (narrow
-// features that the plan's moments missed, paths far out) is weighed again by
-// the whole program in double.
+// A level of a path whose single-precision entries are too large in sum -- 2^-30 of
+// the smaller of one and the level's typical weight, or of a weight beyond one --
+// (narrow features that the plan's moments missed, paths far out) is weighed again
+// by the whole program in double: a few 2^-24 of the entries stay below a double's
+// rounding of the weight's exponential.
 #include <cstdint>
 
 #include "sampler_impl.cuh"
@@ -20,7 +22,7 @@ namespace su {
 namespace {
 
 constexpr int kGenSeg = 5;   // the path in segments of 2^5 slices
-constexpr float kGenTail = 0x1p-22f;   // largest single-precision part, of max(1, |w|)
+constexpr float kGenTail = 0x1p-30f;   // largest single-precision part of a weight beyond one, as lim of one up to it
 
 // V^(j)(x) / j!, j = 0..J, of two slices
 __device__ __forceinline__ void taylor_pair(float x0, float x1, const GeneralDev *__restrict__ G, float2 (*U)[4], int m) {
@@ -84,12 +86,13 @@ __device__ __forceinline__ void taylor_pair(float x0, float x1, const GeneralDev
 }
 
 // 2 BP slices between the points q[k0 stp ..]: the single-precision part of
-// -eps W_p; adds to sum and its magnitude to mag
+// -eps W_p; adds to sum, and its nodes' magnitudes to mag (the roundings are of
+// the entries: what cancels between them does not cancel there)
 template <int BP>
 __device__ __noinline__ void gen_single(const GeneralDev *__restrict__ G, const GeneralNode *__restrict__ nodes,
                                         const float *__restrict__ coef, const double *q, int k0, int stp, float &sum,
                                         float &mag) {
-    float2 U[kGenMaxSym][4], stk[kGenMaxDepth + 1][BP], Y[BP], w[BP];
+    float2 U[kGenMaxSym][4], stk[kGenMaxDepth + 1][BP], Y[BP], w[BP], m[BP];
 #pragma unroll 1
     for (int i = 0; i < BP; ++i) {
         const double a = q[(k0 + 2 * i) * stp], b = q[(k0 + 2 * i + 1) * stp], c = q[(k0 + 2 * i + 2) * stp];
@@ -100,7 +103,7 @@ __device__ __noinline__ void gen_single(const GeneralDev *__restrict__ G, const 
         const double a = q[(k0 + 2 * i) * stp], b = q[(k0 + 2 * i + 1) * stp], c = q[(k0 + 2 * i + 2) * stp];
         const float2 vs = make_float2(__double2float_rn(b - a), __double2float_rn(c - b));
         Y[i] = __fmul2_rn(vs, vs);
-        w[i] = make_float2(0.f, 0.f);
+        w[i] = m[i] = make_float2(0.f, 0.f);
     }
     const int nn = G->n_nodes;
 #pragma unroll 1
@@ -131,13 +134,18 @@ __device__ __noinline__ void gen_single(const GeneralDev *__restrict__ G, const 
                 for (int i = 0; i < BP; ++i) h[i] = __ffma2_rn(h[i], Y[i], ce);
             }
 #pragma unroll
-            for (int i = 0; i < BP; ++i) w[i] = __ffma2_rn(h[i], mu[i], w[i]);
+            for (int i = 0; i < BP; ++i) {
+                const float2 x = __fmul2_rn(h[i], mu[i]);
+                w[i] = __fadd2_rn(w[i], x);
+                m[i].x += fabsf(x.x);
+                m[i].y += fabsf(x.y);
+            }
         }
     }
 #pragma unroll
     for (int i = 0; i < BP; ++i) {
         sum += w[i].x + w[i].y;
-        mag += fabsf(w[i].x) + fabsf(w[i].y);
+        mag += m[i].x + m[i].y;
     }
 }
 
@@ -188,7 +196,8 @@ __global__ void __launch_bounds__(kThreads, 4) general_kernel(const __grid_const
             st.slo = (uint32_t)sample;
             st.shi = (uint32_t)(sample >> 32);
             double w[SU_MAX_S];
-            for (int pass = 0; pass < 2; ++pass) {
+            uint32_t todo = (1u << L) - 1u;   // levels of this pass
+            for (int pass = 0; pass < 2 && todo; ++pass) {
                 uint32_t have = 0xffffffffu;
                 double z0 = 0, z1 = 0;
                 auto normal = [&](uint32_t g) {
@@ -200,10 +209,11 @@ __global__ void __launch_bounds__(kThreads, 4) general_kernel(const __grid_const
                 };
                 float tsum[SU_MAX_S], tmag[SU_MAX_S];
                 for (int d = 0; d < L; ++d) {
-                    w[d] = 0;
+                    if (todo >> d & 1u) w[d] = 0;
                     tsum[d] = tmag[d] = 0;
                 }
                 auto slices = [&](int d, const double *q, int stp, int ns) {
+                    if (!(todo >> d & 1u)) return;
                     const bool split = pass == 0 && P.gs.hn[d] > 0;
                     if (split) {
                         const float *c = tail + (size_t)d * P.M;
@@ -256,12 +266,13 @@ __global__ void __launch_bounds__(kThreads, 4) general_kernel(const __grid_const
 #pragma unroll 1
                     for (int d = 0; d < min(F, L); ++d) slices(d, seg, 1 << d, NF >> d);
                 }
-                bool far = false;
-                for (int d = 0; d < L; ++d) {
-                    w[d] += (double)tsum[d];
-                    if (pass == 0 && P.gs.hn[d] > 0) far |= !(tmag[d] <= kGenTail * fmaxf(1.0f, fabsf(__double2float_rn(w[d]))));
-                }
-                if (!far) break;
+                uint32_t far = 0;
+                for (int d = 0; d < L; ++d)
+                    if (pass == 0 && P.gs.hn[d] > 0) {
+                        w[d] += (double)tsum[d];
+                        if (!(tmag[d] <= fmaxf(P.gs.lim[d], kGenTail * fabsf(__double2float_rn(w[d]))))) far |= 1u << d;
+                    }
+                todo = far;
             }
             bool bad = false;
             for (int d = 0; d < L; ++d) bad |= isnan(w[d]) || (isinf(w[d]) && w[d] > 0);

@@ -39,8 +39,8 @@ void general_moments(const GeneralEffective &G, const GeneralPotential &V, doubl
     for (double &v : ms) v = std::sqrt(v);
 }
 
-void general_split(const GeneralEffective &G, const std::vector<double> &ms, double a, double b, double T, int n,
-                   const double *table, std::vector<int> &head) {
+double general_split(const GeneralEffective &G, const std::vector<double> &ms, double a, double b, double T, int n,
+                     const double *table, std::vector<int> &head) {
     const double N = std::ldexp(1.0, n), eps = T / N, s2 = eps + (b - a) * (b - a) / (N * N);
     std::vector<double> my((size_t)G.K, 1.0);
     for (int k = 1; k < G.K; ++k) my[(size_t)k] = my[(size_t)k - 1] * s2 * std::sqrt((4.0 * k - 1) * (4.0 * k - 3));
@@ -54,7 +54,7 @@ void general_split(const GeneralEffective &G, const std::vector<double> &ms, dou
         }
     if (!std::isfinite(all)) {   // sizes beyond a double: nothing to split by
         head.assign(G.count.begin(), G.count.end());
-        return;
+        return 0;
     }
     // the smallest entries up to the sum: whole octaves, then the last one's in order
     const double most = 0x1p-33 * std::min(1.0, N * all) / N;
@@ -82,6 +82,7 @@ void general_split(const GeneralEffective &G, const std::vector<double> &ms, dou
             const int o = octave(v);
             if (o > oct || (o == oct && v >= least)) head[t] = k + 1;
         }
+    return N * most;
 }
 
 }  // namespace su

@@ -69,11 +69,14 @@ struct FxParams {
 
 // The split general program (general.cu; built by general_split): byte offsets
 // from the tables, and per level (row d) the double part's nodes, entries and
-// highest derivative (hn = 0: the whole program in double).
+// highest derivative (hn = 0: the whole program in double), and the largest sum of
+// the single-precision entries' magnitudes over a path (lim; kGenReach times the
+// plan's estimate).
 struct GeneralSplit {
     int on, staged, n_nodes;
     int64_t tail, hnodes, hcoef;
     int hn[SU_MAX_S], h0[SU_MAX_S], hc[SU_MAX_S], hj[SU_MAX_S];
+    float lim[SU_MAX_S];
 };
 
 struct SamplerParams {
@@ -116,9 +119,11 @@ struct SamplerParams {
 // root mean squares of the general program's monomials over the bridge
 void general_moments(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T,
                      std::vector<double> &ms);
-// head[t] = the leading entries of node t that need double precision on level n
-void general_split(const GeneralEffective &G, const std::vector<double> &ms, double a, double b, double T, int n,
-                   const double *table, std::vector<int> &head);
+// head[t] = the leading entries of node t that need double precision on level n;
+// the bound of the others' root mean squares, summed over the path
+double general_split(const GeneralEffective &G, const std::vector<double> &ms, double a, double b, double T, int n,
+                     const double *table, std::vector<int> &head);
+constexpr double kGenReach = 8;
 
 // The fixed-point plan of a double-precision plan's tables (rows of M entries,
 // kernel_table's, for levels n = S..1): fills P.fx (on = 0 where the ranges do

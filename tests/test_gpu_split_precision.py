@@ -92,3 +92,21 @@ def test_general_split_is_no_further_off_than_the_whole_program(V, p, s):
     assert np.any(w["auto"] != w["generic"])   # two programs
     rms = {k: np.sqrt(np.mean((v - ref) ** 2)) for k, v in w.items()}
     assert rms["auto"] <= 1.5 * rms["generic"]
+
+
+# samples of seed 1234 whose first normal is -6.17, -6.43: q_{N/2} some 3 sqrt(T) from the endpoints
+FAR = [492790794, 2573160571]
+
+
+def test_general_path_beyond_the_split_is_weighed_by_the_whole_program():
+    """The single-precision entries of such a path in the exponentials of a
+    Morse potential are a hundred times their typical sum: on the levels where
+    they are too many the weight is the whole program's, bit for bit, while
+    its neighbours' are the split's."""
+    a, b, T, p, s, n = 0.0, 0.6, 0.2, 8, 6, 12_000
+    for f in FAR:
+        w = {k: _general(MORSE, a, b, T, p, s, n, sample0=f - 100, seed=1234, kernel=k) for k in ("auto", "generic")}
+        same = w["auto"] == w["generic"]
+        assert same[100, 2] and same[100, 3]
+        assert not same[:, 3].all()
+        assert np.all(np.abs(w["auto"] - w["generic"]) <= 2.0 ** -50 * np.maximum(1.0, np.abs(w["generic"])))
