@@ -24,10 +24,12 @@ namespace {
 constexpr int kGenSeg = 5;   // the path in segments of 2^5 slices
 constexpr float kGenTail = 0x1p-30f;   // largest single-precision part of a weight beyond one, as lim of one up to it
 
-// V^(j)(x) / j!, j = 0..J, of two slices
-__device__ __forceinline__ void taylor_pair(float x0, float x1, const GeneralDev *__restrict__ G, float2 (*U)[4], int m) {
+// V^(j)(x) / j!, j = 0..J, of two slices.  (A feature's offset from x is taken in
+// double: far from the origin a rounded x would be off by a part of the feature.)
+__device__ __forceinline__ void taylor_pair(double xa, double xb, const GeneralDev *__restrict__ G, float2 (*U)[4], int m) {
     const int J = G->J;
-    const float2 x = make_float2(x0, x1);
+    auto offset = [&](double c) { return make_float2(__double2float_rn(xa - c), __double2float_rn(xb - c)); };
+    const float2 x = offset(0.0);
     for (int j = 0; j <= J; ++j) {
         float2 v = make_float2(0.f, 0.f);
         if (j <= G->deg)
@@ -35,11 +37,10 @@ __device__ __forceinline__ void taylor_pair(float x0, float x1, const GeneralDev
         U[j][m] = v;
     }
     for (int g = 0; g < G->ng; ++g) {
-        const float c = (float)G->gauss[g][2], sb = (float)G->gauss[g][3], beta = (float)G->gauss[g][1], A = (float)G->gauss[g][0];
-        const float u0 = x0 - c, u1 = x1 - c;
+        const float beta = (float)G->gauss[g][1], A = (float)G->gauss[g][0];
+        const float2 u = offset(G->gauss[g][2]);
         // g_n = (-sb)^n H_n(sb u) / n!: g_{n+1} = -2 beta (u g_n + g_{n-1}) / (n + 1)
-        float2 p = make_float2(0.f, 0.f), q = make_float2(A * expf(-beta * u0 * u0), A * expf(-beta * u1 * u1));
-        const float2 u = make_float2(u0, u1);
+        float2 p = make_float2(0.f, 0.f), q = make_float2(A * expf(-beta * u.x * u.x), A * expf(-beta * u.y * u.y));
         for (int n = 0; n <= J; ++n) {
             U[n][m] = __fadd2_rn(U[n][m], q);
             const float f = -2.0f * beta * G->invf[n + 1];
@@ -49,12 +50,12 @@ __device__ __forceinline__ void taylor_pair(float x0, float x1, const GeneralDev
         }
     }
     for (int s = 0; s < G->ns; ++s) {
-        const float al = (float)G->sech[s][1], d = (float)G->sech[s][2];
+        const float al = (float)G->sech[s][1];
+        const float2 u = offset(G->sech[s][2]);
         float t[2], t1[2];
-        const float xs[2] = {x0, x1};
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const float w = al * (xs[i] - d), em = expm1f(-2.0f * fabsf(w)), den = 2.0f + em;
+            const float w = al * (i ? u.y : u.x), em = expm1f(-2.0f * fabsf(w)), den = 2.0f + em;
             t[i] = copysignf(-em / den, w);               // tanh w
             t1[i] = 4.0f * (1.0f + em) / (den * den);     // sech^2 w
         }
@@ -75,8 +76,9 @@ __device__ __forceinline__ void taylor_pair(float x0, float x1, const GeneralDev
         }
     }
     for (int q = 0; q < G->ne; ++q) {
-        const float kap = (float)G->expo[q][1], E = (float)G->expo[q][0], c = (float)G->expo[q][2];
-        float2 e = make_float2(E * expf(-kap * (x0 - c)), E * expf(-kap * (x1 - c)));
+        const float kap = (float)G->expo[q][1], E = (float)G->expo[q][0];
+        const float2 u = offset(G->expo[q][2]);
+        float2 e = make_float2(E * expf(-kap * u.x), E * expf(-kap * u.y));
         for (int n = 0; n <= J; ++n) {
             U[n][m] = __fadd2_rn(U[n][m], e);
             const float f = -kap * G->invf[n + 1];
@@ -96,7 +98,7 @@ __device__ __noinline__ void gen_single(const GeneralDev *__restrict__ G, const 
 #pragma unroll 1
     for (int i = 0; i < BP; ++i) {
         const double a = q[(k0 + 2 * i) * stp], b = q[(k0 + 2 * i + 1) * stp], c = q[(k0 + 2 * i + 2) * stp];
-        taylor_pair(__double2float_rn(0.5 * (a + b)), __double2float_rn(0.5 * (b + c)), G, U, i);
+        taylor_pair(0.5 * (a + b), 0.5 * (b + c), G, U, i);
     }
 #pragma unroll
     for (int i = 0; i < BP; ++i) {

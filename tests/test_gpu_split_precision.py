@@ -110,3 +110,13 @@ def test_general_path_beyond_the_split_is_weighed_by_the_whole_program():
         assert same[100, 2] and same[100, 3]
         assert not same[:, 3].all()
         assert np.all(np.abs(w["auto"] - w["generic"]) <= 2.0 ** -50 * np.maximum(1.0, np.abs(w["generic"])))
+
+
+def test_general_split_far_from_the_origin():
+    """Features about 1000: both programs take the offsets from the same
+    points, so they differ by what they do near the origin -- the guard's
+    2^-30 in single precision, a few 2^-24 of it, and the sums' own rounding."""
+    V = dict(poly=(0.0,), gauss=[(1.5, 2.0, 1000.3)], sech=[(-1.0, 2.0, 1000.0)])
+    w = {k: _general(V, 999.5, 1000.7, 0.25, 8, 7, 20_000, kernel=k) for k in ("auto", "generic")}
+    assert np.any(w["auto"][:, -1] != w["generic"][:, -1])
+    assert np.all(np.abs(w["auto"] - w["generic"]) <= 2.0 ** -50 * np.maximum(1.0, np.abs(w["generic"])))
