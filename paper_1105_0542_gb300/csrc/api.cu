@@ -203,7 +203,7 @@ struct su_plan {
     int64_t n_blocks = 1;
     su::SamplerParams P{};
     void *d_tables = nullptr;
-    bool tables_async = false;   // d_tables is stream-ordered on opt.stream (a plan inside one call)
+    bool tables_async = false;   // d_tables and d_general are stream-ordered on opt.stream (a plan inside one call)
     int device = 0;
     int grid = 0;
     size_t smem = 0;
@@ -330,8 +330,9 @@ static int validate(int model, const double *params, int n_params, double a, dou
 }
 
 // Device image of the general program and potential: one allocation holding
-// GeneralDev and the depth-first nodes.
-static int general_image(const su::GeneralEffective &G, const su::GeneralPotential &V, void **d_out) {
+// GeneralDev and the depth-first nodes; stream-ordered on *st where given.
+static int general_image(const su::GeneralEffective &G, const su::GeneralPotential &V, void **d_out,
+                         const cudaStream_t *st = nullptr) {
     using namespace su;
     *d_out = nullptr;
     GeneralDev D;
@@ -391,17 +392,22 @@ static int general_image(const su::GeneralEffective &G, const su::GeneralPotenti
         for (int n = 0; n <= G.J; ++n) D.sech_tay[q][n] = (float)(V.sech[q][0] * std::pow(V.sech[q][1], n) * (n + 1));
     const size_t o_nodes = (sizeof(GeneralDev) + 15) & ~(size_t)15;
     const size_t bytes = o_nodes + nodes.size() * sizeof(GeneralNode);
-    CU(dmalloc(d_out, bytes), "device allocation (general program)");
+    CU(st ? dmalloc_async(d_out, bytes, *st) : dmalloc(d_out, bytes), "device allocation (general program)");
     char *base = static_cast<char *>(*d_out);
     D.nodes = reinterpret_cast<const GeneralNode *>(base + o_nodes);
     std::vector<unsigned char> blob(bytes, 0);
     std::memcpy(blob.data(), &D, sizeof D);
     std::memcpy(blob.data() + o_nodes, nodes.data(), nodes.size() * sizeof(GeneralNode));
-    CU(cudaMemcpy(*d_out, blob.data(), bytes, cudaMemcpyHostToDevice), "upload general program");
+    CU(st ? cudaMemcpyAsync(*d_out, blob.data(), bytes, cudaMemcpyHostToDevice, *st)
+          : cudaMemcpy(*d_out, blob.data(), bytes, cudaMemcpyHostToDevice),
+       "upload general program");
     return SU_OK;
 }
 
-static int upload_general(su_plan &pl) { return general_image(*pl.G, pl.V, &pl.d_general); }
+static int upload_general(su_plan &pl) {
+    cudaStream_t st = (cudaStream_t)pl.opt.stream;
+    return general_image(*pl.G, pl.V, &pl.d_general, pl.tables_async ? &st : nullptr);
+}
 
 // The plan's device block of tables: stream-ordered for a plan that lives
 // inside one call, else allocated and uploaded when the plan is made.
@@ -418,13 +424,13 @@ static int upload_tables(su_plan &pl, const std::vector<unsigned char> &blob) {
 }
 
 static void free_tables(su_plan &pl) {
-    if (pl.d_tables && pl.tables_async)
-        cudaFreeAsync(pl.d_tables, (cudaStream_t)pl.opt.stream);
-    else if (pl.d_tables)
-        cudaFree(pl.d_tables);
-    pl.d_tables = nullptr;
-    if (pl.d_general) cudaFree(pl.d_general);
-    pl.d_general = nullptr;
+    for (void **p : {&pl.d_tables, &pl.d_general}) {
+        if (*p && pl.tables_async)
+            cudaFreeAsync(*p, (cudaStream_t)pl.opt.stream);
+        else if (*p)
+            cudaFree(*p);
+        *p = nullptr;
+    }
 }
 
 // The level tables of a plan (rows d = 0..S-1 for levels n = S..1), each
@@ -480,75 +486,23 @@ static int plan_rounds(su_plan &pl, int rounds, int sms, int smem_max) {
     return occ;
 }
 
-// The general potential's program split by size (general_split): the level's
-// single-precision entries (times the factorials that the kernel's derivatives
-// are short of), and its double part's nodes and entries, behind the tables.
+// The general potential's program split by size (general_split), its images
+// behind the tables.
 static void split_general(su_plan &pl, std::vector<unsigned char> &blob, int smem_max) {
     using namespace su;
     SamplerParams &P = pl.P;
-    const GeneralEffective &G = *pl.G;
-    const int S = pl.s, M = P.M;
-    const size_t nn = G.depth.size();
-    const std::vector<double> tab(reinterpret_cast<const double *>(blob.data()),
-                                  reinterpret_cast<const double *>(blob.data()) + (size_t)S * M);
-    std::vector<double> ms, fact(nn, 1.0), fs((size_t)G.J + 1, 1.0), stk((size_t)G.J + 3 * G.p + 2, 1.0);
-    general_moments(G, pl.V, pl.a, pl.b, pl.T, ms);
-    for (int j = 2; j <= G.J; ++j) fs[(size_t)j] = fs[(size_t)j - 1] * j;
-    for (size_t t = 1; t < nn; ++t) {
-        fact[t] = stk[(size_t)G.depth[t] - 1] * fs[(size_t)G.sym[t]];
-        stk[(size_t)G.depth[t]] = fact[t];
-    }
-    std::vector<float> tail((size_t)S * M, 0.0f);
-    std::vector<GeneralNode> hnodes;
-    std::vector<double> hcoef;
-    std::vector<int> head;
-    bool any = false;
-    for (int d = 0; d < pl.levels; ++d) {
-        const double *t = tab.data() + (size_t)d * M;
-        P.gs.lim[d] = (float)(kGenReach * general_split(G, ms, pl.a, pl.b, pl.T, S - d, t, head));
-        int total = 0;
-        bool fits = true;
-        for (size_t k = 0; k < nn; ++k) {
-            total += head[k];
-            for (int e = head[k]; e < G.count[k]; ++e) {
-                const double c = t[G.first[k] + e] * fact[k];
-                fits = fits && std::fabs(c) < 1e30;
-                tail[(size_t)d * M + G.first[k] + e] = (float)c;
-            }
-        }
-        if (!fits || total == 0 || 2 * total > M) continue;
-        // the nodes with entries and their ancestors, in order
-        std::vector<char> keep(nn, 0);
-        std::vector<size_t> path((size_t)kGenMaxDepth + 1, 0);
-        for (size_t k = 0; k < nn; ++k) {
-            path[(size_t)G.depth[k]] = k;
-            if (head[k])
-                for (int q = 0; q <= G.depth[k]; ++q) keep[path[(size_t)q]] = 1;
-        }
-        P.gs.h0[d] = (int)hnodes.size();
-        P.gs.hc[d] = (int)hcoef.size();
-        for (size_t k = 0; k < nn; ++k) {
-            if (!keep[k] && k) continue;
-            hnodes.push_back({(unsigned char)G.depth[k], (unsigned char)G.sym[k], (unsigned short)head[k],
-                              (int)hcoef.size() - P.gs.hc[d]});
-            for (int e = 0; e < head[k]; ++e) hcoef.push_back(t[G.first[k] + e]);
-            if (k) P.gs.hj[d] = std::max(P.gs.hj[d], G.sym[k]);
-        }
-        P.gs.hn[d] = (int)hnodes.size() - P.gs.h0[d];
-        any = true;
-    }
-    if (!any) return;
+    GeneralImages im;
+    if (!general_split(*pl.G, pl.V, pl.a, pl.b, pl.T, pl.s, pl.levels, reinterpret_cast<const double *>(blob.data()), P.gs, im))
+        return;
     auto put = [&](const void *src, size_t bytes) {
         const size_t at = (blob.size() + 15) / 16 * 16;
         blob.resize(at + bytes);
         if (bytes) std::memcpy(blob.data() + at, src, bytes);
         return (int64_t)at;
     };
-    P.gs.on = 1;
-    P.gs.n_nodes = (int)nn;
-    P.gs.tail = put(tail.data(), tail.size() * sizeof(float));
-    P.gs.hnodes = put(hnodes.data(), hnodes.size() * sizeof(GeneralNode));
-    P.gs.hcoef = put(hcoef.data(), hcoef.size() * sizeof(double));
+    P.gs.tail = put(im.tail.data(), im.tail.size() * sizeof(float));
+    P.gs.hnodes = put(im.hnodes.data(), im.hnodes.size() * sizeof(GeneralNode));
+    P.gs.hcoef = put(im.hcoef.data(), im.hcoef.size() * sizeof(double));
     // program and entries in shared memory where four CTAs still fit an SM
     P.gs.staged = 1;
     if (sampler_smem_bytes(P, SU_FP64) > (size_t)std::min(smem_max, 56 * 1024)) P.gs.staged = 0;
@@ -615,12 +569,7 @@ static int plan_shape(su_plan &pl, int sms, int smem_max, std::vector<unsigned c
             std::memcpy(blob.data() + P.fx.tail_off, tail.data(), tail.size() * sizeof(float));
         }
     }
-    // the split pays for its preparation (0.1 to 0.3 ms) from some 1.5e8 entries
-    // evaluated (about 0.5 ms as a whole program)
-    constexpr double kSplitLeast = 1.5e8;
-    const double entries = (double)pl.n_mc * ((pl.levels > 1 ? 2.0 : 1.0) * (double)((int64_t)1 << S)) * P.M;
-    if (general && prec == SU_FP64 && S >= 1 && !P.wf_on && !P.generic && pl.opt.seg_log2 == 0 && pl.opt.rounds == 0 &&
-        entries >= kSplitLeast)
+    if (general && prec == SU_FP64 && S >= 1 && !P.wf_on && !P.generic && pl.opt.seg_log2 == 0 && pl.opt.rounds == 0)
         split_general(pl, blob, smem_max);
     // launch shape: one path per thread, persistent grid over items of
     // 128 * rounds samples

@@ -6,83 +6,214 @@
 // power of vs^2 from a step's second moment.  The smallest entries whose sum
 // stays below 2^-33 of the level's weight go to single precision (their error
 // there is a few 2^-24); of every node the double part takes the leading powers
-// up to the last large one, and with it the node's ancestors.
+// up to the last large one, and with it the node's ancestors.  (These are typical
+// sizes; what a path has is summed by the kernel, and limited there.)
+//
+// The choice depends on the estimator alone, not on how many samples a call has,
+// so that a run's parts have the run's weights.  It takes 0.02 ms (p = 4) to 0.2 ms
+// (p = 12, eight levels) of the host.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "sampler.h"
 
 namespace su {
 
-void general_moments(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T,
-                     std::vector<double> &ms) {
+namespace {
+
+constexpr int kTimes = 8, kPts = 16;   // 7 times, 16 positions to 6 standard deviations
+constexpr double kStep = 12.0 / kPts;
+constexpr int kOctaves = 400;
+
+// Root mean squares over the bridge of the program's monomials (ms) and of the
+// derivatives (ds), the positions of successive times shifted against each other.
+void moments(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T, std::vector<double> &ms,
+             std::vector<double> &ds) {
     const size_t nn = G.depth.size();
-    constexpr int times = 8, half = 8;   // 7 times, 17 positions to 6 standard deviations
-    constexpr double dg = 6.0 / half;
+    const int J = G.J;
     ms.assign(nn, 0.0);
-    std::vector<double> D((size_t)G.J + 1), stk((size_t)G.J + 3 * G.p + 2, 1.0);
-    for (int k = 1; k < times; ++k) {
-        const double u = (double)k / times, mean = a + (b - a) * u, sd = std::sqrt(T * u * (1 - u));
-        for (int g = -half; g <= half; ++g) {
-            const double wgt = std::exp(-0.5 * g * g * dg * dg) * (dg / std::sqrt(2 * 3.14159265358979323846)) / (times - 1);
-            general_derivatives(V, mean + sd * g * dg, G.J, D.data());
-            for (size_t t = 0; t < nn; ++t) {
-                double mu = 1.0;
-                if (t) {
-                    mu = stk[(size_t)G.depth[t] - 1] * D[(size_t)G.sym[t]];
-                    stk[(size_t)G.depth[t]] = mu;
-                }
-                ms[t] += wgt * mu * mu;
+    ds.assign((size_t)J + 1, 0.0);
+    using Row = double[kPts];
+    std::vector<double> buf((size_t)(2 * J + 3 + G.J + 3 * G.p + 2) * kPts);
+    Row *D = reinterpret_cast<Row *>(buf.data()), *t = D + J + 1, *stk = t + J + 2;
+    for (int k = 1; k < kTimes; ++k) {
+        const double u = (double)k / kTimes, mean = a + (b - a) * u, sd = std::sqrt(T * u * (1 - u));
+        Row x, wgt;
+        for (int i = 0; i < kPts; ++i) {
+            const double g = kStep * (i - 0.5 * (kPts - 1) + (k - 0.5 * kTimes) / kTimes);
+            x[i] = mean + sd * g;
+            wgt[i] = std::exp(-0.5 * g * g) * (kStep / std::sqrt(2 * 3.14159265358979323846)) / (kTimes - 1);
+        }
+        for (int j = 0; j <= J; ++j)
+            for (int i = 0; i < kPts; ++i) D[j][i] = 0.0;
+        double der[9];
+        std::copy(V.a, V.a + 9, der);
+        for (int j = 0; j <= std::min(J, 8); ++j) {   // der: the coefficients of the j-th derivative
+            for (int q = 8 - j; q >= 0; --q)
+                for (int i = 0; i < kPts; ++i) D[j][i] = D[j][i] * x[i] + der[q];
+            for (int q = 0; q < 8 - j; ++q) der[q] = der[q + 1] * (q + 1);
+            der[8 - j] = 0.0;
+        }
+        for (int f = 0; f < V.ng; ++f) {
+            // (d/dx)^n A e^{-beta u^2}: D_{n+1} = -2 beta (u D_n + n D_{n-1})
+            const double A = V.gauss[f][0], beta = V.gauss[f][1], c = V.gauss[f][2];
+            Row y, d0, d1;
+            for (int i = 0; i < kPts; ++i) {
+                const double v = x[i] - c;
+                y[i] = -2.0 * beta * v;
+                d0[i] = 0.0;
+                d1[i] = A * std::exp(-beta * v * v);
             }
+            for (int n = 0; n <= J; ++n)
+                for (int i = 0; i < kPts; ++i) {
+                    D[n][i] += d1[i];
+                    const double d2 = y[i] * d1[i] - 2.0 * beta * n * d0[i];
+                    d0[i] = d1[i];
+                    d1[i] = d2;
+                }
+        }
+        for (int f = 0; f < V.ns; ++f) {
+            // Taylor coefficients of tanh, (n+1) t_{n+1} = -sum_k t_k t_{n-k}; sech^2 = tanh'
+            const double alpha = V.sech[f][1], d = V.sech[f][2];
+            for (int i = 0; i < kPts; ++i) {
+                const double w = alpha * (x[i] - d), ch = std::cosh(w);
+                t[0][i] = std::tanh(w);
+                t[1][i] = 1.0 / (ch * ch);
+            }
+            double sc = V.sech[f][0];   // B alpha^n (n+1)!
+            for (int n = 0; n <= J; ++n) {
+                if (n) {
+                    Row acc = {};
+                    for (int q = 0; q < (n + 1) / 2; ++q)
+                        for (int i = 0; i < kPts; ++i) acc[i] += t[q][i] * t[n - q][i];
+                    const double even = n & 1 ? 0.0 : 1.0;
+                    for (int i = 0; i < kPts; ++i)
+                        t[n + 1][i] = (2.0 * acc[i] + even * (t[n / 2][i] * t[n / 2][i])) * (-1.0 / (n + 1));
+                }
+                sc *= (double)(n + 1);
+                for (int i = 0; i < kPts; ++i) D[n][i] += sc * t[n + 1][i];
+                sc *= alpha;
+            }
+        }
+        for (int f = 0; f < V.ne; ++f) {
+            Row e;
+            for (int i = 0; i < kPts; ++i) e[i] = V.expo[f][0] * std::exp(-V.expo[f][1] * (x[i] - V.expo[f][2]));
+            for (int n = 0; n <= J; ++n)
+                for (int i = 0; i < kPts; ++i) {
+                    D[n][i] += e[i];
+                    e[i] *= -V.expo[f][1];
+                }
+        }
+        for (int j = 0; j <= J; ++j)
+            for (int i = 0; i < kPts; ++i) ds[(size_t)j] += wgt[i] * (D[j][i] * D[j][i]);
+        for (int i = 0; i < kPts; ++i) {
+            stk[0][i] = 1.0;
+            ms[0] += wgt[i];
+        }
+        for (size_t q = 1; q < nn; ++q) {
+            const double *up = stk[G.depth[q] - 1], *s = D[G.sym[q]];
+            double *mu = stk[G.depth[q]], sum[4] = {};
+            for (int i = 0; i < kPts; i += 4)
+                for (int r = 0; r < 4; ++r) {
+                    const double m = up[i + r] * s[i + r];
+                    mu[i + r] = m;
+                    sum[r] += wgt[i + r] * (m * m);
+                }
+            ms[q] += (sum[0] + sum[1]) + (sum[2] + sum[3]);
         }
     }
     for (double &v : ms) v = std::sqrt(v);
+    for (double &v : ds) v = std::sqrt(v);
 }
 
-double general_split(const GeneralEffective &G, const std::vector<double> &ms, double a, double b, double T, int n,
-                     const double *table, std::vector<int> &head) {
-    const double N = std::ldexp(1.0, n), eps = T / N, s2 = eps + (b - a) * (b - a) / (N * N);
-    std::vector<double> my((size_t)G.K, 1.0);
-    for (int k = 1; k < G.K; ++k) my[(size_t)k] = my[(size_t)k - 1] * s2 * std::sqrt((4.0 * k - 1) * (4.0 * k - 3));
-    const size_t nn = G.depth.size();
-    std::vector<double> size(G.entry_k.size());
-    double all = 0;
-    for (size_t t = 0; t < nn; ++t)
-        for (int k = 0; k < G.count[t]; ++k) {
-            const size_t e = (size_t)G.first[t] + (size_t)k;
-            all += size[e] = std::fabs(table[e]) * ms[t] * my[(size_t)k];
-        }
-    if (!std::isfinite(all)) {   // sizes beyond a double: nothing to split by
-        head.assign(G.count.begin(), G.count.end());
-        return 0;
+}  // namespace
+
+bool general_split(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T, int S, int levels,
+                   const double *tables, GeneralSplit &gs, GeneralImages &im) {
+    const size_t nn = G.depth.size(), M = G.entry_k.size();
+    std::vector<double> ms, ds, fact(nn, 1.0), fs((size_t)G.J + 1, 1.0), stk((size_t)G.J + 3 * G.p + 2, 1.0);
+    moments(G, V, a, b, T, ms, ds);
+    for (int j = 2; j <= G.J; ++j) fs[(size_t)j] = fs[(size_t)j - 1] * j;
+    for (size_t t = 1; t < nn; ++t) {
+        fact[t] = stk[(size_t)G.depth[t] - 1] * fs[(size_t)G.sym[t]];
+        stk[(size_t)G.depth[t]] = fact[t];
     }
-    // the smallest entries up to the sum: whole octaves, then the last one's in order
-    const double most = 0x1p-33 * std::min(1.0, N * all) / N;
-    constexpr int kOctaves = 400;
-    auto octave = [](double v) { return v > 0 ? std::max(0, std::min(kOctaves - 1, std::ilogb(v) + 300)) : 0; };
-    std::vector<double> sum(kOctaves, 0.0);
-    for (double v : size) sum[(size_t)octave(v)] += v;
-    double rest = 0;
-    int oct = 0;
-    while (oct < kOctaves && rest + sum[(size_t)oct] <= most) rest += sum[(size_t)oct++];
-    std::vector<double> last;
-    for (double v : size)
-        if (octave(v) == oct) last.push_back(v);
-    std::sort(last.begin(), last.end());
-    double least = 0;   // of the large ones
-    for (double v : last) {
-        least = v;
-        if (rest + v > most) break;
-        rest += v;
-    }
-    head.assign(nn, 0);
-    for (size_t t = 0; t < nn; ++t)
-        for (int k = 0; k < G.count[t]; ++k) {
-            const double v = size[(size_t)G.first[t] + (size_t)k];
-            const int o = octave(v);
-            if (o > oct || (o == oct && v >= least)) head[t] = k + 1;
+    im.tail.assign((size_t)S * M, 0.0f);
+    std::vector<double> size(M);
+    std::vector<int> head(nn), bin(M);
+    std::vector<size_t> path((size_t)kGenMaxDepth + 1, 0);
+    std::vector<char> keep(nn);
+    bool any = false;
+    for (int d = 0; d < levels; ++d) {
+        const double *table = tables + (size_t)d * M;
+        const double N = std::ldexp(1.0, S - d), eps = T / N, s2 = eps + (b - a) * (b - a) / (N * N);
+        std::vector<double> my((size_t)G.K, 1.0);
+        for (int k = 1; k < G.K; ++k) my[(size_t)k] = my[(size_t)k - 1] * s2 * std::sqrt((4.0 * k - 1) * (4.0 * k - 3));
+        double all = 0;
+        for (size_t t = 0; t < nn; ++t)
+            for (int k = 0; k < G.count[t]; ++k) {
+                const size_t e = (size_t)G.first[t] + (size_t)k;
+                all += size[e] = std::fabs(table[e]) * ms[t] * my[(size_t)k];
+            }
+        if (!std::isfinite(all)) continue;   // sizes beyond a double: nothing to split by
+        // the smallest entries up to the sum: whole octaves (powers of two, down to
+        // 2^-300), then sixty-fourths of the next one
+        const double most = 0x1p-33 * std::min(1.0, N * all) / N;
+        double sum[kOctaves] = {}, part[64] = {};
+        for (size_t e = 0; e < M; ++e) {
+            int64_t bits;
+            std::memcpy(&bits, &size[e], 8);
+            bin[e] = std::max(0, std::min(64 * kOctaves - 1, (int)(bits >> 46) - 64 * (1023 - 300)));
+            sum[bin[e] / 64] += size[e];
         }
-    return N * most;
+        double rest = 0;
+        int oct = 0, sub = 0;
+        while (oct < kOctaves && rest + sum[oct] <= most) rest += sum[oct++];
+        for (size_t e = 0; e < M; ++e)
+            if (bin[e] / 64 == oct) part[bin[e] % 64] += size[e];
+        while (sub < 64 && rest + part[sub] <= most) rest += part[sub++];
+        const int first = 64 * oct + sub;   // of the large ones
+        int total = 0;
+        for (size_t t = 0; t < nn; ++t) {
+            head[t] = 0;
+            for (int k = 0; k < G.count[t]; ++k)
+                if (bin[(size_t)G.first[t] + (size_t)k] >= first) head[t] = k + 1;
+            total += head[t];
+        }
+        // worth it where the double part is short; the others have to be floats
+        bool fits = total > 0 && 2 * total <= (int)M;
+        for (size_t t = 0; fits && t < nn; ++t)
+            for (int k = head[t]; k < G.count[t]; ++k) {
+                const size_t e = (size_t)G.first[t] + (size_t)k;
+                const double c = table[e] * fact[t];
+                fits = fits && std::fabs(c) < 1e30;
+                im.tail[(size_t)d * M + e] = (float)c;
+            }
+        if (!fits) continue;
+        // the nodes with entries and their ancestors, in order
+        std::fill(keep.begin(), keep.end(), 0);
+        for (size_t t = 0; t < nn; ++t) {
+            path[(size_t)G.depth[t]] = t;
+            if (head[t])
+                for (int q = 0; q <= G.depth[t]; ++q) keep[path[(size_t)q]] = 1;
+        }
+        gs.h0[d] = (int)im.hnodes.size();
+        gs.hc[d] = (int)im.hcoef.size();
+        for (size_t t = 0; t < nn; ++t) {
+            if (!keep[t] && t) continue;
+            im.hnodes.push_back({(unsigned char)G.depth[t], (unsigned char)G.sym[t], (unsigned short)head[t],
+                                 (int)im.hcoef.size() - gs.hc[d]});
+            for (int k = 0; k < head[t]; ++k) im.hcoef.push_back(table[(size_t)G.first[t] + (size_t)k]);
+            if (t) gs.hj[d] = std::max(gs.hj[d], G.sym[t]);
+        }
+        gs.hn[d] = (int)im.hnodes.size() - gs.h0[d];
+        gs.lim[d] = (float)(kGenReach * N * most);
+        any = true;
+    }
+    gs.on = any;
+    gs.n_nodes = (int)nn;
+    return any;
 }
 
 }  // namespace su

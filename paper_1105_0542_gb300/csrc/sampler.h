@@ -116,13 +116,18 @@ struct SamplerParams {
     FxParams fx;                // double precision: the fixed-point sampler where fx.on
 };
 
-// root mean squares of the general program's monomials over the bridge
-void general_moments(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T,
-                     std::vector<double> &ms);
-// head[t] = the leading entries of node t that need double precision on level n;
-// the bound of the others' root mean squares, summed over the path
-double general_split(const GeneralEffective &G, const std::vector<double> &ms, double a, double b, double T, int n,
-                     const double *table, std::vector<int> &head);
+// The split of the general program (rows of entries for levels n = S..1, the
+// first `levels` of them): fills gs but its offsets, and the images that belong
+// there -- the single-precision entries [S][M] (times the factorials that the
+// kernel's derivatives are short of), the double parts' nodes and entries.
+// False (gs.on = 0) where no level has a short enough double part.  Host work.
+struct GeneralImages {
+    std::vector<float> tail;
+    std::vector<GeneralNode> hnodes;
+    std::vector<double> hcoef;
+};
+bool general_split(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T, int S, int levels,
+                   const double *tables, GeneralSplit &gs, GeneralImages &im);
 constexpr double kGenReach = 8;
 
 // The fixed-point plan of a double-precision plan's tables (rows of M entries,

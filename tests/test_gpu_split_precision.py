@@ -120,3 +120,19 @@ def test_general_split_far_from_the_origin():
     w = {k: _general(V, 999.5, 1000.7, 0.25, 8, 7, 20_000, kernel=k) for k in ("auto", "generic")}
     assert np.any(w["auto"][:, -1] != w["generic"][:, -1])
     assert np.all(np.abs(w["auto"] - w["generic"]) <= 2.0 ** -50 * np.maximum(1.0, np.abs(w["generic"])))
+
+
+@pytest.mark.parametrize("s,n", [(6, 12_000), (4, 3000)])
+def test_general_weights_do_not_depend_on_the_sample_count(s, n):
+    """A run in parts by sample0, and one sample of it, have the run's weights
+    bit for bit; so has the top level without the others."""
+    args = (MORSE, 0.0, 0.6, 0.2, 10, s)
+    w = _general(*args, n, sample0=FAR[0] - 100, seed=1234)
+    g = _general(*args, n, sample0=FAR[0] - 100, seed=1234, kernel="generic")
+    assert np.any(w != g)   # the split ran
+    for lo, hi in ((0, 90), (90, n // 2), (n // 2, n), (100, 101)):
+        assert np.array_equal(_general(*args, hi - lo, sample0=FAR[0] - 100 + lo, seed=1234), w[lo:hi])
+    par = su.general_params(MORSE["poly"], (), (), MORSE["expo"])
+    run = [su.speedup_amplitude("general", par, 0.0, 0.6, 0.2, 10, s, n, 1234, sample0=FAR[0] - 100, n_blocks=8, hierarchy=h)
+           for h in (True, False)]
+    assert run[0][s]["amp"] == run[1][s]["amp"] and run[0][s]["err"] == run[1][s]["err"]
