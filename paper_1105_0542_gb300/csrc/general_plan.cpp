@@ -132,29 +132,70 @@ void moments(const GeneralEffective &G, const GeneralPotential &V, double a, dou
 bool general_split(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T, int S, int levels,
                    const double *tables, GeneralSplit &gs, GeneralImages &im) {
     const size_t nn = G.depth.size(), M = G.entry_k.size();
+    // the potential's parameters as floats, far enough inside their range
+    bool floats = true;
+    auto param = [&](double v) { floats = floats && (v == 0.0 || (std::fabs(v) >= 0x1p-100 && std::fabs(v) <= 0x1p100)); };
+    for (double v : V.a) param(v);
+    for (int f = 0; f < V.ng; ++f) param(V.gauss[f][0]), param(V.gauss[f][1]);
+    for (int f = 0; f < V.ns; ++f) param(V.sech[f][0]), param(V.sech[f][1]);
+    for (int f = 0; f < V.ne; ++f) param(V.expo[f][0]), param(V.expo[f][1]);
+    if (!floats) return false;
+    // sizes in units in which the path is about one across (lengths 2^unit, energies
+    // 4^-unit), so that their squares are doubles: deg = the power of 2^-unit of a monomial
+    const int unit = std::ilogb(std::sqrt(T));
+    GeneralPotential U = V;
+    for (int i = 0; i <= 8; ++i) U.a[i] = std::ldexp(U.a[i], unit * (i + 2));
+    for (int f = 0; f < V.ng; ++f) {
+        U.gauss[f][0] = std::ldexp(U.gauss[f][0], 2 * unit);
+        U.gauss[f][1] = std::ldexp(U.gauss[f][1], 2 * unit);
+        U.gauss[f][2] = std::ldexp(U.gauss[f][2], -unit);
+    }
+    for (auto fam : {U.sech, U.expo})
+        for (int f = 0; f < (fam == U.sech ? V.ns : V.ne); ++f) {
+            fam[f][0] = std::ldexp(fam[f][0], 2 * unit);
+            fam[f][1] = std::ldexp(fam[f][1], unit);
+            fam[f][2] = std::ldexp(fam[f][2], -unit);
+        }
+    std::vector<int> deg(nn, 0), sdeg((size_t)G.J + 3 * G.p + 2, 0);
+    for (size_t t = 1; t < nn; ++t) deg[t] = sdeg[(size_t)G.depth[t]] = sdeg[(size_t)G.depth[t] - 1] + G.sym[t] + 2;
     std::vector<double> ms, ds, fact(nn, 1.0), fs((size_t)G.J + 1, 1.0), stk((size_t)G.J + 3 * G.p + 2, 1.0);
-    moments(G, V, a, b, T, ms, ds);
+    moments(G, U, std::ldexp(a, -unit), std::ldexp(b, -unit), std::ldexp(T, -2 * unit), ms, ds);
     for (int j = 2; j <= G.J; ++j) fs[(size_t)j] = fs[(size_t)j - 1] * j;
     for (size_t t = 1; t < nn; ++t) {
         fact[t] = stk[(size_t)G.depth[t] - 1] * fs[(size_t)G.sym[t]];
         stk[(size_t)G.depth[t]] = fact[t];
     }
+    // the kernel's monomials (of derivatives over j!), and the smallest and largest
+    // factor or partial product on the way to each, in typical size
+    const bool near = std::abs(unit) * (2 * G.K + *std::max_element(deg.begin(), deg.end())) < 500;   // no power of the unit overflows
+    std::vector<double> mono(nn, 1.0), mu(nn, 1.0), lo(nn, 1.0), hi(nn, 1.0), slo(stk.size(), 1.0), shi(stk.size(), 1.0);
+    for (size_t t = 1; t < nn; ++t) {
+        const size_t at = (size_t)G.depth[t];
+        const double u = std::ldexp(ds[(size_t)G.sym[t]] / fs[(size_t)G.sym[t]], -unit * (G.sym[t] + 2));
+        mono[t] = std::ldexp(ms[t], -unit * deg[t]);
+        mu[t] = mono[t] / fact[t];
+        lo[t] = slo[at] = std::min(slo[at - 1], std::min(u, mu[t]));
+        hi[t] = shi[at] = std::max(shi[at - 1], std::max(u, mu[t]));
+    }
     im.tail.assign((size_t)S * M, 0.0f);
-    std::vector<double> size(M);
+    std::vector<double> size(M), my((size_t)G.K, 1.0), yk(my);
     std::vector<int> head(nn), bin(M);
     std::vector<size_t> path((size_t)kGenMaxDepth + 1, 0);
     std::vector<char> keep(nn);
     bool any = false;
     for (int d = 0; d < levels; ++d) {
         const double *table = tables + (size_t)d * M;
-        const double N = std::ldexp(1.0, S - d), eps = T / N, s2 = eps + (b - a) * (b - a) / (N * N);
-        std::vector<double> my((size_t)G.K, 1.0);
+        const double N = std::ldexp(1.0, S - d), step = std::ldexp(b - a, -unit) / N;
+        const double s2 = std::ldexp(T, -2 * unit) / N + step * step;
         for (int k = 1; k < G.K; ++k) my[(size_t)k] = my[(size_t)k - 1] * s2 * std::sqrt((4.0 * k - 1) * (4.0 * k - 3));
+        for (int k = 0; k < G.K; ++k) yk[(size_t)k] = std::ldexp(my[(size_t)k], 2 * unit * k);
         double all = 0;
         for (size_t t = 0; t < nn; ++t)
             for (int k = 0; k < G.count[t]; ++k) {
                 const size_t e = (size_t)G.first[t] + (size_t)k;
-                all += size[e] = std::fabs(table[e]) * ms[t] * my[(size_t)k];
+                const double v = std::fabs(table[e]);
+                size[e] = near ? v * mono[t] * yk[(size_t)k] : std::ldexp(v, unit * (2 * k - deg[t])) * ms[t] * my[(size_t)k];
+                all += size[e];
             }
         if (!std::isfinite(all)) continue;   // sizes beyond a double: nothing to split by
         // the smallest entries up to the sum: whole octaves (powers of two, down to
@@ -174,23 +215,33 @@ bool general_split(const GeneralEffective &G, const GeneralPotential &V, double 
             if (bin[e] / 64 == oct) part[bin[e] % 64] += size[e];
         while (sub < 64 && rest + part[sub] <= most) rest += part[sub++];
         const int first = 64 * oct + sub;   // of the large ones
+        // Entries that a float's range does not hold (units in which the potential's
+        // derivatives or the step are far from one) are large ones too: those whose
+        // factors overflow, or lose what counts -- more than a float's rounding of the
+        // others -- where one falls below 2^-126.  Entries that do not count are left out.
+        const double none = 0x1p-24 * most / (double)M;
+        auto in_floats = [&](size_t t, int k, size_t e) {
+            const double c = std::fabs(table[e]) * fact[t], cy = c * yk[(size_t)k];
+            return std::max(c, std::max(cy, hi[t])) <= 0x1p100 && 0x1p-126 * mu[t] * std::max(1.0, yk[(size_t)k]) <= none &&
+                   0x1p-126 * (mu[t] / lo[t]) * cy <= none;
+        };
         int total = 0;
         for (size_t t = 0; t < nn; ++t) {
             head[t] = 0;
-            for (int k = 0; k < G.count[t]; ++k)
-                if (bin[(size_t)G.first[t] + (size_t)k] >= first) head[t] = k + 1;
+            for (int k = 0; k < G.count[t]; ++k) {
+                const size_t e = (size_t)G.first[t] + (size_t)k;
+                if (bin[e] >= first || (!in_floats(t, k, e) && size[e] > none)) head[t] = k + 1;
+            }
             total += head[t];
         }
-        // worth it where the double part is short; the others have to be floats
-        bool fits = total > 0 && 2 * total <= (int)M;
-        for (size_t t = 0; fits && t < nn; ++t)
+        // worth it where the double part is short
+        const bool fits = total > 0 && 2 * total <= (int)M;
+        if (!fits) continue;
+        for (size_t t = 0; t < nn; ++t)
             for (int k = head[t]; k < G.count[t]; ++k) {
                 const size_t e = (size_t)G.first[t] + (size_t)k;
-                const double c = table[e] * fact[t];
-                fits = fits && std::fabs(c) < 1e30;
-                im.tail[(size_t)d * M + e] = (float)c;
+                if (in_floats(t, k, e)) im.tail[(size_t)d * M + e] = (float)(table[e] * fact[t]);
             }
-        if (!fits) continue;
         // the nodes with entries and their ancestors, in order
         std::fill(keep.begin(), keep.end(), 0);
         for (size_t t = 0; t < nn; ++t) {

@@ -136,3 +136,20 @@ def test_general_weights_do_not_depend_on_the_sample_count(s, n):
     run = [su.speedup_amplitude("general", par, 0.0, 0.6, 0.2, 10, s, n, 1234, sample0=FAR[0] - 100, n_blocks=8, hierarchy=h)
            for h in (True, False)]
     assert run[0][s]["amp"] == run[1][s]["amp"] and run[0][s]["err"] == run[1][s]["err"]
+
+
+@pytest.mark.parametrize("V,p,e", [(QUARTIC, 7, -8), (QUARTIC, 5, -12), (NARROW, 7, 12), (MORSE, 10, -4), (MORSE, 10, 40)],
+                         ids=["quartic-8", "quartic-12", "narrow+12", "morse-4", "morse+40"])
+def test_general_split_in_other_units(V, p, e):
+    """Lengths in units of 2^e (times of 4^e, energies of 4^-e): the weights
+    are those of e = 0, whatever of the derivatives a float's range holds.
+    What the split's guard lets through, and both programs' sums of 512 slices,
+    are a few 2^-50 of a weight."""
+    u = 2.0 ** e
+    U = dict(poly=tuple(c * u ** -(i + 2) for i, c in enumerate(V["poly"])),
+             gauss=[(A / u ** 2, beta / u ** 2, c * u) for A, beta, c in V.get("gauss", ())],
+             expo=[(E / u ** 2, kappa / u, x * u) for E, kappa, x in V.get("expo", ())])
+    n = {5: 6510, 7: 1825, 10: 500}[p]
+    w = _general(U, -0.4 * u, 0.6 * u, 0.2 * u * u, p, 9, n)
+    g = _general(V, -0.4, 0.6, 0.2, p, 9, n, kernel="generic")
+    assert np.all(np.abs(w - g) <= 2.0 ** -48 * np.maximum(1.0, np.abs(g)))
