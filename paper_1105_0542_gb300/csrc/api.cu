@@ -719,6 +719,7 @@ static int configure_nd(su_plan &pl) {
     Q.one = 1;
     NdProgram G;
     std::vector<int> every((size_t)M), heads;
+    std::vector<char> part;
     for (int i = 0; i < M; ++i) every[(size_t)i] = i;
     nd_order(pl.N.mono, nv, Q.order);
     nd_program(pl.N.mono, every, nv, Q.order, G);
@@ -733,32 +734,30 @@ static int configure_nd(su_plan &pl) {
     std::vector<uint32_t> hwords;
     std::vector<double> hcoef;
     for (int d = 0; d < S; ++d) {
-        std::vector<char> in_double((size_t)M, 0);
+        part.assign((size_t)M, kNdFloat);
         if (prec == SU_FP64 && d < pl.levels && pl.opt.kernel == 0) {
-            nd_split(pl.N.mono, pl.nd, pl.nd_a.data(), pl.nd_b.data(), pl.T, S - d,
-                     std::vector<double>(tabd.begin() + (long)d * M, tabd.begin() + (long)(d + 1) * M), heads);
-            // worth it where the double part is short; the others have to be floats
-            std::vector<char> head((size_t)M, 0);
-            for (int e : heads) head[(size_t)e] = 1;
-            bool fits = !heads.empty() && 2 * heads.size() <= (size_t)M;
-            for (int e = 0; e < M; ++e) fits = fits && (head[(size_t)e] || std::fabs(scaled(d, e)) < 1e30);
-            if (fits) {
+            const double bound = nd_split(pl.N.mono, pl.nd, pl.nd_a.data(), pl.nd_b.data(), pl.T, S - d, tabd.data() + (size_t)d * M, part);
+            heads.clear();
+            for (int e = 0; e < M; ++e)
+                if (part[(size_t)e] == kNdDouble) heads.push_back(e);
+            // worth it where the double part is short
+            if (!heads.empty() && 2 * heads.size() <= (size_t)M) {
                 NdProgram H;
                 nd_program(pl.N.mono, heads, nv, Q.order, H);
                 Q.heads[d] = (int)heads.size();
+                Q.lim[d] = (float)(kNdReach * bound);
                 Q.hsq[d] = H.sq;
                 Q.hw[d] = (int)hwords.size();
                 Q.hc[d] = (int)hcoef.size();
                 hwords.insert(hwords.end(), H.words.begin(), H.words.end());
                 for (int e : H.slot) hcoef.push_back(e < 0 ? 0.0 : scaled(d, e));
-                for (int e : heads) in_double[(size_t)e] = 1;
             }
         }
         for (int i = 0; i < Mp; ++i) {
             const int e = G.slot[(size_t)i];
             if (e < 0) continue;
             full[(size_t)d * Mp + i] = scaled(d, e);
-            pairs[2 * ((size_t)d * Mp + i)] = pairs[2 * ((size_t)d * Mp + i) + 1] = in_double[(size_t)e] ? 0.0f : (float)scaled(d, e);
+            pairs[2 * ((size_t)d * Mp + i)] = pairs[2 * ((size_t)d * Mp + i) + 1] = part[(size_t)e] != kNdFloat ? 0.0f : (float)scaled(d, e);
         }
     }
     int sms = 0, smem_max = 0;
@@ -811,7 +810,6 @@ static int configure_nd(su_plan &pl) {
     for (int c = 0; c < pl.nd; ++c) {
         Q.a[c] = pl.nd_a[(size_t)c];
         Q.b[c] = pl.nd_b[(size_t)c];
-        Q.reach[c] = std::max(std::fabs(Q.a[c]), std::fabs(Q.b[c])) + 2.4 * std::sqrt(pl.T);
     }
     // program and tables in shared memory where that leaves the register-bound residency
     Q.staged = 1;

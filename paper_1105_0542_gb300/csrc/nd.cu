@@ -92,6 +92,8 @@ __device__ __forceinline__ void nd_poly(const uint32_t *__restrict__ &w, const V
     }
 }
 
+constexpr float kNdTail = 0x1p-28f;   // largest single-precision part of a weight beyond one, as lim of one up to it
+
 // x (rounded to nearest) for |x| < 2^127 as a float, on the integer pipes
 __device__ __forceinline__ float narrow(double x) {
     const uint64_t u = (uint64_t)__double_as_longlong(x);
@@ -101,9 +103,10 @@ __device__ __forceinline__ float narrow(double x) {
 }
 __device__ __forceinline__ float narrow(float x) { return x; }
 
-// the sum of 2 BP slices' -eps W in single precision (points pt(k0 stp).. of R)
+// the sum of 2 BP slices' -eps W in single precision (points pt(k0 stp).. of R), and
+// the sum of its magnitudes
 template <typename R, int D, int BP, typename PT>
-__device__ __forceinline__ float nd_single(const NdParams &Q, const uint32_t *w, const float2 *c, PT &&pt, int k0, int stp) {
+__device__ __forceinline__ float2 nd_single(const NdParams &Q, const uint32_t *w, const float2 *c, PT &&pt, int k0, int stp) {
     Vars<float2, 2 * D, BP> v;
 #pragma unroll
     for (int k = 0; k < 2 * D; ++k) {
@@ -121,10 +124,13 @@ __device__ __forceinline__ float nd_single(const NdParams &Q, const uint32_t *w,
     v.close(Q.sq, Q.one);
     float2 t[BP];
     nd_poly<0>(w, c, v, t);
-    float s = 0;
+    float s = 0, m = 0;
 #pragma unroll
-    for (int i = 0; i < BP; ++i) s += t[i].x + t[i].y;
-    return s;
+    for (int i = 0; i < BP; ++i) {
+        s += t[i].x + t[i].y;
+        m += fabsf(t[i].x) + fabsf(t[i].y);
+    }
+    return make_float2(s, m);
 }
 
 // B slices' -eps W in double
@@ -250,17 +256,11 @@ __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __gr
                 }
             };
             R wloc[SU_MAX_S];
-            // pass 0 with the split levels; again with every level in double
-            // for a path that leaves the split's reach
+            // pass 0 with the split levels; again in double for the levels whose
+            // single-precision part is beyond Q.lim
+            uint32_t todo = (1u << L) - 1u, far = 0;
             for (int pass = 0; pass < 2; ++pass) {
-                bool far = false;
-                auto seen = [&](R v, int c) {
-                    if constexpr (sizeof(R) == 8) {
-                        const int hi = __double2hiint(v) & 0x7fffffff;
-                        far |= hi > __double2hiint(Q.reach[c]);
-                    }
-                    return v;
-                };
+                float mag[sizeof(R) == 8 ? SU_MAX_S : 1];
                 // coarse levels n = 1..S-F: midpoint i at segment endpoint (2i+1) 2^(S-F-n)
                 have = 0xffffffffu;
                 for (int c = 0; c < D; ++c) {
@@ -273,33 +273,38 @@ __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __gr
                     for (int i = 0; i < (1 << (n - 1)); ++i) {
                         const int idx = (2 * i + 1) * h;
                         for (int c = 0; c < D; ++c)
-                            co(idx, c) = seen(fma(sg, normal((uint32_t)((j0 + i) * D + c)), (R)0.5 * (co(idx - h, c) + co(idx + h, c))), c);
+                            co(idx, c) = fma(sg, normal((uint32_t)((j0 + i) * D + c)), (R)0.5 * (co(idx - h, c) + co(idx + h, c)));
                     }
                 }
                 // w_n = -eps_n sum_k W on the level-n subpath (level n = S - dl),
                 // slices in ascending order, several at a time
-                for (int dl = 0; dl < L; ++dl) wloc[dl] = 0;
+                for (int dl = 0; dl < L; ++dl) {
+                    if (todo >> dl & 1u) wloc[dl] = 0;
+                    if constexpr (sizeof(R) == 8) mag[dl] = 0;
+                }
                 auto slices = [&](int dl, auto &&pt, int stp, int ns) {
+                    if (sizeof(R) == 8 && !(todo >> dl & 1u)) return;
                     R w = 0;
                     if constexpr (sizeof(R) == 4) {
                         const float2 *c = pairs + (size_t)dl * P.M;
                         if (ns >= 2 * kBP) {
 #pragma unroll 1
-                            for (int k = 0; k < ns; k += 2 * kBP) w += nd_single<R, D, kBP>(Q, words, c, pt, k, stp);
+                            for (int k = 0; k < ns; k += 2 * kBP) w += nd_single<R, D, kBP>(Q, words, c, pt, k, stp).x;
                         } else {
 #pragma unroll 1
-                            for (int k = 0; k < ns; k += 2) w += nd_single<R, D, 1>(Q, words, c, pt, k, stp);
+                            for (int k = 0; k < ns; k += 2) w += nd_single<R, D, 1>(Q, words, c, pt, k, stp).x;
                         }
                     } else if (pass == 0 && Q.heads[dl] > 0) {
                         const float2 *c = pairs + (size_t)dl * P.M;
-                        float tail = 0;
+                        float2 tail = make_float2(0.f, 0.f);
                         if (ns >= 2 * kBP) {
 #pragma unroll 1
-                            for (int k = 0; k < ns; k += 2 * kBP) tail += nd_single<R, D, kBP>(Q, words, c, pt, k, stp);
+                            for (int k = 0; k < ns; k += 2 * kBP) tail = __fadd2_rn(tail, nd_single<R, D, kBP>(Q, words, c, pt, k, stp));
                         } else {
 #pragma unroll 1
-                            for (int k = 0; k < ns; k += 2) tail += nd_single<R, D, 1>(Q, words, c, pt, k, stp);
+                            for (int k = 0; k < ns; k += 2) tail = __fadd2_rn(tail, nd_single<R, D, 1>(Q, words, c, pt, k, stp));
                         }
+                        mag[dl] += tail.y;
                         if (kBD > 2 && ns >= kBD) {
 #pragma unroll 1
                             for (int k = 0; k < ns; k += kBD)
@@ -309,7 +314,7 @@ __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __gr
                             for (int k = 0; k < ns; k += 2)
                                 w += nd_double<D, 2>(Q, Q.hsq[dl], hwords + Q.hw[dl], hcoef + Q.hc[dl], pt, k, stp);
                         }
-                        w += (double)tail;
+                        w += (double)tail.x;
                     } else {
 #pragma unroll 1
                         for (int k = 0; k < ns; k += 2)
@@ -335,13 +340,19 @@ __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __gr
                         for (int il = 0; il < m; ++il) {
                             const int idx = (2 * il + 1) * h;
                             for (int c = 0; c < D; ++c)
-                                fp(idx, c) = seen(fma(sg, normal((uint32_t)((j0 + il) * D + c)), (R)0.5 * (fp(idx - h, c) + fp(idx + h, c))), c);
+                                fp(idx, c) = fma(sg, normal((uint32_t)((j0 + il) * D + c)), (R)0.5 * (fp(idx - h, c) + fp(idx + h, c)));
                         }
                     }
 #pragma unroll 1
                     for (int dl = 0; dl < min(F, L); ++dl) slices(dl, fp, 1 << dl, NF >> dl);
                 }
-                if (!far) break;
+                if constexpr (sizeof(R) == 8) {
+                    if (pass == 0)
+                        for (int dl = 0; dl < L; ++dl)
+                            if (Q.heads[dl] > 0 && !(mag[dl] <= fmaxf(Q.lim[dl], kNdTail * fabsf(__double2float_rn(wloc[dl]))))) far |= 1u << dl;
+                }
+                todo = far;
+                if (pass || !far) break;
             }
             bool bad = false;
             for (int dl = 0; dl < L; ++dl) bad |= isnan(wloc[dl]) || (isinf(wloc[dl]) && wloc[dl] > 0);

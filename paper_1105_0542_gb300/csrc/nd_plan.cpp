@@ -14,9 +14,10 @@
 //
 // Split (double).  Entries whose root mean square over the bridge is small are
 // left to single precision: what rounding them to floats costs, 2^-25 of their
-// sum, adds up over the N slices and stays below 2^-55 of the level's weight.
-// The others form a program of their own, evaluated in double.  A path that
-// leaves max(|a|, |b|) + 2.4 sqrt(T) in a coordinate (probability 2e-5) is
+// sum, adds up over the N slices to 2^-55 of the level's typical weight.  The
+// others form a program of their own, evaluated in double.  These are typical
+// sizes: what a path's slices have is summed by the kernel, and a level on which
+// that passes four times the plan's bound (one path in some ten thousand) is
 // weighed by the whole program in double.
 #include <algorithm>
 #include <cmath>
@@ -131,9 +132,11 @@ static std::vector<double> moments(double a, double b, double T, int top) {
     return m;
 }
 
-void nd_split(const std::vector<Mono> &mono, int D, const double *a, const double *b, double T, int n,
-              const std::vector<double> &table, std::vector<int> &heads) {
-    const double N = std::ldexp(1.0, n), eps = T / N;
+double nd_split(const std::vector<Mono> &mono, int D, const double *a, const double *b, double T, int n,
+                const double *table, std::vector<char> &part) {
+    const size_t M = mono.size();
+    const double N = std::ldexp(1.0, n);
+    const double eps = T / N;
     std::vector<std::vector<double>> mx((size_t)D), mb((size_t)D);
     for (int c = 0; c < D; ++c) {
         int tx = 0, tb = 0;
@@ -147,21 +150,30 @@ void nd_split(const std::vector<Mono> &mono, int D, const double *a, const doubl
         for (int f = 1; f <= tb; ++f) mb[c][f] = mb[c][f - 1] * std::sqrt(s2 * (2.0 * f - 1));   // E g^2f = (2f - 1)!!
     }
     std::vector<std::pair<double, int>> r;
+    std::vector<int> deg(M, 0);
     double all = 0;
-    for (size_t i = 0; i < mono.size(); ++i) {
+    for (size_t i = 0; i < M; ++i) {
         double v = std::fabs(table[i]);
-        for (int c = 0; c < D; ++c) v *= mx[c][mono[i][(size_t)c]] * mb[c][mono[i][(size_t)(D + c)]];
+        for (int c = 0; c < D; ++c) {
+            v *= mx[c][mono[i][(size_t)c]] * mb[c][mono[i][(size_t)(D + c)]];
+            deg[i] += mono[i][(size_t)c] + mono[i][(size_t)(D + c)];
+        }
         r.emplace_back(v, (int)i);
         all += v;
     }
+    part.assign(M, kNdDouble);
+    if (!std::isfinite(all)) return 0;
     std::sort(r.begin(), r.end());
     // N 2^-25 rest <= 2^-55 min(1, N all)
     const double most = 0x1p-30 * std::min(1.0, N * all) / N;
     double rest = 0;
-    heads.clear();
     size_t k = 0;
-    for (; k < r.size() && rest + r[k].first <= most; ++k) rest += r[k].first;
-    for (; k < r.size(); ++k) heads.push_back(r[k].second);
+    for (; k < M && rest + r[k].first <= most; ++k) rest += r[k].first;
+    for (size_t q = 0; q < k; ++q) {
+        const size_t i = (size_t)r[q].second;
+        if (std::ldexp(std::fabs(table[i]), -deg[i]) < 1e30) part[i] = kNdFloat;
+    }
+    return N * most;
 }
 
 }  // namespace su

@@ -247,9 +247,12 @@ struct NdProgram {
 void nd_order(const std::vector<std::vector<unsigned char>> &mono, int nv, int *order);
 void nd_program(const std::vector<std::vector<unsigned char>> &mono, const std::vector<int> &pick, int nv,
                 const int *order, NdProgram &G);
-// the entries of a level's table that need double precision
-void nd_split(const std::vector<std::vector<unsigned char>> &mono, int D, const double *a, const double *b, double T,
-              int n, const std::vector<double> &table, std::vector<int> &heads);
+// Where the entries of level n's table go (part: one of these each); the bound of
+// the single-precision ones' root mean squares, summed over the path
+enum : char { kNdFloat = 0, kNdDouble = 1 };   // single precision, double
+double nd_split(const std::vector<std::vector<unsigned char>> &mono, int D, const double *a, const double *b, double T,
+                int n, const double *table, std::vector<char> &part);
+constexpr double kNdReach = 4;
 
 struct NdParams {
     SamplerParams base;       // S, levels, M = coefficients of the program per level, sigma, stream, items, outputs
@@ -267,7 +270,7 @@ struct NdParams {
     int n_hwords, n_hcoef;
     int heads[SU_MAX_S], hw[SU_MAX_S], hc[SU_MAX_S];   // row d: its double entries, first word, first coefficient
     unsigned hsq[SU_MAX_S];
-    double reach[kNdMaxDim];  // |q_c| beyond which the path is weighed in double
+    float lim[SU_MAX_S];      // largest sum of the slices' single-precision parts over a path (kNdReach times the plan's)
     int staged;               // program and tables in shared memory
     unsigned one;             // 1
     double a[kNdMaxDim], b[kNdMaxDim];

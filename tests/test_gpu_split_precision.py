@@ -153,3 +153,41 @@ def test_general_split_in_other_units(V, p, e):
     w = _general(U, -0.4 * u, 0.6 * u, 0.2 * u * u, p, 9, n)
     g = _general(V, -0.4, 0.6, 0.2, p, 9, n, kernel="generic")
     assert np.all(np.abs(w - g) <= 2.0 ** -48 * np.maximum(1.0, np.abs(g)))
+
+
+AHO2 = {(2, 0): 0.5, (4, 0): 1 / 24, (2, 2): 1 / 12, (0, 2): 0.5, (0, 4): 1 / 24}
+AHO3 = {(2, 0, 0): 0.5, (0, 2, 0): 0.5, (0, 0, 2): 0.5, (4, 0, 0): 1 / 24, (0, 4, 0): 1 / 24, (0, 0, 4): 1 / 24,
+        (2, 2, 0): 1 / 12, (2, 0, 2): 1 / 12, (0, 2, 2): 1 / 12}
+TWO = {(2, 0, 0, 0): 0.5, (0, 2, 0, 0): 0.5, (0, 0, 2, 0): 0.5, (0, 0, 0, 2): 0.5, (2, 0, 2, 0): 0.1, (1, 0, 1, 0): -0.2,
+       (0, 1, 0, 1): -0.2, (0, 2, 0, 2): 0.1}
+ENDS = {1: ((0.2,), (-0.4,)), 2: ((0.0, 0.0), (1.0, 0.5)), 3: ((0.0, 0.0, 0.0), (1.0, 0.5, -0.5)),
+        4: ((0.3, 0.0, -0.3, 0.1), (0.2, 0.4, -0.1, -0.2))}
+
+
+def _nd(V, T, p, s, n, sample0=0, seed=1234, u=1.0, **kw):
+    out = torch.zeros((n, s), dtype=torch.float64, device="cuda")
+    a, b = ENDS[len(next(iter(V)))]
+    su.speedup_logweights_nd({m: c * u ** -(sum(m) + 2) for m, c in V.items()}, tuple(x * u for x in a),
+                             tuple(x * u for x in b), T * u * u, p, s, sample0, n, seed, out, precision="fp64", **kw)
+    torch.cuda.synchronize()
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("V,T,p,s", [({(3,): 0.1, (2,): 0.5}, 0.5, 9, 6), (AHO2, 1.0, 10, 7), (AHO3, 1.0, 8, 5), (TWO, 1.0, 6, 6)],
+                         ids=["1", "2", "3", "4"])
+def test_nd_split_matches_the_whole_program(V, T, p, s):
+    """One to four coordinates at levels that split: a few 2^-50 of a weight
+    between the two programs (the guard's 2^-28 in single precision, 2^-24 of
+    it a few times over, and the sums)."""
+    w = {k: _nd(V, T, p, s, 1111, kernel=k) for k in ("auto", "generic")}
+    assert np.any(w["auto"][:, -1] != w["generic"][:, -1])
+    assert np.all(np.abs(w["auto"] - w["generic"]) <= 2.0 ** -48 * np.maximum(1.0, np.abs(w["generic"])))
+
+
+@pytest.mark.parametrize("V,p,s,level,sample", [(AHO2, 10, 4, 3, 3424844), (AHO2, 10, 4, 3, 1061362), (TWO, 6, 6, 5, 2883140)])
+def test_nd_level_beyond_the_split_is_weighed_by_the_whole_program(V, p, s, level, sample):
+    """Samples of seed 1234 inside 2.4 sqrt(T) of the endpoints with unusually
+    large steps on one level: the weight there is the whole program's, bit for
+    bit, while the neighbours' are the split's."""
+    same = _nd(V, 1.0, p, s, 100, sample0=sample - 50) == _nd(V, 1.0, p, s, 100, sample0=sample - 50, kernel="generic")
+    assert same[50, level - 1] and not same[:, level - 1].all()
