@@ -736,7 +736,7 @@ static int configure_nd(su_plan &pl) {
     for (int d = 0; d < S; ++d) {
         part.assign((size_t)M, kNdFloat);
         if (prec == SU_FP64 && d < pl.levels && pl.opt.kernel == 0) {
-            const double bound = nd_split(pl.N.mono, pl.nd, pl.nd_a.data(), pl.nd_b.data(), pl.T, S - d, tabd.data() + (size_t)d * M, part);
+            nd_split(pl.N.mono, pl.nd, pl.nd_a.data(), pl.nd_b.data(), pl.T, S - d, tabd.data() + (size_t)d * M, part);
             heads.clear();
             for (int e = 0; e < M; ++e)
                 if (part[(size_t)e] == kNdDouble) heads.push_back(e);
@@ -745,7 +745,6 @@ static int configure_nd(su_plan &pl) {
                 NdProgram H;
                 nd_program(pl.N.mono, heads, nv, Q.order, H);
                 Q.heads[d] = (int)heads.size();
-                Q.lim[d] = (float)(kNdReach * bound);
                 Q.hsq[d] = H.sq;
                 Q.hw[d] = (int)hwords.size();
                 Q.hc[d] = (int)hcoef.size();

@@ -9,11 +9,10 @@
 // busy), most of them the derivatives that the large entries need; the packed program
 // hides behind them.  Two features, p = 10, N = 64, 200 001 samples: 62.4 -> 24.7 ms.
 //
-// A level of a path whose single-precision entries are too large in sum -- 2^-30 of
-// the smaller of one and the level's typical weight, or of a weight beyond one --
-// (narrow features that the plan's moments missed, paths far out) is weighed again
-// by the whole program in double: a few 2^-24 of the entries stay below a double's
-// rounding of the weight's exponential.
+// A level of a path whose single-precision entries are too large in sum, 2^-30 of
+// max(1, |w|) (narrow features that the plan's moments missed, paths far out), is
+// weighed again by the whole program in double: a few 2^-24 of the entries stay
+// below what a double's rounding does to exp(w).
 #include <cstdint>
 
 #include "sampler_impl.cuh"
@@ -22,7 +21,7 @@ namespace su {
 namespace {
 
 constexpr int kGenSeg = 5;   // the path in segments of 2^5 slices
-constexpr float kGenTail = 0x1p-30f;   // largest single-precision part of a weight beyond one, as lim of one up to it
+constexpr float kGenTail = 0x1p-30f;   // largest sum of the single-precision entries' magnitudes, of max(1, |w|)
 
 // V^(j)(x) / j!, j = 0..J, of two slices.  (A feature's offset from x is taken in
 // double: far from the origin a rounded x would be off by a part of the feature.)
@@ -272,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, 4) general_kernel(const __grid_const
                 for (int d = 0; d < L; ++d)
                     if (pass == 0 && P.gs.hn[d] > 0) {
                         w[d] += (double)tsum[d];
-                        if (!(tmag[d] <= fmaxf(P.gs.lim[d], kGenTail * fabsf(__double2float_rn(w[d]))))) far |= 1u << d;
+                        if (!(tmag[d] <= kGenTail * fmaxf(1.0f, fabsf(__double2float_rn(w[d]))))) far |= 1u << d;
                     }
                 todo = far;
             }

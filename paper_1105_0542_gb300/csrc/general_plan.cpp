@@ -259,7 +259,6 @@ bool general_split(const GeneralEffective &G, const GeneralPotential &V, double 
             if (t) gs.hj[d] = std::max(gs.hj[d], G.sym[t]);
         }
         gs.hn[d] = (int)im.hnodes.size() - gs.h0[d];
-        gs.lim[d] = (float)(kGenReach * N * most);
         any = true;
     }
     gs.on = any;

@@ -92,7 +92,13 @@ __device__ __forceinline__ void nd_poly(const uint32_t *__restrict__ &w, const V
     }
 }
 
-constexpr float kNdTail = 0x1p-28f;   // largest single-precision part of a weight beyond one, as lim of one up to it
+// The largest sum of the slices' single-precision parts over a path, of max(1, |w|):
+// typically below 2^-30, where what single precision rounds is below 2^-55; at the
+// limit some 2^-50 (the entries are two to four times their slices' sums).  Beyond
+// it, about one path in a million, the second pass takes the path's own lane 7.5 ms
+// (two coordinates, p = 10, one level of 512 slices), so that a limit of 2^-28
+// doubled the time of a call of 50 001 such paths.
+constexpr float kNdTail = 0x1p-27f;
 
 // x (rounded to nearest) for |x| < 2^127 as a float, on the integer pipes
 __device__ __forceinline__ float narrow(double x) {
@@ -257,7 +263,7 @@ __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __gr
             };
             R wloc[SU_MAX_S];
             // pass 0 with the split levels; again in double for the levels whose
-            // single-precision part is beyond Q.lim
+            // single-precision part is beyond kNdTail
             uint32_t todo = (1u << L) - 1u, far = 0;
             for (int pass = 0; pass < 2; ++pass) {
                 float mag[sizeof(R) == 8 ? SU_MAX_S : 1];
@@ -349,7 +355,7 @@ __global__ void __launch_bounds__(kThreads, D == 3 ? 3 : 4) nd_kernel(const __gr
                 if constexpr (sizeof(R) == 8) {
                     if (pass == 0)
                         for (int dl = 0; dl < L; ++dl)
-                            if (Q.heads[dl] > 0 && !(mag[dl] <= fmaxf(Q.lim[dl], kNdTail * fabsf(__double2float_rn(wloc[dl]))))) far |= 1u << dl;
+                            if (Q.heads[dl] > 0 && !(mag[dl] <= kNdTail * fmaxf(1.0f, fabsf(__double2float_rn(wloc[dl]))))) far |= 1u << dl;
                 }
                 todo = far;
                 if (pass || !far) break;

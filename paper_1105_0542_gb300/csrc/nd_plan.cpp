@@ -17,8 +17,7 @@
 // sum, adds up over the N slices to 2^-55 of the level's typical weight.  The
 // others form a program of their own, evaluated in double.  These are typical
 // sizes: what a path's slices have is summed by the kernel, and a level on which
-// that passes four times the plan's bound (one path in some ten thousand) is
-// weighed by the whole program in double.
+// that passes 2^-27 of max(1, |w|) is weighed by the whole program in double.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -132,8 +131,8 @@ static std::vector<double> moments(double a, double b, double T, int top) {
     return m;
 }
 
-double nd_split(const std::vector<Mono> &mono, int D, const double *a, const double *b, double T, int n,
-                const double *table, std::vector<char> &part) {
+void nd_split(const std::vector<Mono> &mono, int D, const double *a, const double *b, double T, int n,
+              const double *table, std::vector<char> &part) {
     const size_t M = mono.size();
     const double N = std::ldexp(1.0, n);
     const double eps = T / N;
@@ -162,7 +161,7 @@ double nd_split(const std::vector<Mono> &mono, int D, const double *a, const dou
         all += v;
     }
     part.assign(M, kNdDouble);
-    if (!std::isfinite(all)) return 0;
+    if (!std::isfinite(all)) return;
     std::sort(r.begin(), r.end());
     // N 2^-25 rest <= 2^-55 min(1, N all)
     const double most = 0x1p-30 * std::min(1.0, N * all) / N;
@@ -173,7 +172,6 @@ double nd_split(const std::vector<Mono> &mono, int D, const double *a, const dou
         const size_t i = (size_t)r[q].second;
         if (std::ldexp(std::fabs(table[i]), -deg[i]) < 1e30) part[i] = kNdFloat;
     }
-    return N * most;
 }
 
 }  // namespace su

@@ -69,14 +69,11 @@ struct FxParams {
 
 // The split general program (general.cu; built by general_split): byte offsets
 // from the tables, and per level (row d) the double part's nodes, entries and
-// highest derivative (hn = 0: the whole program in double), and the largest sum of
-// the single-precision entries' magnitudes over a path (lim; kGenReach times the
-// plan's estimate).
+// highest derivative (hn = 0: the whole program in double).
 struct GeneralSplit {
     int on, staged, n_nodes;
     int64_t tail, hnodes, hcoef;
     int hn[SU_MAX_S], h0[SU_MAX_S], hc[SU_MAX_S], hj[SU_MAX_S];
-    float lim[SU_MAX_S];
 };
 
 struct SamplerParams {
@@ -128,7 +125,6 @@ struct GeneralImages {
 };
 bool general_split(const GeneralEffective &G, const GeneralPotential &V, double a, double b, double T, int S, int levels,
                    const double *tables, GeneralSplit &gs, GeneralImages &im);
-constexpr double kGenReach = 8;
 
 // The fixed-point plan of a double-precision plan's tables (rows of M entries,
 // kernel_table's, for levels n = S..1): fills P.fx (on = 0 where the ranges do
@@ -247,12 +243,10 @@ struct NdProgram {
 void nd_order(const std::vector<std::vector<unsigned char>> &mono, int nv, int *order);
 void nd_program(const std::vector<std::vector<unsigned char>> &mono, const std::vector<int> &pick, int nv,
                 const int *order, NdProgram &G);
-// Where the entries of level n's table go (part: one of these each); the bound of
-// the single-precision ones' root mean squares, summed over the path
+// where the entries of level n's table go (part: one of these each)
 enum : char { kNdFloat = 0, kNdDouble = 1 };   // single precision, double
-double nd_split(const std::vector<std::vector<unsigned char>> &mono, int D, const double *a, const double *b, double T,
-                int n, const double *table, std::vector<char> &part);
-constexpr double kNdReach = 4;
+void nd_split(const std::vector<std::vector<unsigned char>> &mono, int D, const double *a, const double *b, double T,
+              int n, const double *table, std::vector<char> &part);
 
 struct NdParams {
     SamplerParams base;       // S, levels, M = coefficients of the program per level, sigma, stream, items, outputs
@@ -270,7 +264,6 @@ struct NdParams {
     int n_hwords, n_hcoef;
     int heads[SU_MAX_S], hw[SU_MAX_S], hc[SU_MAX_S];   // row d: its double entries, first word, first coefficient
     unsigned hsq[SU_MAX_S];
-    float lim[SU_MAX_S];      // largest sum of the slices' single-precision parts over a path (kNdReach times the plan's)
     int staged;               // program and tables in shared memory
     unsigned one;             // 1
     double a[kNdMaxDim], b[kNdMaxDim];
