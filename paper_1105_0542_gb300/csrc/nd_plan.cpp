@@ -135,29 +135,49 @@ void nd_split(const std::vector<Mono> &mono, int D, const double *a, const doubl
               const double *table, std::vector<char> &part) {
     const size_t M = mono.size();
     const double N = std::ldexp(1.0, n);
-    const double eps = T / N;
+    // in units in which the path is about one across (lengths 2^unit)
+    const int unit = std::ilogb(std::sqrt(T));
+    const double Tu = std::ldexp(T, -2 * unit), eps = Tu / N;
     std::vector<std::vector<double>> mx((size_t)D), mb((size_t)D);
     for (int c = 0; c < D; ++c) {
-        int tx = 0, tb = 0;
+        int tx = 1, tb = 1;
         for (const Mono &m : mono) {
             tx = std::max(tx, (int)m[(size_t)c]);
             tb = std::max(tb, (int)m[(size_t)(D + c)]);
         }
-        mx[c] = moments(a[c], b[c], T, tx);
-        const double s2 = 0.25 * (eps + (b[c] - a[c]) * (b[c] - a[c]) / (N * N));
+        const double au = std::ldexp(a[c], -unit), bu = std::ldexp(b[c], -unit);
+        mx[c] = moments(au, bu, Tu, tx);
+        const double s2 = 0.25 * (eps + (bu - au) * (bu - au) / (N * N));
         mb[c].assign((size_t)tb + 1, 1.0);
         for (int f = 1; f <= tb; ++f) mb[c][f] = mb[c][f - 1] * std::sqrt(s2 * (2.0 * f - 1));   // E g^2f = (2f - 1)!!
     }
-    std::vector<std::pair<double, int>> r;
+    // the kernel's variables (2 x, 2 xb) in typical size: their powers above one, and
+    // whether their squares are floats
+    std::vector<double> big[2 * kNdMaxDim];
+    bool square[2 * kNdMaxDim];
+    for (int v = 0; v < 2 * D; ++v) {
+        const std::vector<double> &m = v < D ? mx[(size_t)v] : mb[(size_t)(v - D)];
+        const double z = std::ldexp(m[1], unit + 1);
+        square[v] = z >= 0x1p-60 && z <= 0x1p60;
+        big[v].assign(m.size(), 1.0);
+        for (size_t e = 1; e < m.size(); ++e) big[v][e] = big[v][e - 1] * std::max(1.0, z);
+    }
+    std::vector<std::pair<double, int>> r(M);
+    std::vector<double> hi(M, 1.0);
+    std::vector<char> floats(M, 1);
     std::vector<int> deg(M, 0);
     double all = 0;
     for (size_t i = 0; i < M; ++i) {
-        double v = std::fabs(table[i]);
+        double v = 1.0;
         for (int c = 0; c < D; ++c) {
-            v *= mx[c][mono[i][(size_t)c]] * mb[c][mono[i][(size_t)(D + c)]];
-            deg[i] += mono[i][(size_t)c] + mono[i][(size_t)(D + c)];
+            const size_t x = mono[i][(size_t)c], xb = mono[i][(size_t)(D + c)];
+            v *= mx[c][x] * mb[c][xb];
+            hi[i] *= big[c][x] * big[D + c][xb];
+            deg[i] += (int)(x + xb);
+            if ((x && !square[c]) || (xb && !square[D + c])) floats[i] = 0;
         }
-        r.emplace_back(v, (int)i);
+        v *= unit ? std::ldexp(std::fabs(table[i]), unit * deg[i]) : std::fabs(table[i]);
+        r[i] = {v, (int)i};
         all += v;
     }
     part.assign(M, kNdDouble);
@@ -168,9 +188,17 @@ void nd_split(const std::vector<Mono> &mono, int D, const double *a, const doubl
     double rest = 0;
     size_t k = 0;
     for (; k < M && rest + r[k].first <= most; ++k) rest += r[k].first;
+    // Of these, what a float's range does not hold stays in double (a partial product
+    // below 2^-126 loses at most that times the factors to come), or does not count:
+    // less than a float's rounding of the others.
+    const double none = 0x1p-24 * most / (double)M;
     for (size_t q = 0; q < k; ++q) {
         const size_t i = (size_t)r[q].second;
-        if (std::ldexp(std::fabs(table[i]), -deg[i]) < 1e30) part[i] = kNdFloat;
+        const double c = std::ldexp(std::fabs(table[i]), -deg[i]);
+        if (floats[i] && std::max(1.0, c) * hi[i] <= 0x1p100 && 0x1p-126 * hi[i] <= none)
+            part[i] = kNdFloat;
+        else if (r[q].first <= none)
+            part[i] = kNdNone;
     }
 }
 

@@ -244,7 +244,7 @@ void nd_order(const std::vector<std::vector<unsigned char>> &mono, int nv, int *
 void nd_program(const std::vector<std::vector<unsigned char>> &mono, const std::vector<int> &pick, int nv,
                 const int *order, NdProgram &G);
 // where the entries of level n's table go (part: one of these each)
-enum : char { kNdFloat = 0, kNdDouble = 1 };   // single precision, double
+enum : char { kNdFloat = 0, kNdDouble = 1, kNdNone = 2 };   // single precision, double, too small to count
 void nd_split(const std::vector<std::vector<unsigned char>> &mono, int D, const double *a, const double *b, double T,
               int n, const double *table, std::vector<char> &part);
 

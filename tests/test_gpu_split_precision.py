@@ -192,3 +192,12 @@ def test_nd_level_beyond_the_split_is_weighed_by_the_whole_program(p):
     at = 227961
     same = _nd(AHO2, 0.5, p, 9, 100, sample0=at - 50) == _nd(AHO2, 0.5, p, 9, 100, sample0=at - 50, kernel="generic")
     assert same[50, 8] and not same[:, 8].all() and not same[50].all()
+
+
+@pytest.mark.parametrize("V,p,e", [(AHO2, 8, 12), (AHO2, 8, 24), (AHO3, 8, 12), (TWO, 6, 18), (TWO, 6, 36), (AHO2, 8, -12), (TWO, 6, -40)])
+def test_nd_split_in_other_units(V, p, e):
+    """Lengths in units of 2^e: the weights are those of e = 0, whatever of the
+    table's entries a float's range holds."""
+    w = _nd(V, 0.5, p, 6, 1000, u=2.0 ** e)
+    g = _nd(V, 0.5, p, 6, 1000, kernel="generic")
+    assert np.all(np.abs(w - g) <= 2.0 ** -48 * np.maximum(1.0, np.abs(g)))
