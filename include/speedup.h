@@ -96,11 +96,14 @@ typedef struct {
     int rounds;           /* launch shape: paths per thread per work item, 1..8;
                              0 (default) = automatic.  Automatic = the shape
                              su_autotune stored for this precision, model, p and s
-                             in this process, else the built-in rule (seg_log2 =
+                             in this process, for calls whose ranges and tables
+                             give the same sampler as the tuned call's (see
+                             kernel), else the built-in rule (seg_log2 =
                              4 for SU_FP64, 5 for SU_FP32, capped at s; rounds =
                              1, doubled while the per-item tuples would exceed
                              512 MB and as many CTAs stay resident).  The shape
-                             changes the order of the floating-point sums only. */
+                             changes the order of the floating-point sums, and an
+                             explicit seg_log2 also the sampler (kernel). */
     int kernel;           /* 0 (default): a single-precision plan with 32-slice
                              segments whose level tables have a shape compiled
                              into the library (the even-ring shapes of the
@@ -110,11 +113,15 @@ typedef struct {
                              sampler.  Both give the same results bit for bit.
                              In double precision 0 also takes the fixed-point
                              sampler where the ranges of a, b, T and the tables
-                             allow it (even polynomial potentials, automatic
-                             segments), and several-coordinates and general
-                             potentials evaluate the small entries of their
-                             programs in single precision; 1 never does.
-                             They agree to a double's rounding. */
+                             allow it (even polynomial and Poeschl-Teller
+                             potentials, 2^4-slice segments), and
+                             several-coordinates and (with automatic seg_log2)
+                             general potentials evaluate the small entries of
+                             their programs in single precision; 1 never does.
+                             The choice depends on the estimator (potential, p,
+                             s, a, b, T), not on the samples.  Per-sample weights
+                             agree to a double's rounding, rms 2^-53 of
+                             max(1, |w|); single weights to some 2^-50. */
 } su_options;
 
 /* per bisection level n = 0..s (N = 2^n slices) */

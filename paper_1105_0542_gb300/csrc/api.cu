@@ -37,15 +37,24 @@ namespace {
 
 thread_local std::string g_err;
 
-// launch shapes stored by su_autotune, per (precision, model, p, s)
+// The kernels of a one-coordinate plan: which of them its ranges, tables and
+// options give it decides what a launch shape means.
+enum PlanKernel : int { kWhole = 0, kFixedPoint = 1, kSplit = 2 };
+
+// launch shapes stored by su_autotune, per (precision, model, p, s) and the
+// kernel of a plan with automatic shape; each with the kernel that it was timed on
 struct TuneKey {
-    int precision, model, p, s;
+    int precision, model, p, s, kernel;
     bool operator<(const TuneKey &o) const {
-        return std::tie(precision, model, p, s) < std::tie(o.precision, o.model, o.p, o.s);
+        return std::tie(precision, model, p, s, kernel) < std::tie(o.precision, o.model, o.p, o.s, o.kernel);
     }
 };
+struct Tuned {
+    su_tuning shape;
+    int kernel;
+};
 std::mutex g_tune_mu;
-std::map<TuneKey, su_tuning> g_tune;
+std::map<TuneKey, Tuned> g_tune;
 
 // register segments stored by su_batch_autotune, per (precision, model, p, s, hierarchy)
 struct BatchTuneKey {
@@ -56,9 +65,9 @@ struct BatchTuneKey {
 };
 std::map<BatchTuneKey, int> g_btune;
 
-bool tuned_shape(int precision, int model, int p, int s, su_tuning &out) {
+bool tuned_shape(const TuneKey &key, Tuned &out) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune.find({precision, model, p, s});
+    auto it = g_tune.find(key);
     if (it == g_tune.end()) return false;
     out = it->second;
     return true;
@@ -203,6 +212,9 @@ struct su_plan {
     int64_t n_blocks = 1;
     su::SamplerParams P{};
     void *d_tables = nullptr;
+    int kernel = 0;              // PlanKernel (one coordinate)
+    bool tuned = true;           // automatic shape: what su_autotune stored, where it did
+    bool fixed_point = true;     // the fixed-point sampler where its plan fits
     bool tables_async = false;   // d_tables and d_general are stream-ordered on opt.stream (a plan inside one call)
     int device = 0;
     int grid = 0;
@@ -522,14 +534,12 @@ static int plan_shape(su_plan &pl, int sms, int smem_max, std::vector<unsigned c
     P.a = pl.a;
     P.b = pl.b;
     for (int n = 1; n <= S; ++n) P.sigma[n] = pl.opt.width_factor * std::sqrt(pl.T / std::ldexp(1.0, n + 1));
-    // launch shape: explicit, else stored by su_autotune, else the rule
-    su_tuning tuned{};
-    const bool have_tuned = tuned_shape(prec, pl.model, pl.p, S, tuned);
+    // segments: explicit, else the rule (what su_autotune stored: below)
     // rule: 16-slice register segments in double (measured 1-5 % faster than
     // 32 at 2 CTAs per SM), 32 in single precision and for the general
     // potential (4 CTAs per SM; 32 beat 8 and 16 by 25 % and 11 % at N = 1024)
     const int seg_rule = (general || prec != SU_FP64) ? kMaxFine : 4;
-    int seg = pl.opt.seg_log2 > 0 ? pl.opt.seg_log2 : (have_tuned ? tuned.seg_log2 : seg_rule);
+    const int seg = pl.opt.seg_log2 > 0 ? pl.opt.seg_log2 : seg_rule;
     P.S = S;
     P.F = std::min(S, std::max(1, seg));
     P.levels = pl.levels;
@@ -547,16 +557,23 @@ static int plan_shape(su_plan &pl, int sms, int smem_max, std::vector<unsigned c
     P.sample0 = pl.opt.sample0;
     P.n_blocks = pl.n_blocks;
 
-    // tables too large to stage next to the rest (the highest levels) are
-    // read from global memory instead
     P.rounds = 1;
     P.tab_global = 0;
     P.generic = pl.opt.kernel == 1;
-    if (sampler_smem_bytes(P, prec) > (size_t)smem_max) {
-        if (prec != SU_FP64) return fail(SU_ENOTSUP, "the level tables do not fit shared memory in single precision");
-        P.tab_global = 1;
-    }
-    if (prec == SU_FP64 && !general) {
+    // tables too large to stage next to the rest (the highest levels) are
+    // read from global memory instead
+    auto stage_tables = [&] {
+        P.tab_global = 0;
+        if (sampler_smem_bytes(P, prec) > (size_t)smem_max) {
+            if (prec != SU_FP64) return fail(SU_ENOTSUP, "the level tables do not fit shared memory in single precision");
+            P.tab_global = 1;
+        }
+        return (int)SU_OK;
+    };
+    int rc = stage_tables();
+    if (rc) return rc;
+    const size_t tables_end = blob.size();
+    if (prec == SU_FP64 && !general && pl.fixed_point) {
         std::vector<int64_t> head;
         std::vector<float> tail;
         su::fx_plan(P, pl.T, reinterpret_cast<const double *>(blob.data()), head, tail);
@@ -569,8 +586,20 @@ static int plan_shape(su_plan &pl, int sms, int smem_max, std::vector<unsigned c
             std::memcpy(blob.data() + P.fx.tail_off, tail.data(), tail.size() * sizeof(float));
         }
     }
-    if (general && prec == SU_FP64 && S >= 1 && !P.wf_on && !P.generic && pl.opt.seg_log2 == 0 && pl.opt.rounds == 0)
-        split_general(pl, blob, smem_max);
+    if (general && prec == SU_FP64 && S >= 1 && !P.wf_on && !P.generic && pl.opt.seg_log2 == 0) split_general(pl, blob, smem_max);
+    pl.kernel = P.fx.on ? kFixedPoint : P.gs.on ? kSplit : kWhole;
+    // the shape that su_autotune stored for plans of this kernel; where the fastest
+    // was another kernel's, that kernel
+    Tuned tuned{};
+    const bool have_tuned = pl.tuned && tuned_shape({prec, pl.model, pl.p, S, pl.kernel}, tuned);
+    if (have_tuned && pl.opt.seg_log2 == 0 && (tuned.kernel != pl.kernel || tuned.shape.seg_log2 != P.F)) {
+        P.fx.on = P.gs.on = 0;
+        blob.resize(tables_end);
+        pl.kernel = kWhole;
+        P.F = std::min(S, std::max(1, tuned.shape.seg_log2));
+        rc = stage_tables();
+        if (rc) return rc;
+    }
     // launch shape: one path per thread, persistent grid over items of
     // 128 * rounds samples
     const int occ1 = plan_rounds(pl, 1, sms, smem_max);
@@ -583,10 +612,12 @@ static int plan_shape(su_plan &pl, int sms, int smem_max, std::vector<unsigned c
     int rounds = 1;
     while (rounds < 8 && P.n_items * pl.levels * 32 > ((int64_t)512 << 20)) plan_rounds(pl, rounds *= 2, sms, smem_max);
     while (rounds > 1 && plan_rounds(pl, rounds, sms, smem_max) < occ1) rounds /= 2;
-    if (pl.opt.rounds > 0 || (have_tuned && tuned.rounds > 0)) {
-        rounds = pl.opt.rounds > 0 ? pl.opt.rounds : tuned.rounds;
+    if (pl.opt.rounds > 0) {
+        rounds = pl.opt.rounds;
         if (plan_rounds(pl, rounds, sms, smem_max) < 1)
             return fail(SU_ENOTSUP, "rounds = %d does not fit (shared memory %zu bytes)", rounds, pl.smem);
+    } else if (have_tuned && tuned.shape.rounds > 0 && plan_rounds(pl, tuned.shape.rounds, sms, smem_max) >= 1) {
+        rounds = tuned.shape.rounds;
     }
     plan_rounds(pl, rounds, sms, smem_max);
     pl.tuple_bytes = pl.n_blocks * pl.levels * 4 * (int64_t)sizeof(double);
@@ -667,7 +698,7 @@ static int plan_init(su_plan &pl, int model, const double *params, int n_params,
 // in_call: the plan's device block is ordered on the options' stream, and so
 // are all uses of it and its release (a plan inside one entry point).
 static int plan_create(int model, const double *params, int n_params, double a, double b, double T, int p, int s,
-                       int64_t n_mc, uint64_t seed, const su_options *opt, su_plan **out, bool in_call) {
+                       int64_t n_mc, uint64_t seed, const su_options *opt, su_plan **out, bool in_call, bool tuned = true) {
     if (!out) return fail(SU_EINVAL, "plan pointer missing");
     *out = nullptr;
     su_options o;
@@ -678,6 +709,7 @@ static int plan_create(int model, const double *params, int n_params, double a, 
     int rc = plan_init(*pl, model, params, n_params, a, b, T, p, s, n_mc, seed, o);
     if (rc) return rc;
     pl->tables_async = in_call;
+    pl->tuned = tuned;
     rc = configure(*pl);
     if (rc) {
         free_tables(*pl);
@@ -1541,16 +1573,21 @@ int su_autotune(int model, const double *params, int n_params, double a, double 
     CU(cudaEventCreate(&res.e[0]), "event");
     CU(cudaEventCreate(&res.e[1]), "event");
     std::vector<su_tuning> got;
-    for (int F = 1; F <= std::min(s, su::kMaxFine); ++F) {
+    std::vector<int> kernels;   // that each ran
+    int automatic = kWhole;     // kernel of the plans that take what is stored
+    // F = 0: the automatic segments, where they are another kernel's than the explicit ones'
+    for (int F = 0; F <= std::min(s, su::kMaxFine); ++F) {
         for (int r : {1, 2, 4, 8}) {
             su_options oc = o;
             oc.seg_log2 = F;
             oc.rounds = r;
             su_plan *pl = nullptr;
-            rc = su_plan_create(model, params, n_params, a, b, T, p, s, n_probe, seed, &oc, &pl);
+            rc = plan_create(model, params, n_params, a, b, T, p, s, n_probe, seed, &oc, &pl, false, false);
             if (rc == SU_ENOTSUP) continue;   // this shape's shared memory does not fit
             if (rc) return rc;
             std::unique_ptr<su_plan, int (*)(su_plan *)> guard(pl, su_plan_destroy);
+            if (F == 0 && r == 1) automatic = pl->kernel;
+            if (F == 0 && pl->kernel != kSplit) break;
             const size_t need = (size_t)(pl->tuple_bytes + pl->scratch_bytes);
             if (need > res.cap) {
                 if (res.buf) cudaFree(res.buf);
@@ -1574,14 +1611,17 @@ int su_autotune(int model, const double *params, int n_params, double a, double 
                 ms_best = std::min(ms_best, ms);
             }
             got.push_back({pl->P.F, pl->P.rounds, (double)ms_best});
+            kernels.push_back(pl->kernel);
         }
     }
     if (got.empty()) return fail(SU_ENOTSUP, "no launch shape fits this device");
-    const su_tuning top = *std::min_element(got.begin(), got.end(),
-                                            [](const su_tuning &x, const su_tuning &y) { return x.ms < y.ms; });
+    const size_t best_at = (size_t)(std::min_element(got.begin(), got.end(),
+                                                     [](const su_tuning &x, const su_tuning &y) { return x.ms < y.ms; }) -
+                                    got.begin());
+    const su_tuning top = got[best_at];
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune[{o.precision, model, p, s}] = top;
+        g_tune[{o.precision, model, p, s, automatic}] = {top, kernels[best_at]};
     }
     *best = top;
     for (int i = 0; i < (int)got.size() && i < cap; ++i) all[i] = got[(size_t)i];
