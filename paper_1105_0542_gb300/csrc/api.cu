@@ -2859,25 +2859,33 @@ extern "C" int speedup_amplitude_noalloc(int model, const double *params, int n_
     std::vector<unsigned char> blob;
     rc = plan_tables(pl, blob);
     if (rc) return rc;
+    const size_t tables = blob.size();
     int dev = 0, sms = 0, smem_max = 0;
     rc = device_limits(dev, sms, smem_max);
-    if (rc) return rc;
-    rc = plan_shape(pl, sms, smem_max, blob);
     if (rc) return rc;
 
     // scratch layout: tables | per-item tuples | per-block tuples | flag word;
     // where the per-item tuples do not fit, more paths per item (rounds up to
-    // 8, while the shape stays resident), unless the caller fixed rounds
-    const int64_t tab_bytes = up256((int64_t)blob.size());
-    const int64_t tup_bytes = up256(pl.tuple_bytes);
+    // 8, while the shape stays resident), unless the caller fixed rounds; where
+    // the fixed-point sampler's images are too much, the double sampler
+    int64_t tab_bytes = 0, tup_bytes = 0;
     auto fits = [&] { return tab_bytes + up256(pl.partial_bytes) + tup_bytes + 256 <= (int64_t)SU_NOALLOC_SCRATCH_BYTES; };
-    if (!fits() && o.rounds == 0) {
-        int good = pl.P.rounds;
-        for (int r = good * 2; r <= 8 && !fits(); r *= 2) {
-            if (plan_rounds(pl, r, sms, smem_max) < 1) break;   // shared memory or residency
-            good = r;
+    for (;;) {
+        blob.resize(tables);
+        rc = plan_shape(pl, sms, smem_max, blob);
+        if (rc) return rc;
+        tab_bytes = up256((int64_t)blob.size());
+        tup_bytes = up256(pl.tuple_bytes);
+        if (!fits() && o.rounds == 0) {
+            int good = pl.P.rounds;
+            for (int r = good * 2; r <= 8 && !fits(); r *= 2) {
+                if (plan_rounds(pl, r, sms, smem_max) < 1) break;   // shared memory or residency
+                good = r;
+            }
+            plan_rounds(pl, good, sms, smem_max);
         }
-        plan_rounds(pl, good, sms, smem_max);
+        if (fits() || !pl.P.fx.on) break;
+        pl.fixed_point = false;
     }
     if (!fits())
         return fail(SU_ENOTSUP,
