@@ -210,6 +210,7 @@ struct BandMma {
     unsigned long long *scratch_max;
     int *status;                       // bit 0: a wait ran out
 };
+int band_mma_bits();                          // of an element's digits, below the largest one's power of two
 int band_exponent(unsigned long long bits);   // e of |v| = m 2^e, m in [1/2, 1), from v's bits
 cudaError_t launch_diag_max(const double *D, int64_t pitch, int n, int w, unsigned long long *dmax, cudaStream_t st);
 int64_t band_mma_bytes_a(int n, int w);

@@ -42,9 +42,12 @@ namespace su {
 namespace {
 
 // least n w B for the tensor-core product: at n = 1201, w = 158, B = 8 a product
-// takes 0.023 ms there and 0.013 in double, at n = 2001, w = 212, B = 16 0.029
-// and 0.050, at n = 16 385, w = 1297, B = 16 0.090 and 1.16
+// takes 0.023 ms there and 0.013 in double, at n = 2001, w = 212, B = 16 0.032
+// and 0.050, at n = 16 385, w = 1297, B = 16 0.106 and 1.16
 constexpr int64_t kMmaLeast = 3000000;
+// and its least band: below some 36 diagonals the digits' rounding, of the largest
+// element, would pass that of the double product's running sums (spectrum_mma.cu)
+constexpr int kMmaBand = 48;
 
 // symmetric eigenpairs of the k x k matrix A (row-major) by cyclic Jacobi
 // rotations; eigenvalues descending in ev, eigenvectors in the columns of V
@@ -390,10 +393,10 @@ int band_spectrum(const double *D, int64_t pitch, int n, int w, int nev, int deg
         const unsigned long long top = *std::max_element(dm.begin(), dm.end());
         W.M.n = n;
         W.M.ea = band_exponent(top);
-        // diagonals whose elements all round to zero digits (below 2^-48 of the largest's power of two)
+        // diagonals whose elements all round to zero digits
         W.M.w = w;
-        while (W.M.w > 0 && band_exponent(dm[(size_t)W.M.w]) < W.M.ea - 48) --W.M.w;
-        if (W.M.ea > -400 && W.M.ea < 400 && (int64_t)n * w * B >= kMmaLeast) {
+        while (W.M.w > 0 && band_exponent(dm[(size_t)W.M.w]) < W.M.ea - band_mma_bits() - 1) --W.M.w;
+        if (W.M.ea > -400 && W.M.ea < 400 && W.M.w >= kMmaBand && (int64_t)n * w * B >= kMmaLeast) {
             W.mx[0] = dmax + w + 1;
             W.mx[1] = W.mx[0] + 32;
             W.M.scratch_max = W.mx[1] + 32;

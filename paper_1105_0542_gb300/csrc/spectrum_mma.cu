@@ -5,26 +5,29 @@
 // 64-bit integers (the scheme of Ozaki, Ogita, Oishi and Rump, "Error-free
 // transformations of matrix multiplication by using fast routines", 2012).
 //
-// With U = 2^(ea - 47) sum_i d_i 2^(8 (5 - i)), i = 0..5, |d_i| <= 128 (ea: the
+// With U = 2^(ea - 55) sum_i d_i 2^(8 (6 - i)), i = 0..6, |d_i| <= 128 (ea: the
 // exponent of max |U|), and column c of X likewise (its own exponent), the sums
-//   D_g = sum_k sum_{i + j = g} d_i[k] x_j[k],  g = 0..5
-// over K = 128 columns of U stay below 6 * 128 * 2^14 < 2^24: exact.  Dropped: the
-// digits' rounding, 2^-49 of the largest element, and the pairs i + j >= 6, 2^-48.
-// Against the double product's own rounding (2^-53 of a running sum some 300
-// times the largest element) both are small.
+//   D_g = sum_k sum_{i + j = g} d_i[k] x_j[k],  g = 0..6
+// over K = 128 columns of U stay below 7 * 128 * 2^14 < 2^24: exact.  Dropped: the
+// digits' rounding, 2^-57 of the largest element, and the pairs i + j >= 7, 2^-55.
+// Against the product in double, whose rounding is that of its running sums, the
+// root mean square error on bands of 36 diagonals and more is between 0.01 (smooth
+// columns) and 0.9 (random ones) times as large; narrower bands stay in double
+// (band_spectrum).  With six digits it was 1.4 to 240 times as large.
 //
-// Layout: U as row tiles of 128 rows, each over its band in chunks of 64 columns;
-// a chunk is six digit planes of 128 x 64 bfloat16 in the operand layout of
-// mlp.cuh (core matrices of 8 rows x 16 bytes, no swizzle), 96 KB contiguous, so
+// Layout: U as row tiles of 128 rows, each over its band in chunks of 32 columns;
+// a chunk is seven digit planes of 128 x 32 bfloat16 in the operand layout of
+// mlp.cuh (core matrices of 8 rows x 16 bytes, no swizzle), 56 KB contiguous, so
 // that one bulk copy brings it to shared memory.  X's digits lie in chunks of
-// 64 rows of U's columns: rows j * 16 + c (digit j of column c), 12 KB.
-// Per 16 columns of U and digit i one MMA of M = 128, N = 16 (6 - i): A = plane
-// i, B = digits 0..5-i of the 16 columns, D at tensor-memory column 16 i, so that
+// 32 rows of U's columns: rows j * 16 + c (digit j of column c), 7 KB.
+// Per 16 columns of U and digit i one MMA of M = 128, N = 16 (7 - i): A = plane
+// i, B = digits 0..6-i of the 16 columns, D at tensor-memory column 16 i, so that
 // pairs of equal i + j share an accumulator.
 //
-// What bounds it: reading the digit planes, 12 bytes an element once per
-// product (0.48 GB at n = 16 385, w = 1297, in 81 us: 6 TB/s); the product in
-// double took 1161 us at 96 % of the FP64 pipe.
+// What bounds it: reading the digit planes, 14 bytes an element once per
+// product (617 MB at n = 16 385, w = 1297, in 98 us: 6.3 TB/s of a copy's 6.8; tensor
+// cores 21 % busy; 0.106 ms with the digits of X, 0.090 with six digits); the
+// product in double took 1161 us at 96 % of the FP64 pipe.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -37,13 +40,15 @@
 namespace su {
 namespace {
 
-constexpr int kDig = 6;                        // digits of 8 bits
+constexpr int kDig = 7;                        // digits of 8 bits
+constexpr int kBits = 8 * kDig - 1;            // of an element, of its largest one's power of two
 constexpr int kCols = 16;                      // columns of X per pass
-constexpr int kChunk = 64;                     // columns of U per stage
+constexpr int kChunk = 32;                     // columns of U per stage
+constexpr int kWindow = 128 / kChunk;          // stages whose sums share an accumulator buffer
 constexpr int kPlane = 128 * kChunk * 2;       // bytes of one digit plane of a chunk
-constexpr int kABytes = kDig * kPlane;         // 96 KB
-constexpr int kBBytes = kDig * kCols * kChunk * 2;   // 12 KB
-constexpr int kStages = 2;
+constexpr int kABytes = kDig * kPlane;         // 56 KB
+constexpr int kBBytes = kDig * kCols * kChunk * 2;   // 7 KB
+constexpr int kStages = 3;
 constexpr int kMmaThreads = 320;               // eight epilogue warps, one that issues, one that copies
 constexpr int kMmaSmem = kStages * (kABytes + kBBytes) + 128;
 
@@ -52,7 +57,7 @@ __device__ __forceinline__ int exponent_of(unsigned long long bits) {   // v = m
 }
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// the six digits of q (|q| <= 2^47), most significant first
+// the digits of q (|q| <= 2^kBits), most significant first
 __device__ __forceinline__ void digits(long long q, int (&d)[kDig]) {
 #pragma unroll
     for (int i = kDig - 1; i > 0; --i) {
@@ -87,7 +92,7 @@ __device__ __forceinline__ int tile_col0(int rt, int w) { return max(0, rt * 128
 __global__ void __launch_bounds__(256) digits_a_kernel(const double *__restrict__ D, int64_t pitch, int n, int w,
                                                        int nk, int ea, unsigned char *__restrict__ A) {
     const int rt = blockIdx.y, kc = blockIdx.x;
-    const double scale = pow2(47 - ea);
+    const double scale = pow2(kBits - ea);
     unsigned char *out = A + ((int64_t)rt * nk + kc) * kABytes;
     for (int g = threadIdx.x; g < 128 * (kChunk / 8); g += 256) {
         const int lr = g & 127, kg = g >> 7, r = rt * 128 + lr;
@@ -134,7 +139,7 @@ __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict_
     const int c = t & 15, g = t >> 4;
     if (g >= rows8) return;
     const unsigned long long m = xmax[c];
-    const double scale = m ? pow2(47 - exponent_of(m)) : 0.0;
+    const double scale = m ? pow2(kBits - exponent_of(m)) : 0.0;
     int d[8][kDig];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -142,7 +147,7 @@ __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict_
         const double v = (r < n && col0 + c < B) ? X[(int64_t)r * B + col0 + c] : 0.0;
         digits(__double2ll_rn(v * scale), d[j]);
     }
-    unsigned char *out = Xd + (int64_t)(g / 8) * kBBytes;
+    unsigned char *out = Xd + (int64_t)(g / (kChunk / 8)) * kBBytes;
 #pragma unroll
     for (int i = 0; i < kDig; ++i) {
         uint4 q;
@@ -150,7 +155,7 @@ __global__ void __launch_bounds__(256) digits_x_kernel(const double *__restrict_
         q.y = pair_bf16(d[2][i], d[3][i]);
         q.z = pair_bf16(d[4][i], d[5][i]);
         q.w = pair_bf16(d[6][i], d[7][i]);
-        *reinterpret_cast<uint4 *>(out + mlp::cm_off(i * kCols + c, (g & 7) * 8, kChunk)) = q;
+        *reinterpret_cast<uint4 *>(out + mlp::cm_off(i * kCols + c, g % (kChunk / 8) * 8, kChunk)) = q;
     }
 }
 
@@ -191,7 +196,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t addr, int (&v)[8]) {
 }
 
 // Ynew = alpha U X + beta Ycur + gamma Yprev for 16 columns of X, one row tile per
-// CTA.  Warp 9 copies chunks (two stages), warp 8 issues their MMAs into one of two
+// CTA.  Warp 9 copies chunks (three stages), warp 8 issues their MMAs into one of two
 // accumulator buffers per 128 columns of U, warps 0..7 read a finished buffer (two
 // warps per lane quadrant, eight columns each) into 64-bit sums while the other
 // fills.
@@ -217,7 +222,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(const MmaArgs 
     const uint32_t base = (mlp::smem_u32(sm) + 127u) & ~127u;
     const int c0 = tile_col0(rt, P.w);
     const int cend = min(P.n, rt * 128 + 128 + P.w);
-    const int nk = (cend - c0 + kChunk - 1) / kChunk, nw = (nk + 1) / 2;
+    const int nk = (cend - c0 + kChunk - 1) / kChunk, nw = (nk + kWindow - 1) / kWindow;
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             bar_init(full + 8 * s, 1);
@@ -269,8 +274,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(const MmaArgs 
     } else if (warp == 8) {
         if (lane == 0) {
             for (int k = 0; k < nk && ok; ++k) {
-                const int s = k % kStages, win = k >> 1, buf = win & 1;
-                if ((k & 1) == 0 && win >= 2 && !bar_wait(wfree + 8 * buf, (uint32_t)(win / 2 - 1) & 1u)) {
+                const int s = k % kStages, win = k / kWindow, buf = win & 1;
+                if (k % kWindow == 0 && win >= 2 && !bar_wait(wfree + 8 * buf, (uint32_t)(win / 2 - 1) & 1u)) {
                     ok = false;
                     break;
                 }
@@ -288,10 +293,10 @@ __global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(const MmaArgs 
                         asm volatile(
                             "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + buf * 128 + i * kCols),
-                            "l"(ad), "l"(bd), "r"(id), "r"((uint32_t)((k & 1) || ks || i)));
+                            "l"(ad), "l"(bd), "r"(id), "r"((uint32_t)(k % kWindow || ks || i)));
                     }
                 bar_commit(empty + 8 * s);
-                if ((k & 1) || k == nk - 1) bar_commit(wfull + 8 * buf);
+                if (k % kWindow == kWindow - 1 || k == nk - 1) bar_commit(wfull + 8 * buf);
             }
         }
         __syncwarp();
@@ -310,11 +315,10 @@ __global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(const MmaArgs 
                 tmem_ld8(at + buf * 128 + g * kCols, v);
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    const long long x = (long long)v[c] << (8 * (2 - g % 3));
-                    if (g < 3)
-                        hi[c] += x;
+                    if (g < 4)
+                        hi[c] += (long long)v[c] << (8 * (3 - g));
                     else
-                        lo[c] += x;
+                        lo[c] += (long long)v[c] << (8 * (6 - g));
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
@@ -326,15 +330,14 @@ __global__ void __launch_bounds__(kMmaThreads, 1) band_mma_kernel(const MmaArgs 
     __syncthreads();
     if (warp < 8 && !dead) {
         const int r = rt * 128 + 32 * (warp & 3) + lane;
-        const int ea = P.ea - 47;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const int cc = 8 * (warp >> 2) + c, col = P.col0 + cc;
             double y = 0.0;
             const unsigned long long xm = P.xmax[cc];
             if (r < P.n && col < P.B) {
-                // 2^40 (hi 2^24 + lo) in units of both scales
-                y = xm ? fma((double)hi[c], 0x1p24, (double)lo[c]) * pow2(ea + 20) * pow2(exponent_of(xm) - 27) : 0.0;
+                // 2^48 (hi 2^24 + lo) in units of both scales
+                y = xm ? fma((double)hi[c], 0x1p24, (double)lo[c]) * pow2(P.ea - 31) * pow2(exponent_of(xm) - 31) : 0.0;
                 const int64_t at = (int64_t)r * P.B + col;
                 y *= P.alpha;
                 if (P.beta != 0.0) y = fma(P.beta, P.Ycur[at], y);
@@ -415,6 +418,7 @@ int64_t band_mma_bytes_a(int n, int w) { return band_mma_tiles(n) * band_mma_chu
 // (the last tile's last chunk may start up to a chunk past n)
 int64_t band_mma_bytes_x(int n) { return ((int64_t)n / kChunk + 2) * kBBytes; }
 
+int band_mma_bits() { return kBits; }
 int band_exponent(unsigned long long bits) { return (int)((bits >> 52) & 0x7FF) - 1022; }
 
 cudaError_t launch_diag_max(const double *D, int64_t pitch, int n, int w, unsigned long long *dmax, cudaStream_t st) {
