@@ -42,11 +42,46 @@ P_LIST = workloads.CONFIG2_P
 # per SM per clock x 2 flop x 2.07 GHz (nominal GB300 FP64 rate 1.25 TFLOP/s;
 # no FP64 tensor path)
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# DRAM bytes (read + write) of one double-sampler launch of the p = 10 sweep
+# DRAM bytes (read + write) of one launch of sampler_fx_kernel, the p = 10 sweep
 # point on 2e5 samples (an ncu capture of `--profile fp64`); scaled by
 # samples per launch
-FP64_TRAFFIC_BYTES, FP64_TRAFFIC_SAMPLES = 250_368, 200_000
+FP64_TRAFFIC_BYTES, FP64_TRAFFIC_SAMPLES = 470_784, 200_000
 CPU_BUDGET_S = 15.0
+
+
+def finite(x):
+    """The same with null for numbers that JSON does not have."""
+    if isinstance(x, float):
+        return x if math.isfinite(x) else None
+    if isinstance(x, dict):
+        return {k: finite(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [finite(v) for v in x]
+    return x
+
+
+# what of an entry stands on the result line (everything of those not listed); the
+# whole record, some 80 KB, goes to stderr: a log that keeps the end of stdout
+# keeps the line
+SHORT = {
+    "chosen_fp32": ("value", "unit", "ms_per_step", "dtype"),
+    "time_to_rel_1e-4_s": ("p", "plain_fp64", "chosen_fp32"),
+    "roofline": ("bound", "achieved", "peak", "unit", "frac", "kernel"),
+    "cpu_baseline": ("value", "unit", "cores", "kind"),
+}
+ON_LINE = ("impl", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+           "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "chosen_fp32", "time_to_rel_1e-4_s",
+           "roofline", "cpu_baseline")
+
+
+def result_line(record):
+    """The one JSON line of a run's record."""
+    line = {}
+    for k in ON_LINE:
+        if k in record:
+            v = record[k]
+            line[k] = {f: v[f] for f in SHORT[k] if f in v} if k in SHORT and isinstance(v, dict) else v
+    return json.dumps(finite(line), allow_nan=False)
 
 
 def parse():
@@ -221,7 +256,7 @@ def run_reference(args):
                                    "per step on the host cores)"},
             "cpu_baseline": {"value": v, "unit": UNIT, "cores": used, "kind": "oracle", "sample": desc},
             "e2e": {"value": v, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(line))
+    print(json.dumps(finite(line), allow_nan=False))
 
 
 def oracle_precision_table(su, torch, ps, n_sub=1000):
@@ -476,7 +511,8 @@ def run_ours(args):
         "fig2_convergence_fit": fig2,
         "clocks": plain["clocks"],
     }
-    print(json.dumps(line))
+    print(json.dumps(finite(line), allow_nan=False), file=sys.stderr, flush=True)
+    print(result_line(line), flush=True)
     if dist is not None:
         dist.destroy_process_group()
 
