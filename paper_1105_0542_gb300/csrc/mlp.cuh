@@ -72,16 +72,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// erf(v/sqrt 2) from the polynomial of erf_poly.h (one value)
-__device__ __forceinline__ float erf_sqrt2(float v) {
-    const float x = fminf(fmaxf(v, -kErfClamp), kErfClamp);
-    const float z = x * x;
-    float p = erf_poly(kErfTerms - 1);
-#pragma unroll
-    for (int k = kErfTerms - 2; k >= 0; --k) p = fmaf(p, z, erf_poly(k));
-    return x * p;
-}
-
 // GELU of two values, v (1/2 + erf(v/sqrt 2)/2), with erf(v/sqrt 2) from the
 // odd polynomial v Q(v^2) of erf_poly.h (v clamped to [-3 sqrt 2, 3 sqrt 2],
 // error <= 1e-4, below the bfloat16 rounding the epilogue applies; the halves

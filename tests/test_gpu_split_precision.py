@@ -94,6 +94,18 @@ def test_general_split_is_no_further_off_than_the_whole_program(V, p, s):
     assert rms["auto"] <= 1.5 * rms["generic"]
 
 
+@pytest.mark.parametrize("V,p,s,n", [(QUARTIC, 12, 1, 777), (QUARTIC, 4, 10, 130), (NARROW, 8, 9, 300), (MORSE, 10, 4, 1001)],
+                         ids=["two-slices", "p4", "narrow", "exponentials"])
+def test_general_split_matches_the_whole_program(V, p, s, n):
+    """Two slices, the smallest program that splits, a feature narrower than
+    the bridge, exponentials; a partial last item.  A few 2^-50 of a weight
+    (the guard's 2^-30 in single precision, 2^-24 of it a few times over, and
+    the sums of up to 1024 slices)."""
+    w = {k: _general(V, -0.4, 0.6, 0.2, p, s, n, kernel=k) for k in ("auto", "generic")}
+    assert np.any(w["auto"][:, -1] != w["generic"][:, -1])
+    assert np.all(np.abs(w["auto"] - w["generic"]) <= 2.0 ** -48 * np.maximum(1.0, np.abs(w["generic"])))
+
+
 # samples of seed 1234 whose first normal is -6.17, -6.43: q_{N/2} some 3 sqrt(T) from the endpoints
 FAR = [492790794, 2573160571]
 
