@@ -461,13 +461,14 @@ int band_spectrum(const double *D, int64_t pitch, int n, int w, int nev, int deg
         double cut = theta[(size_t)B - 1];
         cut = std::max(cut, lo + 1e-3 * (theta[0] - lo));
         const double c0 = 0.5 * (cut + lo), e0 = 0.5 * (cut - lo);
-        // A degree at which the largest pair is amplified by no more than 2^43 against
-        // the smallest of the block: beyond that the rounding left of it in the others'
-        // vectors outgrows them, and the block loses rank.  (T_m(x) < e^(m acosh x); it
+        // A degree at which the largest pair is amplified by no more than 2^64 against
+        // the smallest of the block: the rounding left of it in the others' vectors,
+        // 2^-53, then outgrows them by no more than 2^11, which the orthonormalization
+        // takes; much further on the block loses rank.  (T_m(x) < e^(m acosh x); it
         // matters where the block reaches down to the spectrum's flat end, short
         // intervals or long times.)
         const double x = (theta[0] - c0) / e0;
-        const int reach = x > 1.0 ? (int)(43 * 0.69314718055994531 / std::acosh(x)) : degree;
+        const int reach = x > 1.0 ? (int)(64 * 0.69314718055994531 / std::acosh(x)) : degree;
         const int m = std::max(2, std::min(it == 0 ? std::min(4, degree) : degree, reach));
         double *ym1 = X, *y = Y0, *yp = Y1;
         if ((e = maxima(W, X)) || (e = product(W, X, X, nullptr, Y0, 1.0 / e0, -c0 / e0, 0.0, 0))) return cuda_err(e, "filter");

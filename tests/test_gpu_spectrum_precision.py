@@ -19,7 +19,7 @@ def test_residuals_are_a_double_products(g, t, L, n, nev):
 
 
 @pytest.mark.parametrize("n,L,t,nev", [(1100, 2.0, 0.05, 10), (1025, 2.0, 0.05, 8), (1025, 2.0, 0.05, 10), (900, 1.5, 0.05, 10),
-                                       (1201, 2.0, 0.1, 2), (257, 2.0, 0.05, 10)])
+                                       (1201, 2.0, 0.1, 2), (257, 2.0, 0.05, 10), (3001, 2.0, 0.05, 20)])
 def test_blocks_that_reach_the_flat_end_of_the_spectrum_keep_their_rank(n, L, t, nev):
     """In a short interval the block's last eigenvalues are far below the
     first: energies against numpy's eigensolver on the dense matrix (its own
