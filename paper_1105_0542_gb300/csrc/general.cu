@@ -192,97 +192,115 @@ __global__ void __launch_bounds__(kThreads, 4) general_kernel(const __grid_const
         const int64_t hi = (b + 1) * P.n_mc / P.n_blocks;
         const int64_t start = lo + r * chunk;
         const int cnt = (int)max((int64_t)0, min((int64_t)chunk, hi - start));
-        for (int t = tid; t < cnt; t += kThreads) {
-            const uint64_t sample = (uint64_t)(P.sample0 + start + t);
-            st.slo = (uint32_t)sample;
-            st.shi = (uint32_t)(sample >> 32);
-            double w[SU_MAX_S];
-            uint32_t todo = (1u << L) - 1u;   // levels of this pass
-            for (int pass = 0; pass < 2 && todo; ++pass) {
-                uint32_t have = 0xffffffffu;
-                double z0 = 0, z1 = 0;
-                auto normal = [&](uint32_t g) {
-                    if ((g >> 1) != have) {
-                        st.pair(g >> 1, z0, z1);
-                        have = g >> 1;
-                    }
-                    return (g & 1u) ? z1 : z0;
-                };
-                float tsum[SU_MAX_S], tmag[SU_MAX_S];
-                for (int d = 0; d < L; ++d) {
-                    if (todo >> d & 1u) w[d] = 0;
-                    tsum[d] = tmag[d] = 0;
-                }
-                auto slices = [&](int d, const double *q, int stp, int ns) {
-                    if (!(todo >> d & 1u)) return;
-                    const bool split = pass == 0 && P.gs.hn[d] > 0;
-                    if (split) {
-                        const float *c = tail + (size_t)d * P.M;
-                        float s = 0, m = 0;
-                        if (ns >= 8) {
-#pragma unroll 1
-                            for (int k = 0; k < ns; k += 8) gen_single<4>(G, nodes, c, q, k, stp, s, m);
-                        } else {
-#pragma unroll 1
-                            for (int k = 0; k < ns; k += 2) gen_single<1>(G, nodes, c, q, k, stp, s, m);
+        for (int t0 = 0; t0 < cnt; t0 += kThreads) {
+            // Pass 0: every lane its sample.  Then, one sample at a time by the whole warp, a
+            // pair of slices a lane, the levels beyond the split's reach by the whole program,
+            // summed in its order.  (By the sample's own lane that held a call of 30 001
+            // samples up by a tenth: p = 12, N = 64, T = 1.)
+            uint32_t todo = (1u << L) - 1u, far = 0;
+            for (unsigned left = 1, pass = 0; left; ++pass) {
+                const int t = t0 + (pass ? (tid & ~31) + __ffs(left) - 1 : tid);
+                double w[SU_MAX_S];
+                if (pass || t < cnt) {
+                    const uint64_t sample = (uint64_t)(P.sample0 + start + t);
+                    st.slo = (uint32_t)sample;
+                    st.shi = (uint32_t)(sample >> 32);
+                    uint32_t have = 0xffffffffu;
+                    double z0 = 0, z1 = 0;
+                    auto normal = [&](uint32_t g) {
+                        if ((g >> 1) != have) {
+                            st.pair(g >> 1, z0, z1);
+                            have = g >> 1;
                         }
-                        tsum[d] += s;
-                        tmag[d] += m;
+                        return (g & 1u) ? z1 : z0;
+                    };
+                    float tsum[SU_MAX_S], tmag[SU_MAX_S];
+                    for (int d = 0; d < L; ++d) {
+                        w[d] = 0;
+                        tsum[d] = tmag[d] = 0;
                     }
-                    const GeneralNode *nd = split ? hnodes + P.gs.h0[d] : nodes;
-                    const int nn = split ? P.gs.hn[d] : G->n_nodes, J = split ? P.gs.hj[d] : G->J;
-                    const double *c = split ? hcoef + P.gs.hc[d] : reinterpret_cast<const double *>(P.tables) + (size_t)d * P.M;
-                    double sum = 0;   // of this segment (one running sum over the path rounds at its full size)
+                    auto slices = [&](int d, const double *q, int stp, int ns) {
+                        if (!(todo >> d & 1u)) return;
+                        const bool split = pass == 0 && P.gs.hn[d] > 0;
+                        if (split) {
+                            const float *c = tail + (size_t)d * P.M;
+                            float s = 0, m = 0;
+                            if (ns >= 8) {
 #pragma unroll 1
-                    for (int k = 0; k < ns; k += 2) {
-                        const double2 v = slice_general<2>(q[k * stp], q[(k + 1) * stp], q[(k + 1) * stp], q[(k + 2) * stp],
-                                                           c, G, nd, nn, J);
-                        sum += v.x + v.y;
-                    }
-                    w[d] += sum;
-                };
-                // coarse levels: the segment endpoints
-                co[0] = P.a;
-                co[C] = P.b;
-                for (int n = 1; n <= Cn; ++n) {
-                    const int h = 1 << (Cn - n);
-                    for (int i = 0; i < (1 << (n - 1)); ++i) {
-                        const int x = (2 * i + 1) * h;
-                        co[x] = fma(P.sigma[n], normal((1u << (n - 1)) - 1u + (uint32_t)i), 0.5 * (co[x - h] + co[x + h]));
-                    }
-                }
+                                for (int k = 0; k < ns; k += 8) gen_single<4>(G, nodes, c, q, k, stp, s, m);
+                            } else {
 #pragma unroll 1
-                for (int d = F; d < L; ++d) slices(d, co, 1 << (d - F), 1 << (S - d));
+                                for (int k = 0; k < ns; k += 2) gen_single<1>(G, nodes, c, q, k, stp, s, m);
+                            }
+                            tsum[d] += s;
+                            tmag[d] += m;
+                        }
+                        const GeneralNode *nd = split ? hnodes + P.gs.h0[d] : nodes;
+                        const int nn = split ? P.gs.hn[d] : G->n_nodes, J = split ? P.gs.hj[d] : G->J;
+                        const double *c = split ? hcoef + P.gs.hc[d] : reinterpret_cast<const double *>(P.tables) + (size_t)d * P.M;
+                        double sum = 0;   // of this segment (one running sum over the path rounds at its full size)
 #pragma unroll 1
-                for (int sg = 0; sg < C; ++sg) {
-                    seg[0] = co[sg];
-                    seg[NF] = co[sg + 1];
-                    for (int n = Cn + 1; n <= S; ++n) {
-                        const int h = 1 << (S - n), m = 1 << (n - Cn - 1);
-                        for (int i = 0; i < m; ++i) {
+                        for (int k = pass ? 2 * lane : 0; k < ns; k += pass ? 64 : 2) {
+                            const double2 v = slice_general<2>(q[k * stp], q[(k + 1) * stp], q[(k + 1) * stp], q[(k + 2) * stp],
+                                                               c, G, nd, nn, J);
+                            sum += v.x + v.y;
+                        }
+                        if (pass) {   // at most 32 pairs, in order
+                            const double mine = sum;
+                            sum = 0;
+                            __syncwarp();
+                            for (int k = 0; k < ns / 2; ++k) sum += __shfl_sync(0xffffffffu, mine, k);
+                        }
+                        w[d] += sum;
+                    };
+                    // coarse levels: the segment endpoints
+                    co[0] = P.a;
+                    co[C] = P.b;
+                    for (int n = 1; n <= Cn; ++n) {
+                        const int h = 1 << (Cn - n);
+                        for (int i = 0; i < (1 << (n - 1)); ++i) {
                             const int x = (2 * i + 1) * h;
-                            seg[x] = fma(P.sigma[n], normal((1u << (n - 1)) - 1u + (uint32_t)(sg * m + i)), 0.5 * (seg[x - h] + seg[x + h]));
+                            co[x] = fma(P.sigma[n], normal((1u << (n - 1)) - 1u + (uint32_t)i), 0.5 * (co[x - h] + co[x + h]));
                         }
                     }
 #pragma unroll 1
-                    for (int d = 0; d < min(F, L); ++d) slices(d, seg, 1 << d, NF >> d);
-                }
-                uint32_t far = 0;
-                for (int d = 0; d < L; ++d)
-                    if (pass == 0 && P.gs.hn[d] > 0) {
-                        w[d] += (double)tsum[d];
-                        if (!(tmag[d] <= kGenTail * fmaxf(1.0f, fabsf(__double2float_rn(w[d]))))) far |= 1u << d;
+                    for (int d = F; d < L; ++d) slices(d, co, 1 << (d - F), 1 << (S - d));
+#pragma unroll 1
+                    for (int sg = 0; sg < C; ++sg) {
+                        seg[0] = co[sg];
+                        seg[NF] = co[sg + 1];
+                        for (int n = Cn + 1; n <= S; ++n) {
+                            const int h = 1 << (S - n), m = 1 << (n - Cn - 1);
+                            for (int i = 0; i < m; ++i) {
+                                const int x = (2 * i + 1) * h;
+                                seg[x] = fma(P.sigma[n], normal((1u << (n - 1)) - 1u + (uint32_t)(sg * m + i)), 0.5 * (seg[x - h] + seg[x + h]));
+                            }
+                        }
+#pragma unroll 1
+                        for (int d = 0; d < min(F, L); ++d) slices(d, seg, 1 << d, NF >> d);
                     }
-                todo = far;
-            }
-            bool bad = false;
-            for (int d = 0; d < L; ++d) bad |= isnan(w[d]) || (isinf(w[d]) && w[d] > 0);
-            if (bad) atomicOr(P.flags, 1);
-            if (per_sample) {
-                double *dst = P.w_out + (start + t) * (int64_t)S;
-                for (int d = 0; d < L; ++d) dst[S - d - 1] = w[d];
-            } else {
-                for (int d = 0; d < L; ++d) sw[(size_t)d * chunk + t] = w[d];
+                    if (pass == 0)
+                        for (int d = 0; d < L; ++d)
+                            if (P.gs.hn[d] > 0) {
+                                w[d] += (double)tsum[d];
+                                if (!(tmag[d] <= kGenTail * fmaxf(1.0f, fabsf(__double2float_rn(w[d]))))) far |= 1u << d;
+                            }
+                    if (pass == 0 || lane == 0) {
+                        bool bad = false;
+                        for (int d = 0; d < L; ++d)
+                            if (pass ? todo >> d & 1u : !(far >> d & 1u)) {
+                                bad |= isnan(w[d]) || (isinf(w[d]) && w[d] > 0);
+                                if (per_sample)
+                                    P.w_out[(start + t) * (int64_t)S + (S - d - 1)] = w[d];
+                                else
+                                    sw[(size_t)d * chunk + t] = w[d];
+                            }
+                        if (bad) atomicOr(P.flags, 1);
+                    }
+                }
+                __syncwarp();
+                left = pass ? left & (left - 1) : __ballot_sync(0xffffffffu, far != 0);
+                if (left) todo = __shfl_sync(0xffffffffu, far, __ffs(left) - 1);
             }
         }
         if (per_sample) continue;
